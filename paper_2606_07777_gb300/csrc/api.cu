@@ -121,8 +121,8 @@ struct Runner {
   int topk = 4;  // one-family sweeps: values tracked per row in the first pass
   bool short_rows = false;   // iteration sweeps take the short-row sweep (sweep_short.cu)
   int upd_ctas = 1;      // update grid width (the largest member's)
-  bool upd_test = false; // some member has the adaptive restart (a test kernel runs first)
   InstDesc *inst_iter = nullptr, *inst_stats = nullptr;
+  InstDesc h_iter0{};  // host copy of inst_iter[0]
   double* cuts = nullptr;  // per-instance DLM_BOX_CUT budgets (box-cut runners only)
   UpdInst* upd = nullptr;
   StatsInst* st_stats = nullptr;
@@ -189,9 +189,8 @@ struct dlm_problem {
   unsigned long long* objq = nullptr;       // fixed-point objective sum of the iteration sweep
   int sO = 0;                               // its exponent
   double* traj = nullptr;                   // [kTrajCap] g(y_t) per iteration (ring)
-  double* upd_part = nullptr;               // update partials [2 update_ctas(m J + 1) + 1]
-  unsigned* upd_ticket = nullptr;           // [2]
-  int32_t* upd_flag = nullptr;
+  double* upd_part = nullptr;               // update partials [update_parts(m J + 1)]
+  unsigned* upd_ticket = nullptr;
   int64_t traj_from = 0;                    // first iteration whose trajectory entry is valid
   double *gamma_tab = nullptr, *calc_gamma = nullptr, *stats_out = nullptr;
   int64_t nstages = 1, gamma_tab_cap = 0;
@@ -453,7 +452,6 @@ dlm_status write_tables(Runner& R) {
     u.traj = p->traj;
     u.part = p->upd_part;
     u.ticket = p->upd_ticket;
-    u.flag = p->upd_flag;
     u.nct = update_ctas(p->D());
     u.iters_per_stage = p->ips;
     u.curv_max = p->curv_max;
@@ -476,15 +474,12 @@ dlm_status write_tables(Runner& R) {
     st[i].grad_out = nullptr;
     st[i].state = p->state;
   }
+  R.h_iter0 = it[0];
   CK(cudaMemcpy(R.inst_iter, it.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.inst_stats, ss.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.upd, up.data(), sizeof(UpdInst) * n, cudaMemcpyHostToDevice));
   R.upd_ctas = 1;
-  R.upd_test = false;
-  for (const UpdInst& u : up) {
-    R.upd_ctas = std::max(R.upd_ctas, u.nct);
-    R.upd_test = R.upd_test || u.adaptive_restart;
-  }
+  for (const UpdInst& u : up) R.upd_ctas = std::max(R.upd_ctas, u.nct);
   CK(cudaMemcpy(R.st_stats, st.data(), sizeof(StatsInst) * n, cudaMemcpyHostToDevice));
   return DLM_OK;
 }
@@ -573,6 +568,7 @@ SweepLaunch launch_of(const Runner& R, const InstDesc* tab) {
   L.nunits = static_cast<int32_t>(R.h_units.size());
   L.ctr = R.ctr;
   L.topk = R.topk;
+  L.inst0 = R.probs.size() == 1 ? &R.h_iter0 : nullptr;
   if (R.short_rows && short_capable(R) && !L.count) {
     L.short_rows = true;
     L.nslices0 = R.probs[0]->lay.nslices;
@@ -595,7 +591,7 @@ cudaError_t dispatch_sweep(const Runner& R, const SweepLaunch& L, bool stats, bo
 
 dlm_status enqueue_iteration(Runner& R) {
   CK(dispatch_sweep(R, launch_of(R, R.inst_iter), false, R.bf16));
-  CK(launch_update(R.upd, static_cast<int>(R.probs.size()), R.upd_ctas, R.upd_test, R.stream));
+  CK(launch_update(R.upd, static_cast<int>(R.probs.size()), R.upd_ctas, R.stream));
   return DLM_OK;
 }
 
@@ -652,7 +648,7 @@ dlm_status runner_step_timed(Runner& R, int64_t n_iters, double* sweep_ms, doubl
   for (int64_t i = 0; i < n_iters; ++i) {
     CK(dispatch_sweep(R, L, false, R.bf16));
     CK(cudaEventRecord(R.events[2 * i + 1], R.stream));
-    CK(launch_update(R.upd, n, R.upd_ctas, R.upd_test, R.stream));
+    CK(launch_update(R.upd, n, R.upd_ctas, R.stream));
     CK(cudaEventRecord(R.events[2 * i + 2], R.stream));
   }
   CK(cudaStreamSynchronize(R.stream));
@@ -739,7 +735,7 @@ void free_problem(dlm_problem* p) {
   }
   void* ptrs[] = {p->b,         p->curv,      p->lam,      p->y,      p->gamma_tab, p->calc_gamma, p->stats_out,
                   p->state,     p->inst_calc, p->st_calc,  p->lam64,  p->y64,       p->traj,       p->upd_part,
-                  p->upd_ticket, p->upd_flag};
+                  p->upd_ticket};
   for (void* q : ptrs) cudaFree(q);
   cudaFreeHost(p->h_out);
   cudaFreeHost(p->h_inst);
@@ -1321,11 +1317,9 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
   CKC(dalloc(&p->lam64, MJ + 1));
   CKC(dalloc(&p->y64, MJ + 1));
   CKC(dalloc(&p->traj, kTrajCap));
-  CKC(dalloc(&p->upd_part, 2 * static_cast<size_t>(update_ctas(MJ + 1)) + 1));
-  CKC(dalloc(&p->upd_ticket, 2));
-  CKC(dalloc(&p->upd_flag, 1));
-  CKC(cudaMemsetAsync(p->upd_ticket, 0, sizeof(unsigned) * 2, p->stream));
-  CKC(cudaMemsetAsync(p->upd_flag, 0, sizeof(int32_t), p->stream));
+  CKC(dalloc(&p->upd_part, static_cast<size_t>(update_parts(MJ + 1))));
+  CKC(dalloc(&p->upd_ticket, 1));
+  CKC(cudaMemsetAsync(p->upd_ticket, 0, sizeof(unsigned), p->stream));
   CKC(cudaMemsetAsync(p->lam64, 0, sizeof(double) * (MJ + 1), p->stream));
   CKC(cudaMemsetAsync(p->y64, 0, sizeof(double) * (MJ + 1), p->stream));
   CKC(cudaMemsetAsync(p->traj, 0, sizeof(double) * kTrajCap, p->stream));
@@ -1745,7 +1739,7 @@ dlm_status dlm_shard_sweep(dlm_problem* p) {
 dlm_status dlm_shard_update(dlm_problem* p) {
   dlm_status st = shard_handle(p);
   if (st != DLM_OK) return st;
-  CK(launch_update(p->run.upd, 1, p->run.upd_ctas, p->run.upd_test, p->stream));
+  CK(launch_update(p->run.upd, 1, p->run.upd_ctas, p->stream));
   return DLM_OK;
 }
 

@@ -49,9 +49,8 @@ struct UpdInst {
   unsigned long long* acc;  // [J] fixed-point A x at y
   unsigned long long* objq; // fixed-point sum of (c x + gamma/2 x^2) at y (reset here)
   double* traj;             // [kTrajCap] g(y_t) at slot t mod kTrajCap
-  double* part;             // [2 nct + 1] per-CTA partials of the update's sums
-  unsigned* ticket;         // [2] CTAs of the instance done (reset by the last)
-  int32_t* flag;            // the adaptive restart decision of the iteration
+  double* part;             // [update_parts(D)] per-CTA partials of the update's sums
+  unsigned* ticket;         // CTAs of the instance done (reset by the last)
   int32_t nct;              // update CTAs of the instance (update_ctas(D))
   int64_t iters_per_stage;
   double curv_max;          // the largest curvature bound (plain step gamma / curv_max)
@@ -136,6 +135,19 @@ __device__ __forceinline__ int lead_caller_pos(uint64_t lead, int k, int d) {
   return c;
 }
 
+// f rounded to a 64-bit integer (ties to even), |f| < 2^55: the bits of
+// __float2ll_rn without the FP64 pipe it runs on (two lanes per clock and SM).
+// The part above 2^32 is read off the significand of a sum rounded
+// down at 2^23; what is left is exact and converts to 32 bits.
+__device__ __forceinline__ unsigned long long fix64(float f) {
+  const float af = fabsf(f);
+  const float m = __fadd_rd(af * 2.3283064365386963e-10f, 8388608.f);  // 2^23 + floor(|f| / 2^32)
+  const uint32_t lo = __float2uint_rn(fmaf(8388608.f - m, 4294967296.f, af));
+  const uint32_t hi = __float_as_uint(m) - 0x4B000000u;
+  const unsigned long long v = (static_cast<unsigned long long>(hi) << 32) | lo;
+  return f < 0.f ? 0ull - v : v;
+}
+
 // A task: slices first, first + stride, ... (< end) of instance `inst`.  The
 // tasks of one CTA are contiguous and grouped by instance.
 struct Task {
@@ -162,6 +174,8 @@ struct SweepLaunch {
   bool count;               // some instance has a global count constraint (its own instantiation)
   int32_t fam;              // capacity families (> 1: the general sweep of sweep_multi.cu)
   int32_t topk = 4;         // one-family sweep: largest values tracked per row in the first pass (4 or 8)
+  // iteration sweeps of one instance: host copy of its descriptor (a kernel parameter)
+  const InstDesc* inst0 = nullptr;
   // Short-row sweep (iteration sweeps of a single one-family handle without a
   // count constraint, sweep_short.cu): slices 0 .. nslices0 - 1 of instance 0.
   bool short_rows = false;
@@ -214,10 +228,10 @@ cudaError_t launch_sweep(const SweepLaunch& L, bool stats, bool bf16);
 cudaError_t sweep_short_prepare(bool bf16);
 cudaError_t launch_sweep_short(const SweepLaunch& L, bool bf16);
 // The update of ninst instances: a grid of max_cta x ninst CTAs (instance i
-// uses its first update_ctas(D_i)); any_test: some instance has the adaptive
-// restart on (a first kernel takes the test).
-cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, bool any_test, cudaStream_t s);
+// uses its first update_ctas(D_i)).
+cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, cudaStream_t s);
 int update_ctas(int64_t D);
+int update_parts(int64_t D);  // doubles of UpdInst::part for D coordinates
 cudaError_t launch_stats(const StatsInst* dev_tab, int ninst, cudaStream_t s);
 // The certificate sweep's objective partials of instance 0 summed into *out.
 cudaError_t launch_seg_sum(const StatsInst* dev_tab, double* out, cudaStream_t s);

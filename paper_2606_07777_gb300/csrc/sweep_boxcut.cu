@@ -347,9 +347,10 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
 // Per CTA its tasks; certificate sweeps deal a task's slices to warps in a
 // static order (first + stride (warp + k nw)), iteration sweeps from a
 // per-CTA ticket counter.
-template <class V, bool STATS>
+// ONE: one instance, its descriptor a kernel parameter (as in sweep.cu).
+template <class V, bool STATS, bool ONE>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-    sweep_boxcut_kernel(const InstDesc* __restrict__ insts, const Task* __restrict__ tasks,
+    sweep_boxcut_kernel(const __grid_constant__ InstDesc one, const InstDesc* __restrict__ insts, const Task* __restrict__ tasks,
                         const int32_t* __restrict__ cta_task, int smemJ, int jlo, int jw,
                         const double* __restrict__ cuts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -360,7 +361,9 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   float* ys = reinterpret_cast<float*>(accG + (STATS ? 3 : 1) * static_cast<size_t>(accN));
   double* wsum = reinterpret_cast<double*>(ys + ((smemJ + 1) & ~1));
 
-  __shared__ InstDesc sD;
+  __shared__ InstDesc s_inst;
+  const InstDesc& sD = ONE ? one : s_inst;
+  __shared__ BSeg sS;
   __shared__ unsigned long long s_next;
   __shared__ unsigned long long s_red[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -371,8 +374,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     const int inst = tasks[t].inst;
     int te = t + 1;
     while (te < t_last && tasks[te].inst == inst) ++te;
-    if (threadIdx.x == 0) sD = insts[inst];
-    __syncthreads();
+    if (!ONE) {
+      if (threadIdx.x == 0) s_inst = insts[inst];
+      __syncthreads();
+    }
     const int J = sD.J;
     const int nacc = STATS ? max(0, min(J - jlo, jw)) : J;
     for (int j = threadIdx.x; j < J; j += blockDim.x) ys[j] = sD.y[j];
@@ -383,8 +388,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
         accQ[j] = 0ull;
       }
     }
-    BSeg S;
-    {
+    if (threadIdx.x == 0) {  // FP64 work once per CTA (as fill_seg)
+      BSeg& S = sS;
       const double g = *sD.gamma;
       S.gamma = static_cast<float>(g);
       S.invg = static_cast<float>(1.0 / g);
@@ -406,6 +411,12 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     }
     if (threadIdx.x == 0) s_next = 0;
     __syncthreads();
+    BSeg S = sS;
+    if (ONE) {
+      S.z = sD.z;
+      S.scaleG = sD.scaleG;
+      S.scaleO = sD.scaleO;
+    }
     double wobj = 0.0;
     unsigned long long oq = 0ull;
     for (int k = t; k < te; ++k) {
@@ -464,10 +475,12 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
 
 template <class V>
 cudaError_t prepare_values(int lim) {
-  cudaError_t e = cudaFuncSetAttribute(&sweep_boxcut_kernel<V, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       lim);
+  cudaError_t e = cudaFuncSetAttribute(&sweep_boxcut_kernel<V, false, true>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(&sweep_boxcut_kernel<V, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  e = cudaFuncSetAttribute(&sweep_boxcut_kernel<V, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(&sweep_boxcut_kernel<V, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
 template <class V>
@@ -478,14 +491,20 @@ cudaError_t launch_values(const SweepLaunch& L, bool stats, const double* cuts) 
     if (w < 1) return cudaErrorInvalidValue;
     const size_t sm = sweep_stats_smem_bytes(L.smemJ, w);
     for (int jlo = 0; jlo < L.smemJ || jlo == 0; jlo += w) {
-      sweep_boxcut_kernel<V, true><<<L.grid, th, sm, L.stream>>>(L.inst, L.tasks, L.cta_task, L.smemJ, jlo, w, cuts);
+      sweep_boxcut_kernel<V, true, false>
+          <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, jlo, w, cuts);
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
   }
-  sweep_boxcut_kernel<V, false><<<L.grid, th, sweep_smem_bytes(L.smemJ, false), L.stream>>>(
-      L.inst, L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
+  const size_t sm = sweep_smem_bytes(L.smemJ, false);
+  if (L.inst0 != nullptr)
+    sweep_boxcut_kernel<V, false, true>
+        <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
+  else
+    sweep_boxcut_kernel<V, false, false>
+        <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
   return cudaGetLastError();
 }
 

@@ -332,9 +332,10 @@ __device__ __forceinline__ void multi_slice(const InstDesc& D, const MSeg& S, co
 
 // Shared memory: accG [m smemJ], then (STATS) accC, accQ [smemJ each], then
 // ys [m smemJ] floats, then 32 doubles of warp partials.
-template <class P, bool STATS, int M>
+// ONE: one instance, its descriptor a kernel parameter (as in sweep.cu).
+template <class P, bool STATS, int M, bool ONE>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-    sweep_multi_kernel(const InstDesc* __restrict__ insts, const Task* __restrict__ tasks,
+    sweep_multi_kernel(const __grid_constant__ InstDesc one, const InstDesc* __restrict__ insts, const Task* __restrict__ tasks,
                        const int32_t* __restrict__ cta_task, int smemJ, int m, bool bf16) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* accG = reinterpret_cast<unsigned long long*>(smem_raw);
@@ -343,7 +344,9 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   float* ys = reinterpret_cast<float*>(accG + static_cast<size_t>(m + (STATS ? 2 : 0)) * smemJ);
   double* wsum = reinterpret_cast<double*>(ys + ((static_cast<size_t>(m) * smemJ + 1) & ~static_cast<size_t>(1)));
 
-  __shared__ InstDesc sD;
+  __shared__ InstDesc s_inst;
+  const InstDesc& sD = ONE ? one : s_inst;
+  __shared__ MSeg sS;
   __shared__ unsigned long long s_next;
   __shared__ unsigned long long s_red[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -354,8 +357,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     const int inst = tasks[t].inst;
     int te = t + 1;
     while (te < t_last && tasks[te].inst == inst) ++te;
-    if (threadIdx.x == 0) sD = insts[inst];
-    __syncthreads();
+    if (!ONE) {
+      if (threadIdx.x == 0) s_inst = insts[inst];
+      __syncthreads();
+    }
     const int J = sD.J;
     const int mJ = sD.m * J;
     for (int q = threadIdx.x; q < mJ; q += blockDim.x) {
@@ -364,8 +369,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     }
     if (STATS)
       for (int j = threadIdx.x; j < J; j += blockDim.x) accC[j] = accQ[j] = 0ull;
-    MSeg S;
-    {
+    if (threadIdx.x == 0) {  // FP64 work once per CTA (as fill_seg)
+      MSeg& S = sS;
       const double g = *sD.gamma;
       S.gamma = static_cast<float>(g);
       S.invg = static_cast<float>(1.0 / g);
@@ -382,6 +387,15 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
       S.J = J;
     }
     __syncthreads();
+    MSeg S = sS;
+    if (ONE) {
+      S.z = sD.z;
+      S.scaleG = sD.scaleG;
+      S.scaleO = sD.scaleO;
+      S.kind = sD.kind;
+      S.m = sD.m;
+      S.J = sD.J;
+    }
     double wobj = 0.0;
     unsigned long long oq = 0ull;
     for (int k = t; k < te; ++k) {
@@ -447,9 +461,12 @@ namespace {
 template <class P, int M>
 cudaError_t prepare_m(int lim) {
   cudaError_t e =
-      cudaFuncSetAttribute(&sweep_multi_kernel<P, false, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+      cudaFuncSetAttribute(&sweep_multi_kernel<P, false, M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(&sweep_multi_kernel<P, true, M>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  e = cudaFuncSetAttribute(&sweep_multi_kernel<P, false, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(&sweep_multi_kernel<P, true, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              lim);
 }
 
 template <class P, int M>
@@ -457,9 +474,14 @@ cudaError_t launch_m(const SweepLaunch& L, bool stats, bool bf16) {
   const size_t sm = sweep_multi_smem_bytes(L.smemJ, L.fam, stats);
   const int th = L.threads > 0 ? L.threads : kSweepThreads;
   if (stats)
-    sweep_multi_kernel<P, true, M><<<L.grid, th, sm, L.stream>>>(L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
+    sweep_multi_kernel<P, true, M, false>
+        <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
+  else if (L.inst0 != nullptr)
+    sweep_multi_kernel<P, false, M, true>
+        <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
   else
-    sweep_multi_kernel<P, false, M><<<L.grid, th, sm, L.stream>>>(L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
+    sweep_multi_kernel<P, false, M, false>
+        <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
   return cudaGetLastError();
 }
 

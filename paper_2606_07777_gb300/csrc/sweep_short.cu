@@ -341,74 +341,67 @@ __device__ __forceinline__ void wide_slice(const InstDesc& D, const Seg& S, cons
 
 // Every slice of instance 0, dealt to the warps in turn (every warp gets the
 // same mix of widths); item sums in shared memory, flushed once per CTA.
+// The instance's descriptor is a kernel parameter (one instance per launch):
+// its fields are constant-bank operands and take no registers.
 template <class P>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-    sweep_short_kernel(const InstDesc* __restrict__ insts, int64_t nslices) {
+    sweep_short_kernel(const __grid_constant__ InstDesc D, int64_t nslices) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ InstDesc sD;
+  __shared__ Seg sS;
   __shared__ unsigned long long s_red[32];
-  if (threadIdx.x == 0) sD = insts[0];
-  __syncthreads();
-  const int J = sD.J;
+  const int J = D.J;
   unsigned long long* accG = reinterpret_cast<unsigned long long*>(smem_raw);
   float* ys = reinterpret_cast<float*>(accG + J);
   for (int j = threadIdx.x; j < J; j += blockDim.x) {
-    ys[j] = sD.y[j];
+    ys[j] = D.y[j];
     accG[j] = 0ull;
   }
-  Seg S{};
-  {
-    const double g = *sD.gamma;
-    S.gamma = static_cast<float>(g);
-    S.invg = static_cast<float>(1.0 / g);
-    const double gz = g * static_cast<double>(sD.z);
-    S.gz = static_cast<float>(gz);
-    S.gzl = static_cast<float>(gz - static_cast<double>(S.gz));
-    S.z = sD.z;
-    S.scaleG = sD.scaleG;
-    S.scaleO = sD.scaleO;
-    S.kind = sD.kind;
-  }
+  if (threadIdx.x == 0) fill_seg(D, 0, J, sS);
   __syncthreads();
+  Seg S = sS;
+  S.z = D.z;
+  S.scaleG = D.scaleG;
+  S.scaleO = D.scaleO;
+  S.kind = D.kind;
   unsigned long long oq = 0ull;
   const int nw = blockDim.x >> 5;
   const int64_t step = static_cast<int64_t>(gridDim.x) * nw;
   for (int64_t s = static_cast<int64_t>(blockIdx.x) * nw + (threadIdx.x >> 5); s < nslices; s += step) {
-    const int64_t off = __ldg(sD.slice_off + s);
-    const int w = __ldg(sD.slice_w + s);
+    const int64_t off = __ldg(D.slice_off + s);
+    const int w = __ldg(D.slice_w + s);
     // width classes (warp-uniform branch)
     if (w > kShortRowW)
-      wide_slice<P>(sD, S, ys, accG, off, w, oq);
+      wide_slice<P>(D, S, ys, accG, off, w, oq);
     else if (w > 24)
-      short_slice<P, 32>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 32>(D, S, ys, accG, off, w, oq);
     else if (w > 16)
-      short_slice<P, 24>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 24>(D, S, ys, accG, off, w, oq);
     else if (w > 12)
-      short_slice<P, 16>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 16>(D, S, ys, accG, off, w, oq);
     else if (w > 10)
-      short_slice<P, 12>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 12>(D, S, ys, accG, off, w, oq);
     else if (w > 8)
-      short_slice<P, 10>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 10>(D, S, ys, accG, off, w, oq);
     else if (w > 6)
-      short_slice<P, 8>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 8>(D, S, ys, accG, off, w, oq);
     else if (w > 4)
-      short_slice<P, 6>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 6>(D, S, ys, accG, off, w, oq);
     else
-      short_slice<P, 4>(sD, S, ys, accG, off, w, oq);
+      short_slice<P, 4>(D, S, ys, accG, off, w, oq);
   }
   __syncthreads();
   for (int j = threadIdx.x; j < J; j += blockDim.x) {
     const unsigned long long v = accG[j];
-    if (v) atomicAdd(sD.acc + j, v);
+    if (v) atomicAdd(D.acc + j, v);
   }
-  cta_add_u64(oq, s_red, sD.objq);
+  cta_add_u64(oq, s_red, D.objq);
 }
 
 template <class V>
 cudaError_t launch_short_values(const SweepLaunch& L) {
   const int th = L.threads > 0 ? L.threads : kSweepThreads;
   const size_t sm = sweep_smem_bytes(L.smemJ, false);
-  sweep_short_kernel<Narrow<V>><<<L.grid, th, sm, L.stream>>>(L.inst, L.nslices0);
+  sweep_short_kernel<Narrow<V>><<<L.grid, th, sm, L.stream>>>(*L.inst0, L.nslices0);
   return cudaGetLastError();
 }
 
