@@ -307,7 +307,7 @@ __global__ void __launch_bounds__(128) k_gemm(GemmArgs g) {
 // ---------------------------------------------------------------------------
 
 __device__ __forceinline__ float softplus_f(float z) { return fmaxf(z, 0.f) + log1pf(expf(-fabsf(z))); }
-__device__ __forceinline__ float sigmoid_f(float z) { return 0.5f * (1.f + tanhf(0.5f * z)); }
+__device__ __forceinline__ float sigmoid_f(float z) { return 1.f / (1.f + expf(-z)); }  // accurate in both tails
 __device__ __forceinline__ float softplus_inv_f(float y) { return y + logf(-expm1f(-y)); }
 
 __global__ void k_norm_apply(const float* __restrict__ X, int64_t n, const float* __restrict__ mu,
@@ -471,25 +471,535 @@ __global__ void k_normalizer(const float* __restrict__ X, int64_t n, float* __re
   }
 }
 
-// Adam (bias-corrected) on the FP32 master weights, then their bf16 copies.
+// One bias-corrected Adam step of a parameter; returns its new value.
+__device__ __forceinline__ float adam_step(float th, float gi, float* m, float* v, float lr, float c1, float c2) {
+  constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
+  const float mi = b1 * *m + (1.f - b1) * gi;
+  const float vi = b2 * *v + (1.f - b2) * gi * gi;
+  *m = mi;
+  *v = vi;
+  return th - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+
+// Adam on the FP32 master weights (widths above kMaxFused).
 __global__ void k_adam(float* __restrict__ th, const float* __restrict__ g, float* __restrict__ m,
                        float* __restrict__ v, int64_t P, float lr, float c1, float c2) {
-  constexpr float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < P;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    th[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-  }
+       i += static_cast<int64_t>(gridDim.x) * blockDim.x)
+    th[i] = adam_step(th[i], g[i], m + i, v + i, lr, c1, c2);
 }
 
 __global__ void k_to_bf16(const float* __restrict__ src, int64_t n, bf16* __restrict__ dst) {
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < n;
        i += static_cast<int64_t>(gridDim.x) * blockDim.x)
     dst[i] = __float2bfloat16_rn(src[i]);
+}
+
+// ---------------------------------------------------------------------------
+// The network fused (widths up to 256): one CTA of 256 threads takes a tile
+// of 128 rows through the forward pass and, with BWD, the whole backward pass,
+// every intermediate in shared memory and TMEM.
+//
+// What bounds it: the products are small (17,000 rows x 128: 1.8 GFLOP, 1 us
+// of the tensor cores) and each depends on the one before it, so the time is
+// the chain of a tile -- load, five products, three epilogues -- and not any
+// throughput; the tiles are spread one per SM.  As separate launches (five
+// products through global memory with scalar staging, six elementwise kernels,
+// six reductions) loss and gradient took MLP_BEFORE us at 17,000 x 128; fused
+// MLP_NOW us.
+//
+// Shared-memory operands are unswizzled 8 x 16-byte core matrices in columns
+// of 16-byte pieces: element (r, k) of a row buffer at
+// (k / 8) kCS + 16 r + 2 (k % 8), kCS = 128 rows * 16 + 16 (the 16 bytes of
+// padding put the pieces of one row in different banks).  The same buffer
+// serves as a K-major operand (rows as M or N, k as K: row groups of eight
+// 128 bytes apart, K pieces kCS apart) and, for the weight gradients, as an
+// MN-major one (k as M or N in pieces kCS apart, rows as K in groups of eight
+// 128 bytes apart), so nothing is transposed or copied.
+//
+// The products' K order, the layer-3 sum's order and every rounding to BF16
+// are those of the separate kernels, so the forward pass gives the same bits.  The
+// column sums (biases, w3) add FP32 terms as float pairs (TwoSum), the tiles'
+// results in FP64.  Partial gradients go to one slot per CTA and are added in
+// slot order by k_mlp_reduce: results do not depend on timing.
+// ---------------------------------------------------------------------------
+
+constexpr int kMlpThreads = 256;
+constexpr int kMlpRows = 128;
+constexpr int kMaxFused = 256;                 // widest network of the fused kernel
+constexpr uint32_t kCS = kMlpRows * 16 + 16;   // bytes between 8-wide column pieces of a row buffer
+constexpr uint32_t kW1S = 16 * 16 + 16;        // the same for W1 (16 rows: the features, zero filled)
+constexpr uint32_t kXS = 17;                   // floats between rows of the exchange buffer
+
+constexpr int mlp_smem(int HB) {
+  return static_cast<int>(2 * kCS + (HB / 8) * kW1S + 3 * (HB / 8) * kCS + 3 * HB * 4 + kMlpRows * 4 +
+                          kMlpRows * kXS * 4);
+}
+
+struct MlpArgs {
+  const float* X;       // [n x F]
+  const float* y;       // [n] (BWD)
+  int64_t n;
+  int H;
+  int64_t ntiles;
+  const float *mu, *sd, *b1, *b2, *b3;
+  const bf16 *W1, *W2, *w3;
+  float* out;           // [n] or nullptr
+  float* part;          // [slots][F H + H H] partial dW1, dW2 (BWD)
+  double* dpart;        // [slots][3 H + 2] partial db1, db2, dw3, db3, loss (BWD)
+  int* err;
+};
+
+__device__ __forceinline__ void pair_add(float& h, float& l, float v) {
+  const float s = h + v;
+  const float b = s - h;
+  l += (h - (s - b)) + (v - b);
+  h = s;
+}
+
+// Sixteen accumulator columns of the thread's TMEM lane.
+__device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
+  uint32_t r[16];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(addr));
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+  for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  const __nv_bfloat162 p = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const uint32_t*>(&p);
+}
+
+// One product: ksteps steps of K = 16 from the operands' descriptors, which
+// advance by astep, bstep bytes a step.  One thread.
+__device__ __forceinline__ void mma_run(uint32_t d, uint64_t ad, uint32_t astep, uint64_t bd, uint32_t bstep,
+                                        uint32_t idesc, int ksteps, bool acc0) {
+  for (int k = 0; k < ksteps; ++k) {
+    const uint32_t acc = (acc0 || k > 0) ? 1u : 0u;
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+        "l"(ad + static_cast<uint64_t>((astep * k) >> 4)), "l"(bd + static_cast<uint64_t>((bstep * k) >> 4)),
+        "r"(idesc), "r"(acc));
+  }
+}
+__device__ __forceinline__ void mma_commit(uint32_t bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
+// HB: the width rounded up to 128 or 256 (columns past the width are zero).
+template <int HB, bool BWD>
+__global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
+  constexpr int NC = HB / 8;                      // column pieces
+  constexpr int NB = HB / 128;                    // 128-column blocks of W2
+  constexpr uint32_t kW2S = HB * 16 + 16;         // piece stride of a W2 block held with HB rows
+  constexpr uint32_t kColZ2 = HB, kCols = 2 * HB; // TMEM columns: z1 (dH1, dW2's second block), z2 (dW2's first)
+  constexpr uint32_t kBase = (1u << 4) | (1u << 7) | (1u << 10) | (8u << 24);  // F32 += BF16 x BF16, M = 128
+  constexpr uint32_t kTA = 1u << 15, kTB = 1u << 16;                           // A, B MN-major
+  auto nbits = [](uint32_t n) { return (n >> 3) << 17; };
+  extern __shared__ __align__(128) unsigned char gsm[];
+  __shared__ __align__(8) uint64_t mbar;
+  __shared__ uint32_t tslot;
+  __shared__ double sred[2][kMlpThreads / 32];
+  unsigned char* sX = gsm;
+  unsigned char* sW1 = sX + 2 * kCS;
+  unsigned char* sH = sW1 + NC * kW1S;   // h1
+  unsigned char* sD = sH + NC * kCS;     // h2, then dz2
+  unsigned char* sW = sD + NC * kCS;     // W2 (a block of it), then dz1
+  float* sb1 = reinterpret_cast<float*>(sW + NC * kCS);
+  float* sb2 = sb1 + HB;
+  float* sw3 = sb2 + HB;
+  float* sdz = sw3 + HB;
+  float* sxc = sdz + kMlpRows;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int quad = warp & 3, half = warp >> 2;
+  const int row = 32 * quad + lane;
+  const int H = g.H;
+  const uint32_t bar = smem_addr(&mbar);
+
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(&tslot)),
+                 "r"(kCols));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(1));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  // weights and biases, zero past the width
+  const uint4 zero4 = make_uint4(0, 0, 0, 0);
+  for (int i = tid; i < NC * 16; i += kMlpThreads) {
+    const int f = i / NC, q = i % NC;
+    const bool on = f < kF && 8 * q < H;
+    *reinterpret_cast<uint4*>(sW1 + q * kW1S + f * 16) =
+        on ? __ldg(reinterpret_cast<const uint4*>(g.W1 + static_cast<int64_t>(f) * H + 8 * q)) : zero4;
+  }
+  for (int i = tid; i < HB; i += kMlpThreads) {
+    sb1[i] = i < H ? g.b1[i] : 0.f;
+    sb2[i] = i < H ? g.b2[i] : 0.f;
+    sw3[i] = i < H ? __bfloat162float(g.w3[i]) : 0.f;
+  }
+  // rows r0 .. r0 + nr - 1 of W2, pieces q0 .. q0 + nq - 1, at piece stride st
+  auto load_w2 = [&](int r0, int nr, int q0, int nq, uint32_t st) {
+    for (int i = tid; i < nr * nq; i += kMlpThreads) {
+      const int r = i / nq, q = i % nq;
+      const bool on = r0 + r < H && 8 * (q0 + q) < H;
+      *reinterpret_cast<uint4*>(sW + q * st + r * 16) =
+          on ? __ldg(reinterpret_cast<const uint4*>(g.W2 + static_cast<int64_t>(r0 + r) * H + 8 * (q0 + q))) : zero4;
+    }
+  };
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;");
+  const uint32_t tm = tslot;
+  const uint32_t tl = tm + (static_cast<uint32_t>(32 * quad) << 16);  // this warp's TMEM lanes
+  uint32_t phase = 0;
+  bool ok = true;
+  // shared-memory writes and TMEM reads of every thread ordered before the products issued next
+  auto hand_over = [&]() {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+  };
+  // waits for the products committed last (the outcome is made uniform across the CTA)
+  auto finished = [&]() {
+    ok = __syncthreads_and(mbar_wait(bar, phase)) != 0;
+    phase ^= 1u;
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    return ok;
+  };
+  const uint32_t aX = smem_addr(sX), aW1 = smem_addr(sW1), aH = smem_addr(sH), aD = smem_addr(sD), aW = smem_addr(sW);
+  float* part = BWD ? g.part + static_cast<int64_t>(blockIdx.x) * (static_cast<int64_t>(kF) * H + static_cast<int64_t>(H) * H)
+                    : nullptr;
+  // column sums of this thread's column (two threads per column at HB = 128, 64 rows each), as float pairs
+  const int col = tid & (HB - 1);
+  const int rlo = HB == 128 ? 64 * (tid >> 7) : 0, rn = HB == 128 ? 64 : 128;
+  float w3h = 0.f, w3l = 0.f, b2h = 0.f, b2l = 0.f, b1h = 0.f, b1l = 0.f, b3h = 0.f, b3l = 0.f;
+  double loss = 0.0;
+  const float two_n = BWD ? static_cast<float>(2.0 / static_cast<double>(g.n)) : 0.f;
+  const float bias3 = g.b3[0];
+
+  for (int64_t tile = blockIdx.x; tile < g.ntiles; tile += gridDim.x) {
+    const bool first = tile == blockIdx.x;
+    const int64_t r0 = tile * kMlpRows;
+    // normalized features (columns kF .. 15 zero)
+    {
+      const int64_t r = r0 + row;
+      float x[8];
+#pragma unroll
+      for (int f = 0; f < 8; ++f) x[f] = 0.f;
+      if (half == 0) {
+        if (r < g.n) {
+#pragma unroll
+          for (int f = 0; f < kF; ++f) x[f] = (__ldg(g.X + r * kF + f) - __ldg(g.mu + f)) / __ldg(g.sd + f);
+        }
+      }
+      *reinterpret_cast<uint4*>(sX + half * kCS + row * 16) =
+          make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
+    }
+    load_w2(0, HB, 0, 16, kW2S);
+    hand_over();
+    // z1 = Xn W1
+    if (tid == 0) {
+      mma_run(tm, smem_desc(aX, kCS, 128), 0, smem_desc(aW1, 128, kW1S), 0, kBase | kTB | nbits(HB), 1, false);
+      mma_commit(bar);
+    }
+    if (!finished()) break;
+    // h1 = bf16(relu(z1 + b1))
+#pragma unroll 2
+    for (int c = 16 * half; c < HB; c += 32) {
+      float v[16];
+      tmem_ld16(tl + c, v);
+#pragma unroll
+      for (int q = 0; q < 16; ++q) v[q] = fmaxf(v[q] + sb1[c + q], 0.f);
+#pragma unroll
+      for (int p = 0; p < 2; ++p)
+        *reinterpret_cast<uint4*>(sH + ((c >> 3) + p) * kCS + row * 16) =
+            make_uint4(pack_bf16(v[8 * p], v[8 * p + 1]), pack_bf16(v[8 * p + 2], v[8 * p + 3]),
+                       pack_bf16(v[8 * p + 4], v[8 * p + 5]), pack_bf16(v[8 * p + 6], v[8 * p + 7]));
+    }
+    // z2 = H1 W2, in blocks of 128 columns
+    for (int nb = 0; nb < NB; ++nb) {
+      if (nb > 0) load_w2(0, HB, 16 * nb, 16, kW2S);
+      hand_over();
+      if (tid == 0) {
+        mma_run(tm + kColZ2 + 128 * nb, smem_desc(aH, kCS, 128), 2 * kCS, smem_desc(aW, 128, kW2S), 256,
+                kBase | kTB | nbits(128), HB / 16, false);
+        mma_commit(bar);
+      }
+      if (!finished()) break;
+    }
+    if (!ok) break;
+    // h2 = bf16(relu(z2 + b2)) and its product with w3: the thread sums the columns of its half of each 32, then the
+    // sums are added in the order of a warp's shuffle tree over the 32 columns
+    float acc[16];
+#pragma unroll
+    for (int q = 0; q < 16; ++q) acc[q] = 0.f;
+#pragma unroll 2
+    for (int c = 16 * half; c < HB; c += 32) {
+      float v[16];
+      tmem_ld16(tl + kColZ2 + c, v);
+      uint32_t pk[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        pk[q] = pack_bf16(fmaxf(v[2 * q] + sb2[c + 2 * q], 0.f), fmaxf(v[2 * q + 1] + sb2[c + 2 * q + 1], 0.f));
+        acc[2 * q] = fmaf(__uint_as_float(pk[q] << 16), sw3[c + 2 * q], acc[2 * q]);
+        acc[2 * q + 1] = fmaf(__uint_as_float(pk[q] & 0xffff0000u), sw3[c + 2 * q + 1], acc[2 * q + 1]);
+      }
+      if (BWD) {
+        *reinterpret_cast<uint4*>(sD + (c >> 3) * kCS + row * 16) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
+        *reinterpret_cast<uint4*>(sD + ((c >> 3) + 1) * kCS + row * 16) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
+      }
+    }
+    if (half == 1) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) sxc[row * kXS + q] = acc[q];
+    }
+    __syncthreads();
+    if (half == 0) {
+#pragma unroll
+      for (int q = 0; q < 16; ++q) acc[q] += sxc[row * kXS + q];
+#pragma unroll
+      for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < o; ++q) acc[q] += acc[q + o];
+      const int64_t r = r0 + row;
+      float dz = 0.f;
+      if (r < g.n) {
+        const float s = acc[0] + bias3 + softplus_inv_f(fmaxf(__ldg(g.X + r * kF + 4), kLamFloor));
+        const float o = softplus_f(s);
+        if (g.out) g.out[r] = o;
+        if (BWD) {
+          const float e = o - __ldg(g.y + r);
+          dz = two_n * e * sigmoid_f(s);
+          loss += static_cast<double>(e) * e;
+          pair_add(b3h, b3l, dz);
+        }
+      }
+      if (BWD) sdz[row] = dz;
+    }
+    if (!BWD) continue;
+    // W2 by rows for dH1 (HB = 128: the block already held serves)
+    if (NB > 1) load_w2(0, 128, 0, NC, kCS);
+    __syncthreads();
+    // dz2 = bf16(dz3 w3 [z2 > 0]) over h2 in place, by columns, with the column sums of dz2 and h2 dz3
+    {
+      unsigned char* p = sD + (col >> 3) * kCS + (col & 7) * 2 + rlo * 16;
+      const float w = sw3[col];
+#pragma unroll 4
+      for (int r = 0; r < rn; ++r) {
+        bf16* e = reinterpret_cast<bf16*>(p + r * 16);
+        const float h = __bfloat162float(*e), d = sdz[rlo + r];
+        const bf16 q = __float2bfloat16_rn(h > 0.f ? d * w : 0.f);
+        *e = q;
+        const float t = h * d;
+        pair_add(w3h, w3l, t);
+        w3l += fmaf(h, d, -t);
+        pair_add(b2h, b2l, __bfloat162float(q));
+      }
+    }
+    hand_over();
+    // dH1 = dZ2 W2^T and dW2 = H1^T dZ2 (its first 128 rows)
+    for (int nb = 0; nb < NB; ++nb) {
+      if (nb > 0) {
+        load_w2(128 * nb, 128, 0, NC, kCS);
+        hand_over();
+      }
+      if (tid == 0) {
+        mma_run(tm + 128 * nb, smem_desc(aD, kCS, 128), 2 * kCS, smem_desc(aW, kCS, 128), 2 * kCS,
+                kBase | nbits(128), HB / 16, false);
+        if (nb == NB - 1)
+          mma_run(tm + kColZ2, smem_desc(aH, 128, kCS), 256, smem_desc(aD, 128, kCS), 256,
+                  kBase | kTA | kTB | nbits(HB), kMlpRows / 16, false);
+        mma_commit(bar);
+      }
+      if (!finished()) break;
+    }
+    if (!ok) break;
+    // dz1 = bf16(dH1 [z1 > 0]) over W2's buffer
+#pragma unroll 2
+    for (int c = 16 * half; c < HB; c += 32) {
+      float v[16];
+      tmem_ld16(tl + c, v);
+#pragma unroll
+      for (int p = 0; p < 2; ++p) {
+        const uint4 h = *reinterpret_cast<const uint4*>(sH + ((c >> 3) + p) * kCS + row * 16);
+        const uint32_t hw[4] = {h.x, h.y, h.z, h.w};
+        uint32_t o[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)  // h1 >= 0: positive where its bits are not zero
+          o[q] = pack_bf16((hw[q] & 0xffffu) ? v[8 * p + 2 * q] : 0.f, (hw[q] >> 16) ? v[8 * p + 2 * q + 1] : 0.f);
+        *reinterpret_cast<uint4*>(sW + ((c >> 3) + p) * kCS + row * 16) = make_uint4(o[0], o[1], o[2], o[3]);
+      }
+    }
+    hand_over();
+    // the second 128 rows of dW2 (HB = 256), over dH1's columns
+    if (NB > 1 && tid == 0) {
+      mma_run(tm, smem_desc(aH + 16 * kCS, 128, kCS), 256, smem_desc(aD, 128, kCS), 256,
+              kBase | kTA | kTB | nbits(HB), kMlpRows / 16, false);
+      mma_commit(bar);
+    }
+    // rows mb of the accumulators at column c0 to this CTA's slot, added to earlier tiles'
+    auto store_dw2 = [&](uint32_t c0, int h) {
+      float* dst = part + static_cast<int64_t>(kF) * H + static_cast<int64_t>(h) * H;
+      for (int c = 16 * half; c < HB; c += 32) {
+        float v[16];
+        tmem_ld16(tl + c0 + c, v);
+        if (h < H) {
+#pragma unroll
+          for (int p = 0; p < 4; ++p) {
+            const int o = c + 4 * p;
+            if (o < H) {
+              float4 t = make_float4(v[4 * p], v[4 * p + 1], v[4 * p + 2], v[4 * p + 3]);
+              if (!first) {
+                const float4 b = *reinterpret_cast<const float4*>(dst + o);
+                t.x += b.x, t.y += b.y, t.z += b.z, t.w += b.w;
+              }
+              *reinterpret_cast<float4*>(dst + o) = t;
+            }
+          }
+        }
+      }
+    };
+    store_dw2(kColZ2, row);
+    {  // column sums of dz1
+      const unsigned char* p = sW + (col >> 3) * kCS + (col & 7) * 2 + rlo * 16;
+#pragma unroll 8
+      for (int r = 0; r < rn; ++r) pair_add(b1h, b1l, __bfloat162float(*reinterpret_cast<const bf16*>(p + r * 16)));
+    }
+    if (NB > 1 && !finished()) break;
+    if (NB > 1) store_dw2(0, 128 + row);
+    hand_over();
+    // dW1^T = dZ1^T Xn (16 columns, kF of them features)
+    if (tid == 0) {
+      for (int mb = 0; mb < NB; ++mb)
+        mma_run(tm + kColZ2 + 16 * mb, smem_desc(aW + 16 * mb * kCS, 128, kCS), 256, smem_desc(aX, 128, kCS), 256,
+                kBase | kTA | kTB | nbits(16), kMlpRows / 16, false);
+      mma_commit(bar);
+    }
+    if (!finished()) break;
+    for (int mb = half; mb < NB; mb += 2) {
+      float v[16];
+      tmem_ld16(tl + kColZ2 + 16 * mb, v);
+      const int h = 128 * mb + row;
+      if (h < H) {
+#pragma unroll
+        for (int f = 0; f < kF; ++f) {
+          float* dst = part + static_cast<int64_t>(f) * H + h;
+          *dst = first ? v[f] : *dst + v[f];
+        }
+      }
+    }
+    asm volatile("tcgen05.fence::before_thread_sync;");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;");
+  }
+  if (!ok && tid == 0) {
+    atomicOr(g.err, 1);
+    mbar_wait(bar, phase ^ 1u);  // a last bounded wait for the products in flight
+  }
+  if (BWD) {
+    // this CTA's column sums, db3 and loss in FP64 (slots of CTAs without a tile hold zeros)
+    double* dp = g.dpart + static_cast<int64_t>(blockIdx.x) * (3 * H + 2);
+    double* sc = reinterpret_cast<double*>(sxc);  // [HB = 128: 3][128]
+    const double s1 = static_cast<double>(b1h) + b1l, s2 = static_cast<double>(b2h) + b2l,
+                 s3 = static_cast<double>(w3h) + w3l;
+    __syncthreads();
+    if (HB == 128 && tid >= 128) {
+      sc[col] = s1;
+      sc[128 + col] = s2;
+      sc[256 + col] = s3;
+    }
+    double t3 = static_cast<double>(b3h) + b3l;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      t3 += __shfl_down_sync(0xffffffffu, t3, o);
+      loss += __shfl_down_sync(0xffffffffu, loss, o);
+    }
+    if (lane == 0) {
+      sred[0][warp] = t3;
+      sred[1][warp] = loss;
+    }
+    __syncthreads();
+    if (tid < HB && col < H) {
+      dp[col] = s1 + (HB == 128 ? sc[col] : 0.0);
+      dp[H + col] = s2 + (HB == 128 ? sc[128 + col] : 0.0);
+      dp[2 * H + col] = s3 + (HB == 128 ? sc[256 + col] : 0.0);
+    }
+    if (tid == 0) {
+      double a = 0.0, b = 0.0;
+      for (int w = 0; w < kMlpThreads / 32; ++w) {
+        a += sred[0][w];
+        b += sred[1][w];
+      }
+      dp[3 * H] = a;
+      dp[3 * H + 1] = b;
+    }
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tm), "r"(kCols));
+}
+
+// The slots' partials added in slot order (eight threads of a parameter take
+// every eighth slot, their sums in order): the gradient, the loss, and with
+// `adam` the parameter's update and its BF16 copy.  A CTA of 32 x 8 threads
+// takes 32 parameters, so a warp's loads are consecutive.
+struct AdamArgs {
+  bool on;
+  float *theta, *m, *v;
+  float lr, c1, c2;
+  bf16 *W1, *W2, *w3;
+};
+__global__ void __launch_bounds__(256) k_mlp_reduce(const float* __restrict__ part, const double* __restrict__ dpart,
+                                                    int slots, int H, int64_t n, float* __restrict__ grad,
+                                                    double* __restrict__ loss, const AdamArgs a) {
+  constexpr int kG = 8;
+  __shared__ double sh[kG][32];
+  const int64_t fh = static_cast<int64_t>(kF) * H, hh = static_cast<int64_t>(H) * H;
+  const int64_t P = fh + H + hh + 2 * H + 1;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * 32 + threadIdx.x;  // parameter; P: the loss
+  const int gq = threadIdx.y;
+  // where parameter i's partials are: theta is W1, b1, W2, b2, w3, b3
+  int64_t at = -1, dat = -1;
+  if (i < fh) at = i;
+  else if (i < fh + H) dat = i - fh;
+  else if (i < fh + H + hh) at = i - H;
+  else if (i < P) dat = H + (i - fh - H - hh);
+  else if (i == P) dat = 3 * H + 1;
+  double s = 0.0;
+  if (at >= 0) {
+    float f = 0.f;
+#pragma unroll 8
+    for (int z = gq; z < slots; z += kG) f += __ldg(part + z * (fh + hh) + at);
+    s = f;
+  } else if (dat >= 0) {
+    for (int z = gq; z < slots; z += kG) s += __ldg(dpart + z * (3 * static_cast<int64_t>(H) + 2) + dat);
+  }
+  sh[gq][threadIdx.x] = s;
+  __syncthreads();
+  if (gq != 0 || i > P) return;
+#pragma unroll
+  for (int q = 1; q < kG; ++q) s += sh[q][threadIdx.x];
+  if (i == P) {
+    *loss = s / static_cast<double>(n);
+    return;
+  }
+  const float gi = static_cast<float>(s);
+  grad[i] = gi;
+  if (a.on) {
+    const float th = adam_step(a.theta[i], gi, a.m + i, a.v + i, a.lr, a.c1, a.c2);
+    a.theta[i] = th;
+    if (i < fh) a.W1[i] = __float2bfloat16_rn(th);
+    else if (i >= fh + H && i < fh + H + hh) a.W2[i - fh - H] = __float2bfloat16_rn(th);
+    else if (i >= fh + 2 * H + hh && i < P - 1) a.w3[i - fh - 2 * H - hh] = __float2bfloat16_rn(th);
+  }
 }
 
 int grid_for(int64_t n, int threads = 256) {
@@ -541,7 +1051,18 @@ struct dlm_ws {
   int64_t part_cap = 0;
   double* loss = nullptr;  // [loss_cap]
   int64_t loss_cap = 0;
+  // result block: the gradient (grad, P floats), then a loss and gemm_err, so that one copy brings them to the host
+  void* res = nullptr;
+  void* h_res = nullptr;    // pinned
+  double* res_loss = nullptr;
   int* gemm_err = nullptr;  // set by a tensor-core product whose completion wait ran out (device)
+  size_t res_bytes() const { return res_tail() + 16; }
+  size_t res_tail() const { return (static_cast<size_t>(P) * 4 + 7) / 8 * 8; }
+  // fused network (H <= kMaxFused): one slot of partial gradients per CTA
+  int sms = 0;
+  float* mpart = nullptr;
+  double* mdpart = nullptr;
+  bool fused() const { return H <= kMaxFused; }
 };
 
 namespace {
@@ -591,7 +1112,7 @@ dlm_status ensure_part(dlm_ws* w, int64_t need) {
 }
 
 dlm_status ensure_work(dlm_ws* w, int64_t n) {
-  if (n <= w->cap) return DLM_OK;
+  if (w->fused() || n <= w->cap) return DLM_OK;  // the fused network needs no workspace of rows
   WCK(cudaStreamSynchronize(w->stream));
   free_work(w);
   const int64_t nh = n * w->H;
@@ -653,13 +1174,69 @@ int last_splits(int64_t K, int splits) {
 // DLM_ERR_TIMEOUT when a tensor-core product's completion wait ran out
 // (the word is cleared for the next call).
 dlm_status check_gemm(dlm_ws* w) {
-  int h = 0;
-  WCK(cudaMemcpyAsync(&h, w->gemm_err, sizeof(int), cudaMemcpyDeviceToHost, w->stream));
+  int* hp = static_cast<int*>(w->h_res);
+  WCK(cudaMemcpyAsync(hp, w->gemm_err, sizeof(int), cudaMemcpyDeviceToHost, w->stream));
   WCK(cudaStreamSynchronize(w->stream));
+  const int h = *hp;
   if (h) {
     WCK(cudaMemsetAsync(w->gemm_err, 0, sizeof(int), w->stream));
     return wfail(DLM_ERR_TIMEOUT, "a tensor-core product did not complete in time");
   }
+  return DLM_OK;
+}
+
+// The fused network over n rows: the outputs into `out` (may be null) and, with y, the partial gradients.
+dlm_status fused_run(dlm_ws* w, const float* X, const float* y, int64_t n, float* out, int* slots) {
+  MlpArgs g;
+  g.X = X;
+  g.y = y;
+  g.n = n;
+  g.H = w->H;
+  g.ntiles = (n + kMlpRows - 1) / kMlpRows;
+  g.mu = w->mu;
+  g.sd = w->sd;
+  g.b1 = w->theta + w->ob1;
+  g.b2 = w->theta + w->ob2;
+  g.b3 = w->theta + w->ob3;
+  g.W1 = w->W1b;
+  g.W2 = w->W2b;
+  g.w3 = w->w3b;
+  g.out = out;
+  g.err = w->gemm_err;
+  if (y && !w->mpart) {
+    const int64_t H = w->H;
+    WCK(walloc(&w->mpart, w->sms * (kF * H + H * H)));
+    WCK(walloc(&w->mdpart, w->sms * (3 * H + 2)));
+  }
+  g.part = w->mpart;
+  g.dpart = w->mdpart;
+  const int grid = static_cast<int>(std::min<int64_t>(g.ntiles, w->sms));
+  if (w->H <= 128) {
+    if (y)
+      k_mlp<128, true><<<grid, kMlpThreads, mlp_smem(128), w->stream>>>(g);
+    else
+      k_mlp<128, false><<<grid, kMlpThreads, mlp_smem(128), w->stream>>>(g);
+  } else {
+    if (y)
+      k_mlp<256, true><<<grid, kMlpThreads, mlp_smem(256), w->stream>>>(g);
+    else
+      k_mlp<256, false><<<grid, kMlpThreads, mlp_smem(256), w->stream>>>(g);
+  }
+  WCK(cudaGetLastError());
+  if (slots) *slots = grid;
+  return DLM_OK;
+}
+
+// Loss (into *loss) and gradient (into w->grad) of the fused network at the current weights; with `adam` on,
+// the Adam step as well.
+dlm_status fused_loss_grad(dlm_ws* w, const float* X, const float* y, int64_t n, double* loss, const AdamArgs& adam) {
+  int slots = 0;
+  dlm_status st = fused_run(w, X, y, n, nullptr, &slots);
+  if (st != DLM_OK) return st;
+  const dim3 block(32, 8);
+  k_mlp_reduce<<<static_cast<unsigned>((w->P + 1 + 31) / 32), block, 0, w->stream>>>(w->mpart, w->mdpart, slots, w->H, n,
+                                                                                  w->grad, loss, adam);
+  WCK(cudaGetLastError());
   return DLM_OK;
 }
 
@@ -689,13 +1266,14 @@ dlm_status forward(dlm_ws* w, const float* X, int64_t n) {
   return DLM_OK;
 }
 
-// Loss (into w->loss[slot]) and gradient (into w->grad) at the current weights.
-dlm_status loss_grad(dlm_ws* w, const float* X, const float* y, int64_t n, int64_t slot) {
+// Loss (into *loss) and gradient (into w->grad) at the current weights.
+dlm_status loss_grad(dlm_ws* w, const float* X, const float* y, int64_t n, double* loss) {
+  if (w->fused()) return fused_loss_grad(w, X, y, n, loss, AdamArgs{});
   dlm_status st = forward(w, X, n);
   if (st != DLM_OK) return st;
   const int H = w->H;
   const int64_t nh = n * H;
-  k_loss<<<1, 1024, 0, w->stream>>>(w->out, w->s, y, n, w->dz3, w->loss + slot);
+  k_loss<<<1, 1024, 0, w->stream>>>(w->out, w->s, y, n, w->dz3, loss);
   k_dz2<<<grid_for(nh), 256, 0, w->stream>>>(w->dz3, w->w3b, w->Z2, n, H, w->dZ2);
   WCK(cudaGetLastError());
   // dW2 = H1^T dZ2 (split over rows)
@@ -787,7 +1365,6 @@ dlm_status dlm_ws_create(int32_t width, uint64_t seed, void* stream, dlm_ws** ou
     if (e != cudaSuccess && s == DLM_OK) s = wfail(DLM_ERR_CUDA, cudaGetErrorString(e));
   };
   ck(walloc(&w->theta, w->P));
-  ck(walloc(&w->grad, w->P));
   ck(walloc(&w->m, w->P));
   ck(walloc(&w->v, w->P));
   ck(walloc(&w->W1b, kF * H));
@@ -795,17 +1372,33 @@ dlm_status dlm_ws_create(int32_t width, uint64_t seed, void* stream, dlm_ws** ou
   ck(walloc(&w->w3b, H));
   ck(walloc(&w->mu, kF));
   ck(walloc(&w->sd, kF));
-  ck(walloc(&w->gemm_err, 1));
-  if (s == DLM_OK) ck(cudaMemset(w->gemm_err, 0, sizeof(int)));
+  ck(cudaMalloc(&w->res, w->res_bytes()));
+  ck(cudaMallocHost(&w->h_res, w->res_bytes()));
+  if (s == DLM_OK) {
+    w->grad = static_cast<float*>(w->res);
+    w->res_loss = reinterpret_cast<double*>(static_cast<char*>(w->res) + w->res_tail());
+    w->gemm_err = reinterpret_cast<int*>(w->res_loss + 1);
+    ck(cudaMemset(w->res, 0, w->res_bytes()));
+    int dev = 0;
+    ck(cudaGetDevice(&dev));
+    ck(cudaDeviceGetAttribute(&w->sms, cudaDevAttrMultiProcessorCount, dev));
+  }
   if (s == DLM_OK) {
     ck(cudaMemcpy(w->theta, th.data(), sizeof(float) * w->P, cudaMemcpyHostToDevice));
     ck(cudaMemset(w->m, 0, sizeof(float) * w->P));
     ck(cudaMemset(w->v, 0, sizeof(float) * w->P));
-    ck(cudaMemset(w->grad, 0, sizeof(float) * w->P));
     ck(cudaMemcpy(w->mu, zero.data(), sizeof(float) * kF, cudaMemcpyHostToDevice));
     ck(cudaMemcpy(w->sd, one.data(), sizeof(float) * kF, cudaMemcpyHostToDevice));
   }
-  if (s == DLM_OK) ck(cudaFuncSetAttribute(k_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, kGemmSmem));
+  const auto smem = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (s == DLM_OK && !w->fused()) ck(cudaFuncSetAttribute(k_gemm, smem, kGemmSmem));
+  if (s == DLM_OK && w->fused() && H <= 128) {
+    ck(cudaFuncSetAttribute(&k_mlp<128, true>, smem, mlp_smem(128)));
+    ck(cudaFuncSetAttribute(&k_mlp<128, false>, smem, mlp_smem(128)));
+  } else if (s == DLM_OK && w->fused()) {
+    ck(cudaFuncSetAttribute(&k_mlp<256, true>, smem, mlp_smem(256)));
+    ck(cudaFuncSetAttribute(&k_mlp<256, false>, smem, mlp_smem(256)));
+  }
   if (s == DLM_OK) s = refresh_bf16(w);
   if (s == DLM_OK) s = ensure_loss(w, 1);
   if (s == DLM_OK) {
@@ -875,12 +1468,17 @@ dlm_status dlm_ws_loss_grad(dlm_ws* w, const float* X, const float* y, int64_t n
   if (!w || !y) return wfail(DLM_ERR_INVALID_ARG, "null argument");
   dlm_status s = check_rows(X, n);
   if (s == DLM_OK) s = ensure_work(w, n);
-  if (s == DLM_OK) s = loss_grad(w, X, y, n, 0);
+  if (s == DLM_OK) s = loss_grad(w, X, y, n, w->res_loss);
   if (s != DLM_OK) return s;
-  if (loss) WCK(cudaMemcpyAsync(loss, w->loss, sizeof(double), cudaMemcpyDeviceToHost, w->stream));
-  if (grad) WCK(cudaMemcpyAsync(grad, w->grad, sizeof(float) * w->P, cudaMemcpyDeviceToHost, w->stream));
+  WCK(cudaMemcpyAsync(w->h_res, w->res, w->res_bytes(), cudaMemcpyDeviceToHost, w->stream));
   WCK(cudaStreamSynchronize(w->stream));
-  return check_gemm(w);
+  const char* tail = static_cast<const char*>(w->h_res) + w->res_tail();
+  int err = 0;
+  std::memcpy(&err, tail + sizeof(double), sizeof(int));
+  if (err) return check_gemm(w);
+  if (loss) std::memcpy(loss, tail, sizeof(double));
+  if (grad) std::memcpy(grad, w->h_res, sizeof(float) * w->P);
+  return DLM_OK;
 }
 
 dlm_status dlm_ws_train(dlm_ws* w, const float* X, const float* y, int64_t n, int32_t steps, float lr,
@@ -893,11 +1491,19 @@ dlm_status dlm_ws_train(dlm_ws* w, const float* X, const float* y, int64_t n, in
   if (s == DLM_OK) s = ensure_loss(w, steps > 0 ? steps : 1);
   if (s != DLM_OK) return s;
   for (int32_t k = 0; k < steps; ++k) {
-    s = loss_grad(w, X, y, n, k);
+    const double t = static_cast<double>(w->t + 1);
+    const float c1 = static_cast<float>(1.0 - std::pow(0.9, t));
+    const float c2 = static_cast<float>(1.0 - std::pow(0.999, t));
+    if (w->fused()) {
+      s = fused_loss_grad(w, X, y, n, w->loss + k,
+                          AdamArgs{true, w->theta, w->m, w->v, lr, c1, c2, w->W1b, w->W2b, w->w3b});
+      if (s != DLM_OK) return s;
+      ++w->t;
+      continue;
+    }
+    s = loss_grad(w, X, y, n, w->loss + k);
     if (s != DLM_OK) return s;
     ++w->t;
-    const float c1 = static_cast<float>(1.0 - std::pow(0.9, static_cast<double>(w->t)));
-    const float c2 = static_cast<float>(1.0 - std::pow(0.999, static_cast<double>(w->t)));
     k_adam<<<grid_for(w->P), 256, 0, w->stream>>>(w->theta, w->grad, w->m, w->v, w->P, lr, c1, c2);
     WCK(cudaGetLastError());
     s = refresh_bf16(w);
@@ -917,10 +1523,10 @@ dlm_status dlm_ws_predict(dlm_ws* w, const float* X, int64_t n, float* out) {
   if (!w || !out) return wfail(DLM_ERR_INVALID_ARG, "null argument");
   dlm_status s = check_rows(X, n);
   if (s == DLM_OK) s = ensure_work(w, n);
-  if (s == DLM_OK) s = forward(w, X, n);
+  if (s == DLM_OK) s = w->fused() ? fused_run(w, X, nullptr, n, out, nullptr) : forward(w, X, n);
   if (s != DLM_OK) return s;
-  WCK(cudaMemcpyAsync(out, w->out, sizeof(float) * n, cudaMemcpyDeviceToDevice, w->stream));
-  WCK(cudaStreamSynchronize(w->stream));
+  if (!w->fused())
+    WCK(cudaMemcpyAsync(out, w->out, sizeof(float) * n, cudaMemcpyDeviceToDevice, w->stream));
   return check_gemm(w);
 }
 
@@ -928,8 +1534,9 @@ void dlm_ws_destroy(dlm_ws* w) {
   if (!w) return;
   if (w->stream) cudaStreamSynchronize(w->stream);
   free_work(w);
-  void* ptrs[] = {w->theta, w->grad, w->m, w->v, w->W1b, w->W2b, w->w3b, w->mu, w->sd, w->part, w->loss, w->gemm_err};
+  void* ptrs[] = {w->theta, w->res, w->m, w->v, w->W1b, w->W2b, w->w3b, w->mu, w->sd, w->part, w->loss, w->mpart, w->mdpart};
   for (void* q : ptrs) cudaFree(q);
+  cudaFreeHost(w->h_res);
   if (w->own_stream && w->stream) cudaStreamDestroy(w->stream);
   delete w;
 }
