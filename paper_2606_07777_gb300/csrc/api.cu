@@ -726,7 +726,7 @@ void free_problem(dlm_problem* p) {
   runner_free(p->run);
   cudaStream_t s = p->stream;
   void* pooled[] = {p->lay.slice_off, p->lay.slice_w, p->lay.col16, p->lay.ca, p->lay.orig_off,
-                    p->lay.udeg,      p->lay.lead,    p->lay.n2,  p->a_ext};
+                    p->lay.udeg,      p->lay.lead,    p->a_ext};
   for (void* q : pooled) dev_free(q, s);
   if (s) cudaStreamSynchronize(s);
   if (p->own_sums) {

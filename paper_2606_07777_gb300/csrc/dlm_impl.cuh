@@ -256,7 +256,6 @@ struct LayoutOut {
   int32_t* udeg = nullptr;       // [num_active_users + 32]
   uint64_t* lead = nullptr;      // [num_active_users + 32] lead edges of each sorted row (lead_caller_pos)
   int64_t num_active_users = 0, nslices = 0, padded_nnz = 0;
-  double* n2 = nullptr;          // [J] sum_i a_ij^2
   double n2max = 0;
   std::vector<double> h_n2, h_s1;  // host copies: sum_i a_ij^2, sum_i a_ij
   int64_t max_item_deg = 0;

@@ -25,6 +25,7 @@
 // the same size then maps no new memory.
 #include <cub/cub.cuh>
 
+#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <cstdint>
@@ -41,6 +42,7 @@ constexpr int kT = 256;
 
 enum : int { kBadRowPtr = 1, kBadItem = 2, kBadValue = 4, kBadB = 8, kNegA = 16, kDupItem = 32 };
 constexpr unsigned kFullMask = 0xffffffffu;
+const char* const kDupMsg = "an item appears twice in one row (the eligible items of a user must be distinct)";
 constexpr int kDupThreads = 256;
 
 __device__ __forceinline__ float load_val(const void* p, int64_t e, bool bf16) {
@@ -71,10 +73,33 @@ __global__ void k_rows(const int64_t* rp, int64_t I, int64_t nnz, int32_t* deg, 
   if (z) atomicAdd(zero_cnt, z);
 }
 
+// Four consecutive values from edge 4 q on (aligned: see aligned4), as floats.
+__device__ __forceinline__ void load_val4(const void* p, int64_t q, bool bf16, float (&v)[4]) {
+  if (bf16) {
+    const uint2 w = __ldg(static_cast<const uint2*>(p) + q);
+    v[0] = __uint_as_float(w.x << 16), v[1] = __uint_as_float(w.x & 0xffff0000u);
+    v[2] = __uint_as_float(w.y << 16), v[3] = __uint_as_float(w.y & 0xffff0000u);
+  } else {
+    const float4 w = __ldg(static_cast<const float4*>(p) + q);
+    v[0] = w.x, v[1] = w.y, v[2] = w.z, v[3] = w.w;
+  }
+}
+// Whether the caller's arrays start on the boundaries that loads of four
+// edges need (any array of its own does; a view into one may not).
+inline bool aligned4(const int32_t* col, const void* c, const void* a, bool bf16) {
+  const uintptr_t m = bf16 ? 7 : 15;
+  return (reinterpret_cast<uintptr_t>(col) & 15) == 0 && ((reinterpret_cast<uintptr_t>(c) | reinterpret_cast<uintptr_t>(a)) & m) == 0;
+}
+
 // Edge checks, item degrees, max |a|, max |c|.  With J <= 16384 each block
-// counts its contiguous edge range in shared memory and flushes once per item.
-__global__ void k_edges(const int32_t* col, const void* c, const void* a, bool bf16, int64_t nnz, int64_t J,
-                        unsigned long long* item_deg, unsigned* max_a, unsigned* max_c, int* bad) {
+// counts its share of the edges in shared memory and flushes once per item.
+// Bound by the loads in flight: with `quad` (aligned arrays) a thread takes
+// four edges a step, two steps at a time (50M BF16 edges, 1,000 items: 233 us with
+// one edge a step).
+__global__ void __launch_bounds__(1024) k_edges(const int32_t* __restrict__ col, const void* __restrict__ c,
+                                                const void* __restrict__ a, bool bf16, int64_t nnz, int64_t J, bool quad,
+                                                unsigned long long* item_deg, unsigned* max_a, unsigned* max_c,
+                                                int* bad) {
   extern __shared__ unsigned scnt[];
   __shared__ unsigned s_ma, s_mc;
   const bool sm = J <= 16384;
@@ -84,25 +109,40 @@ __global__ void k_edges(const int32_t* col, const void* c, const void* a, bool b
   __syncthreads();
   int flag = 0;
   unsigned ma = 0, mc = 0;
-  const int64_t per = (nnz + gridDim.x - 1) / gridDim.x;
-  const int64_t e0 = blockIdx.x * per, e1 = e0 + per < nnz ? e0 + per : nnz;
-  for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const int32_t j = col[e];
+  auto take = [&](int32_t j, float cv, float av) {
     if (j < 0 || j >= J)
       flag |= kBadItem;
     else if (sm)
       atomicAdd(&scnt[j], 1u);
     else
       atomicAdd(&item_deg[j], 1ull);
-    const float cv = load_val(c, e, bf16), av = load_val(a, e, bf16);
     if (!isfinite(cv) || !isfinite(av)) flag |= kBadValue;
     if (av < 0.f) flag |= kNegA;
     ma = max(ma, __float_as_uint(fabsf(av)));
     mc = max(mc, __float_as_uint(fabsf(cv)));
+  };
+  const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  const int64_t nt = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t n4 = quad ? nnz >> 2 : 0;
+#pragma unroll 2
+  for (int64_t q = t; q < n4; q += nt) {
+    const int4 j = __ldg(reinterpret_cast<const int4*>(col) + q);
+    float cv[4], av[4];
+    load_val4(c, q, bf16, cv);
+    load_val4(a, q, bf16, av);
+    take(j.x, cv[0], av[0]);
+    take(j.y, cv[1], av[1]);
+    take(j.z, cv[2], av[2]);
+    take(j.w, cv[3], av[3]);
   }
+  for (int64_t e = 4 * n4 + t; e < nnz; e += nt) take(col[e], load_val(c, e, bf16), load_val(a, e, bf16));
+  ma = __reduce_max_sync(kFullMask, ma);
+  mc = __reduce_max_sync(kFullMask, mc);
   if (flag) atomicOr(bad, flag);
-  atomicMax(&s_ma, ma);
-  atomicMax(&s_mc, mc);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&s_ma, ma);
+    atomicMax(&s_mc, mc);
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
     atomicMax(max_a, s_ma);
@@ -193,20 +233,6 @@ __global__ void k_slices(const int32_t* sdeg, int64_t nslices, int32_t* width, i
   }
 }
 
-// The cost c of edge e as a float (bf16 bits widened exactly, or FP32).
-template <typename CA>
-__device__ __forceinline__ float cost_of(const void* c, int64_t e);
-template <>
-__device__ __forceinline__ float cost_of<float2>(const void* c, int64_t e) {
-  return static_cast<const float*>(c)[e];
-}
-template <>
-__device__ __forceinline__ float cost_of<uint32_t>(const void* c, int64_t e) {
-  return __uint_as_float(static_cast<uint32_t>(static_cast<const unsigned short*>(c)[e]) << 16);
-}
-
-// One warp per slice: lane t copies user t's row into column t of the slice,
-// in lead order (dlm_impl.cuh: the row's four lowest-cost edges first).
 // CA = float2 {c, a} (FP32) or uint32 (bf16 c low, bf16 a high).
 template <typename CA>
 __device__ __forceinline__ CA pack_ca(const void* c, const void* a, int64_t e);
@@ -230,97 +256,261 @@ __device__ __forceinline__ uint32_t pad_ca<uint32_t>() {
   return 0x00007F80u;  // c = bf16 +inf, a = 0
 }
 
+// Lanes' keys that order like the floats they encode (-0 as +0).
+__device__ __forceinline__ unsigned cost_key(float c) {
+  const unsigned u = __float_as_uint(c + 0.f);
+  return (u & 0x80000000u) ? ~u : u | 0x80000000u;
+}
+
+// The slices' edge streams, rows in lead order (dlm_impl.cuh: the four
+// lowest-cost edges first, of equal costs the earlier one).
+//
+// A warp takes a slice and reads each of its rows with consecutive lanes (the
+// caller's rows are contiguous), where a lane per row read every sector eight
+// times over: first for the lead edges (warp minima of the costs' keys), then
+// 32 slice positions of every row at a time, put into the slice's order in shared
+// memory -- groups of four edges 4 elements further apart than in the slice,
+// so that a row's groups fall into different banks -- and written out in whole
+// 128-bit pieces.  Slices are dealt by a counter, widest first.  The row's
+// items are at hand, so the check that none repeats is taken here too (rows of
+// at most 32 edges by __match_any_sync, longer ones by marking a bitmap of the
+// items in shared memory).  50M BF16 edges (2M rows): 1,015 us with a lane per
+// row and 480 us for the check in a pass of its own; with the item sums, a new
+// handle of that size and ten iterations went from 4,346 to 3,274 us.
+// Every item is in [0, J) here (checked before).
+constexpr int kGatherWarps = 8;
+constexpr int kStripGroups = 8;                             // groups of four edges of a strip
+constexpr int kStripElems = kStripGroups * 132 + 3 * 32;    // staged elements: the groups, then the slice's tail
 template <typename CA>
-__global__ void k_gather(const int64_t* rp, const int32_t* col, const void* c, const void* a, const int32_t* perm,
-                         const int32_t* sdeg, int64_t In, int64_t nslices, const int64_t* slice_off,
-                         const int32_t* width, uint16_t* col_o, CA* ca_o, int64_t* orig_off, int32_t* udeg,
-                         uint64_t* lead_o) {
-  const int lane = threadIdx.x & 31;
-  const int64_t w0 = (blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x) >> 5;
-  const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-  for (int64_t s = w0; s < nslices; s += nwarps) {
+__global__ void __launch_bounds__(32 * kGatherWarps)
+    k_gather(const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const void* __restrict__ c,
+             const void* __restrict__ a, const int32_t* __restrict__ perm, const int32_t* __restrict__ sdeg, int64_t In,
+             int64_t nslices, const int64_t* __restrict__ slice_off, const int32_t* __restrict__ width,
+             uint16_t* __restrict__ col_o, CA* __restrict__ ca_o, int64_t* __restrict__ orig_off,
+             int32_t* __restrict__ udeg, uint64_t* __restrict__ lead_o, int J, unsigned* __restrict__ ticket,
+             int* __restrict__ dup) {
+  constexpr bool kBf = sizeof(CA) == 4;
+  extern __shared__ __align__(16) unsigned char gsm[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  CA* sca = reinterpret_cast<CA*>(gsm + static_cast<size_t>(warp) * kStripElems * (sizeof(CA) + 2));
+  uint16_t* scol = reinterpret_cast<uint16_t*>(sca + kStripElems);
+  const int words = (J + 31) >> 5;
+  unsigned* seen = reinterpret_cast<unsigned*>(gsm + static_cast<size_t>(kGatherWarps) * kStripElems * (sizeof(CA) + 2)) +
+                   warp * words;
+  for (int k = lane; k < words; k += 32) seen[k] = 0u;
+  __syncwarp();
+  bool twice = false;
+  for (;;) {
+    unsigned tk = 0;
+    if (lane == 0) tk = atomicAdd(ticket, 1u);
+    const int64_t s = __shfl_sync(kFullMask, tk, 0);
+    if (s >= nslices) break;
     const int64_t u = 32 * s + lane;
     int64_t r = 0;
     int d = 0;
     if (u < In) {
-      const int32_t o = perm[u];
-      r = rp[o];
+      r = rp[perm[u]];
       d = sdeg[u];
       orig_off[u] = r;
       udeg[u] = d;
     }
-    // lead edges: min(4, d) edges of the row's lowest costs, ascending, by a
-    // sorted insertion with strict comparisons (a deterministic choice among
-    // edges of equal cost)
-    float lv[4] = {INFINITY, INFINITY, INFINITY, INFINITY};
-    int lp[4] = {0, 0, 0, 0};
-    for (int k = 0; k < d && k < 0xFFFF; ++k) {  // positions fit 16 bits
-      float x = cost_of<CA>(c, r + k);
-      int xi = k;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const bool lt = x < lv[q];
-        const float hv = lt ? lv[q] : x;
-        const int hi = lt ? lp[q] : xi;
-        lv[q] = lt ? x : lv[q];
-        lp[q] = lt ? xi : lp[q];
-        x = hv;
-        xi = hi;
-      }
-    }
-    uint64_t lead = 0;
-#pragma unroll
-    for (int q = 0; q < 4; ++q) lead |= static_cast<uint64_t>(q < d ? lp[q] : 0xFFFF) << (16 * q);
-    if (u < In) lead_o[u] = lead;
     const int w = width[s];
     const int w4 = w >> 2;
     const int64_t base = slice_off[s];
-    for (int k = 0; k < w; ++k) {
-      const bool v = k < d;
-      const int64_t e = k < 4 * w4 ? base + 4 * (32 * static_cast<int64_t>(k >> 2) + lane) + (k & 3)
-                                   : base + 128 * static_cast<int64_t>(w4) + 32 * static_cast<int64_t>(k - 4 * w4) + lane;
-      const int64_t src = v ? r + lead_caller_pos(lead, k, d) : 0;
-      col_o[e] = v ? static_cast<uint16_t>(col[src]) : uint16_t(0);
-      ca_o[e] = v ? pack_ca<CA>(c, a, src) : pad_ca<CA>();
+    // lead edges: lane t keeps row t's
+    uint64_t lead = 0;
+    if (w <= 32) {
+#pragma unroll 4
+      for (int t = 0; t < 32; ++t) {
+        const int64_t rt = __shfl_sync(kFullMask, r, t);
+        const int dt = __shfl_sync(kFullMask, d, t);
+        unsigned key = lane < dt ? cost_key(load_val(c, rt + lane, kBf)) : 0xffffffffu;
+        uint64_t ld = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const unsigned m = __reduce_min_sync(kFullMask, key);
+          const int who = __ffs(__ballot_sync(kFullMask, key == m)) - 1;
+          if (lane == who) key = 0xffffffffu;
+          ld |= static_cast<uint64_t>(q < dt ? who : 0xFFFF) << (16 * q);
+        }
+        if (lane == t) lead = ld;
+        const int j = lane < dt ? __ldg(col + rt + lane) : -1 - lane;  // idle lanes: distinct negative keys
+        const unsigned same = __match_any_sync(kFullMask, j);  // (by every lane, whatever it has found before)
+        if (__popc(same) > 1) twice = true;
+      }
+    } else {
+      for (int t = 0; t < 32; ++t) {
+        const int64_t rt = __shfl_sync(kFullMask, r, t);
+        const int dt = __shfl_sync(kFullMask, d, t);
+        // the lane's four lowest of edges lane, lane + 32, ... (positions fit 16 bits)
+        unsigned lk[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
+        unsigned lp[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
+        const int de = dt < 0xFFFF ? dt : 0xFFFF;
+#pragma unroll 4
+        for (int k = lane; k < de; k += 32) {
+          unsigned x = cost_key(load_val(c, rt + k, kBf)), xi = static_cast<unsigned>(k);
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const bool lt = x < lk[q];
+            const unsigned hv = lt ? lk[q] : x, hi = lt ? lp[q] : xi;
+            lk[q] = lt ? x : lk[q];
+            lp[q] = lt ? xi : lp[q];
+            x = hv;
+            xi = hi;
+          }
+        }
+        uint64_t ld = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const unsigned m = __reduce_min_sync(kFullMask, lk[0]);
+          const unsigned p = __reduce_min_sync(kFullMask, lk[0] == m ? lp[0] : 0xffffffffu);
+          if (lp[0] == p && p != 0xffffffffu) {
+#pragma unroll
+            for (int z = 0; z < 3; ++z) lk[z] = lk[z + 1], lp[z] = lp[z + 1];
+            lk[3] = lp[3] = 0xffffffffu;
+          }
+          ld |= static_cast<uint64_t>(q < dt ? p & 0xFFFFu : 0xFFFFu) << (16 * q);
+        }
+        if (lane == t) lead = ld;
+        twice = twice || dt > J;  // more edges than items: some item repeats
+        if (dt > J) continue;     // (warp-uniform)
+        for (int k = lane; k < dt; k += 32) {
+          const int j = __ldg(col + rt + k);
+          const unsigned bit = 1u << (j & 31);
+          if (atomicOr(&seen[j >> 5], bit) & bit) twice = true;
+        }
+        __syncwarp();
+        for (int k = lane; k < dt; k += 32) seen[__ldg(col + rt + k) >> 5] = 0u;
+        __syncwarp();
+      }
+    }
+    if (u < In) lead_o[u] = lead;
+    // positions 32 st .. of every row, then the strip's elements in order
+    for (int st = 0; 32 * st < w; ++st) {
+      const int k = 32 * st + lane;
+      const int at = k < 4 * w4 ? (lane >> 2) * 132 + (lane & 3) : kStripGroups * 132 + 32 * (k - 4 * w4);
+      const int by = k < 4 * w4 ? 4 : 1;
+#pragma unroll 4
+      for (int t = 0; t < 32; ++t) {
+        const int64_t rt = __shfl_sync(kFullMask, r, t);
+        const int dt = __shfl_sync(kFullMask, d, t);
+        const uint64_t lt = __shfl_sync(kFullMask, lead, t);
+        CA v = pad_ca<CA>();
+        uint16_t j = 0;
+        if (k < dt) {
+          const int64_t src = rt + lead_caller_pos(lt, k, dt);
+          v = pack_ca<CA>(c, a, src);
+          j = static_cast<uint16_t>(__ldg(col + src));
+        }
+        if (k < w) {
+          sca[at + by * t] = v;
+          scol[at + by * t] = j;
+        }
+      }
+      __syncwarp();
+      const int ng = min(kStripGroups, w4 - kStripGroups * st);
+      const int64_t o = base + 128 * static_cast<int64_t>(kStripGroups * st);
+      for (int g = 0; g < ng; ++g) {
+        if (kBf) {
+          reinterpret_cast<uint4*>(ca_o + o + 128 * g)[lane] = reinterpret_cast<const uint4*>(sca + 132 * g)[lane];
+        } else {
+          reinterpret_cast<uint4*>(ca_o + o + 128 * g)[lane] = reinterpret_cast<const uint4*>(sca + 132 * g)[lane];
+          reinterpret_cast<uint4*>(ca_o + o + 128 * g)[32 + lane] =
+              reinterpret_cast<const uint4*>(sca + 132 * g)[32 + lane];
+        }
+        reinterpret_cast<uint2*>(col_o + o + 128 * g)[lane] = reinterpret_cast<const uint2*>(scol + 132 * g)[lane];
+      }
+      if (w - 32 * st <= 32) {  // the last strip holds the tail
+        for (int q = 0; q < w - 4 * w4; ++q) {
+          const int64_t e = base + 128 * static_cast<int64_t>(w4) + 32 * q + lane;
+          ca_o[e] = sca[kStripGroups * 132 + 32 * q + lane];
+          col_o[e] = scol[kStripGroups * 132 + 32 * q + lane];
+        }
+      }
+      __syncwarp();
     }
   }
+  if (__any_sync(kFullMask, twice) && lane == 0) *dup = 1;
 }
 
+// f rounded to a 64-bit integer: fix64 where it holds, the conversion elsewhere
+// (items of small degree leave terms of up to 2^61).
+__device__ __forceinline__ unsigned long long fix_any(float f) {
+  return fabsf(f) < 36028797018963968.f ? fix64(f) : static_cast<unsigned long long>(__float2ll_rn(f));
+}
 
-// sum_i a_ij^2 (or sum_i a_ij) per item in 64-bit fixed point (exact, order
-// independent).
-// With J <= kSmemItems each block sums its contiguous edge range in shared
-// memory and flushes once per item.
-constexpr int kSmemItems = 16384;
-__global__ void k_item_sq(const int32_t* col, const void* a, bool bf16, int64_t nnz, int64_t J, float scale,
-                          bool square, unsigned long long* acc) {
+// sum_i a_ij^2 (sums[0 .. J)) and sum_i a_ij (sums[J .. 2 J)) per item in
+// 64-bit fixed point (exact, order independent); SQ, S1: which of the two.
+// Blocks add in shared memory where it holds the sums (SMEM) and flush once per
+// item.  Bound by the shared-memory atomics of the popular items: one pass
+// over the edges for both sums instead of two, four edges a step
+// (`quad`: aligned arrays), conversions off the FP64 pipe.  50M BF16 edges, 1,000 items:
+// 2 x 338 us in two passes.
+template <bool SQ, bool S1, bool SMEM>
+__global__ void __launch_bounds__(1024) k_item_sums(const int32_t* __restrict__ col, const void* __restrict__ a, bool bf16,
+                                                    int64_t nnz, int64_t J, float scale_sq, float scale_s1, bool quad,
+                                                    unsigned long long* __restrict__ sums) {
   extern __shared__ unsigned long long sacc[];
-  const bool sm = J <= kSmemItems;
-  if (sm) {
-    for (int64_t j = threadIdx.x; j < J; j += blockDim.x) sacc[j] = 0ull;
+  unsigned long long* sq = SMEM ? sacc : sums;
+  unsigned long long* s1 = (SMEM && !SQ) ? sacc : sq + J;
+  const int64_t held = (SQ && S1) ? 2 * J : J;
+  if (SMEM) {
+    for (int64_t j = threadIdx.x; j < held; j += blockDim.x) sacc[j] = 0ull;
     __syncthreads();
   }
-  const int64_t per = (nnz + gridDim.x - 1) / gridDim.x;
-  const int64_t e0 = blockIdx.x * per, e1 = e0 + per < nnz ? e0 + per : nnz;
-  for (int64_t e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-    const float av = load_val(a, e, bf16);
-    const unsigned long long q = static_cast<unsigned long long>(__float2ll_rn((square ? av * av : av) * scale));
-    if (sm)
-      atomicAdd(&sacc[col[e]], q);
-    else
-      atomicAdd(&acc[col[e]], q);
+  auto take = [&](int32_t j, float av) {
+    if (SQ) atomicAdd(&sq[j], fix_any(av * av * scale_sq));
+    if (S1) atomicAdd(&s1[j], fix_any(av * scale_s1));
+  };
+  const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
+  const int64_t nt = static_cast<int64_t>(gridDim.x) * blockDim.x;
+  const int64_t n4 = quad ? nnz >> 2 : 0;
+#pragma unroll 2
+  for (int64_t q = t; q < n4; q += nt) {
+    const int4 j = __ldg(reinterpret_cast<const int4*>(col) + q);
+    float av[4];
+    load_val4(a, q, bf16, av);
+    take(j.x, av[0]);
+    take(j.y, av[1]);
+    take(j.z, av[2]);
+    take(j.w, av[3]);
   }
-  if (sm) {
+  for (int64_t e = 4 * n4 + t; e < nnz; e += nt) take(col[e], load_val(a, e, bf16));
+  if (SMEM) {
     __syncthreads();
-    for (int64_t j = threadIdx.x; j < J; j += blockDim.x)
-      if (sacc[j]) atomicAdd(&acc[j], sacc[j]);
+    unsigned long long* out = sums + (SQ ? 0 : J);
+    for (int64_t j = threadIdx.x; j < held; j += blockDim.x)
+      if (sacc[j]) atomicAdd(&out[j], sacc[j]);
   }
 }
 
-__global__ void k_fix_to_double(const unsigned long long* acc, int64_t J, double inv_scale, double* out) {
-  for (int64_t j = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; j < J;
-       j += static_cast<int64_t>(gridDim.x) * blockDim.x)
-    out[j] = static_cast<double>(static_cast<long long>(acc[j])) * inv_scale;
+// Both sums into sums[2 J] (cleared here): one pass where shared memory holds
+// both, two passes where it holds one, else global atomics.
+cudaError_t launch_item_sums(const int32_t* col, const void* a, bool bf16, int64_t nnz, int64_t J, int ssq, int ss1,
+                             unsigned long long* sums, cudaStream_t s) {
+  cudaError_t e = cudaMemsetAsync(sums, 0, sizeof(unsigned long long) * 2 * (J > 0 ? J : 1), s);
+  if (e != cudaSuccess || nnz <= 0) return e;
+  const size_t lim = sweep_smem_limit();
+  const size_t one = sizeof(unsigned long long) * static_cast<size_t>(J);
+  const float fq = std::ldexp(1.0f, ssq), f1 = std::ldexp(1.0f, ss1);
+  const bool quad = aligned4(col, a, a, bf16);
+  int dev = 0, sms = 0;
+  e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  const int g = static_cast<int>(std::min<int64_t>(sms, nnz / 8192 + 1));  // one block of 1,024 threads per SM
+  auto go = [&](auto kernel, size_t smem) {
+    cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (f != cudaSuccess) return f;
+    kernel<<<g, 1024, smem, s>>>(col, a, bf16, nnz, J, fq, f1, quad, sums);
+    return cudaGetLastError();
+  };
+  if (2 * one <= lim) return go(&k_item_sums<true, true, true>, 2 * one);
+  if (one <= lim) {
+    e = go(&k_item_sums<true, false, true>, one);
+    return e != cudaSuccess ? e : go(&k_item_sums<false, true, true>, one);
+  }
+  return go(&k_item_sums<true, true, false>, 0);
 }
 
 int grid_for(int64_t n) {
@@ -404,19 +594,10 @@ void item_sum_shifts(int64_t max_item_deg, double max_abs_a, int* ssq, int* ss1)
 
 dlm_status item_sums(int64_t J, int64_t nnz, const int32_t* col, const void* a, bool bf16, int ssq, int ss1,
                      cudaStream_t s, int64_t* sq, int64_t* s1, std::string* msg) {
-  cudaFuncSetAttribute(k_item_sq, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kSmemItems);
   unsigned long long* acc = nullptr;
   dlm_status st = DLM_OK;
-  const int g = static_cast<int>(nnz / 8192 + 1 < 608 ? nnz / 8192 + 1 : 608);
-  const size_t smem = J <= kSmemItems ? sizeof(unsigned long long) * J : 0;
   DLM_CK(dev_alloc(reinterpret_cast<void**>(&acc), sizeof(unsigned long long) * 2 * (J > 0 ? J : 1), s));
-  DLM_CK(cudaMemsetAsync(acc, 0, sizeof(unsigned long long) * 2 * (J > 0 ? J : 1), s));
-  if (nnz > 0) {
-    k_item_sq<<<g, 1024, smem, s>>>(col, a, bf16, nnz, J, std::ldexp(1.0f, ssq), true, acc);
-    DLM_CK(cudaGetLastError());
-    k_item_sq<<<g, 1024, smem, s>>>(col, a, bf16, nnz, J, std::ldexp(1.0f, ss1), false, acc + J);
-    DLM_CK(cudaGetLastError());
-  }
+  DLM_CK(launch_item_sums(col, a, bf16, nnz, J, ssq, ss1, acc, s));
   DLM_CK(cudaMemcpyAsync(sq, acc, sizeof(int64_t) * J, cudaMemcpyDeviceToHost, s));
   DLM_CK(cudaMemcpyAsync(s1, acc + J, sizeof(int64_t) * J, cudaMemcpyDeviceToHost, s));
   DLM_CK(cudaStreamSynchronize(s));
@@ -438,7 +619,6 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
                       (k > 0 ? out->phase_s[0] : 0.0) - (k > 1 ? out->phase_s[1] : 0.0);
   };
   const size_t vs = bf16 ? 2 : 4;
-  cudaFuncSetAttribute(k_item_sq, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kSmemItems);
   cudaFuncSetAttribute(k_edges, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 16384);
   dlm_status st = DLM_OK;
   int32_t *deg = nullptr, *sdeg = nullptr, *idx = nullptr, *perm = nullptr;
@@ -448,19 +628,18 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
   int* bad = nullptr;
   void* tmp = nullptr;
   size_t tmp_bytes = 0;
-  int h_bad = 0;
+  int h_bad = 0, h_dup = 0;
   unsigned h_mx[2] = {0, 0};
   unsigned long long h_zero = 0;
   std::vector<unsigned long long> h_deg;
-  double bound_sq = 0;
-  int ssq = 0;
+  int ssq = 0, ss1 = 0;
   int64_t In = 0, ns = 0;
 
   DLM_CK(dev_alloc(reinterpret_cast<void**>(&deg), sizeof(int32_t) * (I > 0 ? I : 1), s));
   DLM_CK(dev_alloc(reinterpret_cast<void**>(&zero_cnt), sizeof(unsigned long long), s));
   DLM_CK(dev_alloc(reinterpret_cast<void**>(&item_deg), sizeof(unsigned long long) * (J > 0 ? J : 1), s));
   DLM_CK(dev_alloc(reinterpret_cast<void**>(&mx), sizeof(unsigned) * 2, s));
-  DLM_CK(dev_alloc(reinterpret_cast<void**>(&bad), sizeof(int), s));
+  DLM_CK(dev_alloc(reinterpret_cast<void**>(&bad), 2 * sizeof(int), s));
   DLM_CK(cudaMemsetAsync(zero_cnt, 0, sizeof(unsigned long long), s));
   DLM_CK(cudaMemsetAsync(item_deg, 0, sizeof(unsigned long long) * (J > 0 ? J : 1), s));
   DLM_CK(cudaMemsetAsync(mx, 0, sizeof(unsigned) * 2, s));
@@ -483,19 +662,21 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
     goto done;
   }
   if (nnz > 0) {
-    const int g = static_cast<int>(nnz / 8192 + 1 < 608 ? nnz / 8192 + 1 : 608);
-    const size_t smem = J <= 16384 ? sizeof(unsigned) * J : 0;
-    k_edges<<<g, 1024, smem, s>>>(col, c, a, bf16, nnz, J, item_deg, mx, mx + 1, bad);
-    DLM_CK(cudaGetLastError());
-    const size_t dsm = sizeof(unsigned) * static_cast<size_t>((J + 31) / 32) * (kDupThreads / 32);
-    if (dsm > 48 * 1024) DLM_CK(cudaFuncSetAttribute(k_dups, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                    static_cast<int>(dsm)));
     int dev = 0, sms = 0;
     DLM_CK(cudaGetDevice(&dev));
     DLM_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const int64_t want = (I + kDupThreads - 1) / kDupThreads;
-    const int gd = static_cast<int>(want < 8LL * sms ? (want > 0 ? want : 1) : 8LL * sms);
-    k_dups<<<gd, kDupThreads, dsm, s>>>(rp, col, I, J, bad);
+    const int g = static_cast<int>(std::min<int64_t>(sms, nnz / 8192 + 1));  // one block of 1,024 threads per SM
+    const size_t smem = J <= 16384 ? sizeof(unsigned) * J : 0;
+    k_edges<<<g, 1024, smem, s>>>(col, c, a, bf16, nnz, J, aligned4(col, c, a, bf16), item_deg, mx, mx + 1, bad);
+    DLM_CK(cudaGetLastError());
+    if (measure) {  // no layout is built: the items' repeats are checked apart
+      const size_t dsm = sizeof(unsigned) * static_cast<size_t>((J + 31) / 32) * (kDupThreads / 32);
+      if (dsm > 48 * 1024) DLM_CK(cudaFuncSetAttribute(k_dups, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                      static_cast<int>(dsm)));
+      const int64_t want = (I + kDupThreads - 1) / kDupThreads;
+      const int gd = static_cast<int>(want < 8LL * sms ? (want > 0 ? want : 1) : 8LL * sms);
+      k_dups<<<gd, kDupThreads, dsm, s>>>(rp, col, I, J, bad);
+    }
   }
   DLM_CK(cudaGetLastError());
   DLM_CK(cudaMemcpyAsync(&h_bad, bad, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -516,7 +697,7 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
     goto done;
   }
   if (h_bad & kDupItem) {
-    *msg = "an item appears twice in one row (the eligible items of a user must be distinct)";
+    *msg = kDupMsg;
     st = DLM_ERR_INVALID_ARG;
     goto done;
   }
@@ -600,19 +781,37 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
   DLM_CK(dev_alloc(reinterpret_cast<void**>(&out->lead), sizeof(uint64_t) * (In + 32), s));
   DLM_CK(cudaMemsetAsync(out->col16 + out->padded_nnz, 0, sizeof(uint16_t) * 64, s));
   if (ns > 0) {
-    const int g = grid_for(ns * 32);
-    if (bf16)
-      k_gather<uint32_t><<<g, kT, 0, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off, out->slice_w, out->col16,
-                                          static_cast<uint32_t*>(out->ca), out->orig_off, out->udeg, out->lead);
-    else
-      k_gather<float2><<<g, kT, 0, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off, out->slice_w, out->col16,
-                                        static_cast<float2*>(out->ca), out->orig_off, out->udeg, out->lead);
+    // `bad` has been read: its words serve as the slice counter and the flag of a repeated item
+    DLM_CK(cudaMemsetAsync(bad, 0, 2 * sizeof(int), s));
+    unsigned* ticket = reinterpret_cast<unsigned*>(bad);
+    int dev = 0, sms = 0;
+    DLM_CK(cudaGetDevice(&dev));
+    DLM_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int gsm = kGatherWarps * (kStripElems * static_cast<int>(2 + 2 * vs) + 4 * static_cast<int>((J + 31) / 32));
+    const int64_t want = (ns + kGatherWarps - 1) / kGatherWarps;
+    const int64_t most = static_cast<int64_t>(sms) * (bf16 ? 4 : 2);  // blocks that fit at once
+    const int g = static_cast<int>(want < most ? want : most);
+    if (bf16) {
+      DLM_CK(cudaFuncSetAttribute(&k_gather<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, gsm));
+      k_gather<uint32_t><<<g, 32 * kGatherWarps, gsm, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off,
+                                                           out->slice_w, out->col16, static_cast<uint32_t*>(out->ca),
+                                                           out->orig_off, out->udeg, out->lead, static_cast<int>(J),
+                                                           ticket, bad + 1);
+    } else {
+      DLM_CK(cudaFuncSetAttribute(&k_gather<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, gsm));
+      k_gather<float2><<<g, 32 * kGatherWarps, gsm, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off,
+                                                         out->slice_w, out->col16, static_cast<float2*>(out->ca),
+                                                         out->orig_off, out->udeg, out->lead, static_cast<int>(J),
+                                                           ticket, bad + 1);
+    }
     DLM_CK(cudaGetLastError());
   }
 
   // ---- n_j = sum_i a_ij^2 and s_j = sum_i a_ij (exact fixed point; the
   // whole instance's sums for a shard) ----
   if (shard) {
+    DLM_CK(cudaMemcpyAsync(&h_dup, bad + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
+    DLM_CK(cudaStreamSynchronize(s));
     int sq_shift = 0, s1_shift = 0;
     item_sum_shifts(out->max_item_deg, out->max_abs_a, &sq_shift, &s1_shift);
     out->h_n2.assign(J > 0 ? J : 1, 0.0);
@@ -623,47 +822,33 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
       out->h_s1[j] = static_cast<double>(shard->item_sum[j]) * std::ldexp(1.0, -s1_shift);
       out->n2max = out->h_n2[j] > out->n2max ? out->h_n2[j] : out->n2max;
     }
-    DLM_CK(dev_alloc(reinterpret_cast<void**>(&out->n2), sizeof(double) * (J > 0 ? J : 1), s));
-    DLM_CK(cudaMemcpyAsync(out->n2, out->h_n2.data(), sizeof(double) * out->h_n2.size(), cudaMemcpyHostToDevice, s));
     DLM_CK(cudaStreamSynchronize(s));
     lap(2);
-    goto done;
+    goto checked;
   }
-  bound_sq = static_cast<double>(out->max_item_deg) * out->max_abs_a * out->max_abs_a;
-  ssq = fixed_point_shift(bound_sq);
-  DLM_CK(dev_alloc(reinterpret_cast<void**>(&sq), sizeof(unsigned long long) * (J > 0 ? J : 1), s));
-  DLM_CK(dev_alloc(reinterpret_cast<void**>(&out->n2), sizeof(double) * (J > 0 ? J : 1), s));
-  DLM_CK(cudaMemsetAsync(sq, 0, sizeof(unsigned long long) * (J > 0 ? J : 1), s));
-  if (nnz > 0) {
-    const int g = static_cast<int>(nnz / 8192 + 1 < 608 ? nnz / 8192 + 1 : 608);
-    const size_t smem = J <= kSmemItems ? sizeof(unsigned long long) * J : 0;
-    k_item_sq<<<g, 1024, smem, s>>>(col, a, bf16, nnz, J, std::ldexp(1.0f, ssq), true, sq);
-  }
-  DLM_CK(cudaGetLastError());
-  if (J > 0) k_fix_to_double<<<grid_for(J), kT, 0, s>>>(sq, J, std::ldexp(1.0, -ssq), out->n2);
-  DLM_CK(cudaGetLastError());
-  out->h_n2.assign(J > 0 ? J : 1, 0.0);
-  DLM_CK(cudaMemcpyAsync(out->h_n2.data(), out->n2, sizeof(double) * out->h_n2.size(), cudaMemcpyDeviceToHost, s));
-  // ---- s_j = sum_i a_ij (the coupling of item rows with a count row) ----
-  ssq = fixed_point_shift(static_cast<double>(out->max_item_deg) * out->max_abs_a);
-  DLM_CK(cudaMemsetAsync(sq, 0, sizeof(unsigned long long) * (J > 0 ? J : 1), s));
-  if (nnz > 0) {
-    const int g = static_cast<int>(nnz / 8192 + 1 < 608 ? nnz / 8192 + 1 : 608);
-    const size_t smem = J <= kSmemItems ? sizeof(unsigned long long) * J : 0;
-    k_item_sq<<<g, 1024, smem, s>>>(col, a, bf16, nnz, J, std::ldexp(1.0f, ssq), false, sq);
-  }
-  DLM_CK(cudaGetLastError());
+  item_sum_shifts(out->max_item_deg, out->max_abs_a, &ssq, &ss1);
+  DLM_CK(dev_alloc(reinterpret_cast<void**>(&sq), sizeof(unsigned long long) * 2 * (J > 0 ? J : 1), s));
+  DLM_CK(launch_item_sums(col, a, bf16, nnz, J, ssq, ss1, sq, s));
   {
-    std::vector<unsigned long long> q(J > 0 ? J : 1);
+    std::vector<unsigned long long> q(2 * static_cast<size_t>(J > 0 ? J : 1));
+    DLM_CK(cudaMemcpyAsync(&h_dup, bad + 1, sizeof(int), cudaMemcpyDeviceToHost, s));
     DLM_CK(cudaMemcpyAsync(q.data(), sq, sizeof(unsigned long long) * q.size(), cudaMemcpyDeviceToHost, s));
     DLM_CK(cudaStreamSynchronize(s));
+    out->h_n2.assign(J > 0 ? J : 1, 0.0);
     out->h_s1.assign(J > 0 ? J : 1, 0.0);
-    for (int64_t j = 0; j < J; ++j)
-      out->h_s1[j] = static_cast<double>(static_cast<long long>(q[j])) * std::ldexp(1.0, -ssq);
     out->n2max = 0;
-    for (int64_t j = 0; j < J; ++j) out->n2max = out->h_n2[j] > out->n2max ? out->h_n2[j] : out->n2max;
+    for (int64_t j = 0; j < J; ++j) {
+      out->h_n2[j] = static_cast<double>(static_cast<long long>(q[j])) * std::ldexp(1.0, -ssq);
+      out->h_s1[j] = static_cast<double>(static_cast<long long>(q[J + j])) * std::ldexp(1.0, -ss1);
+      out->n2max = out->h_n2[j] > out->n2max ? out->h_n2[j] : out->n2max;
+    }
   }
   lap(2);
+checked:
+  if (ns > 0 && h_dup) {
+    *msg = kDupMsg;
+    st = DLM_ERR_INVALID_ARG;
+  }
   goto done;
 
 fail:
@@ -688,7 +873,6 @@ done:
     dev_free(out->orig_off, s);
     dev_free(out->udeg, s);
     dev_free(out->lead, s);
-    dev_free(out->n2, s);
     out->slice_w = nullptr;
     out->slice_off = nullptr;
     out->col16 = nullptr;
@@ -696,7 +880,6 @@ done:
     out->orig_off = nullptr;
     out->udeg = nullptr;
     out->lead = nullptr;
-    out->n2 = nullptr;
   }
   return st;
 }
