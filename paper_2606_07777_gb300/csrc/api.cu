@@ -38,8 +38,6 @@ dlm_status fail(dlm_status s, const std::string& m) {
     if (e_ != cudaSuccess) return fail(DLM_ERR_CUDA, std::string(#x) + ": " + cudaGetErrorString(e_)); \
   } while (0)
 
-__global__ void k_set_double(double* p, double v) { *p = v; }
-
 // lam <- max(src, 0), y <- lam, theta <- 1 (warm start); the FP64 iterate
 // and its FP32 copies.
 __global__ void k_warm(const float* src, double* lam64, double* y64, float* lam, float* y, int64_t J,
@@ -122,7 +120,8 @@ struct Runner {
   bool short_rows = false;   // iteration sweeps take the short-row sweep (sweep_short.cu)
   int upd_ctas = 1;      // update grid width (the largest member's)
   InstDesc *inst_iter = nullptr, *inst_stats = nullptr;
-  InstDesc h_iter0{};  // host copy of inst_iter[0]
+  InstDesc h_iter0{}, h_stats0{};  // host copies of inst_iter[0], inst_stats[0]
+  StatsInst h_st0{};               // and of st_stats[0]
   double* cuts = nullptr;  // per-instance DLM_BOX_CUT budgets (box-cut runners only)
   UpdInst* upd = nullptr;
   StatsInst* st_stats = nullptr;
@@ -192,16 +191,12 @@ struct dlm_problem {
   double* upd_part = nullptr;               // update partials [update_parts(m J + 1)]
   unsigned* upd_ticket = nullptr;
   int64_t traj_from = 0;                    // first iteration whose trajectory entry is valid
-  double *gamma_tab = nullptr, *calc_gamma = nullptr, *stats_out = nullptr;
+  double *gamma_tab = nullptr, *stats_out = nullptr;
   int64_t nstages = 1, gamma_tab_cap = 0;
   DevState* state = nullptr;
-  InstDesc* inst_calc = nullptr;
-  StatsInst* st_calc = nullptr;
 
   // pinned host staging
-  double* h_out = nullptr;  // 8 doubles
-  InstDesc* h_inst = nullptr;
-  StatsInst* h_stinst = nullptr;
+  double* h_out = nullptr;  // kStatsOut doubles
 
   double gamma0 = 1e-2, gamma_end = 1e-2, factor = 0.5;
   int64_t ips = 1 << 30;
@@ -262,6 +257,8 @@ StatsInst base_stats(const dlm_problem* p, const Runner& R, int i) {
   s.inv_sC = std::ldexp(1.0, -p->sC);
   s.inv_sQ = std::ldexp(1.0, -p->sQ);
   s.out = p->stats_out;
+  s.part = p->upd_part;
+  s.ticket = p->upd_ticket;
   s.certified = p->certified ? 1 : 0;
   s.count_on = p->count_on ? 1 : 0;
   s.cnt = p->cnt2;
@@ -475,6 +472,8 @@ dlm_status write_tables(Runner& R) {
     st[i].state = p->state;
   }
   R.h_iter0 = it[0];
+  R.h_stats0 = ss[0];
+  R.h_st0 = st[0];
   CK(cudaMemcpy(R.inst_iter, it.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.inst_stats, ss.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(R.upd, up.data(), sizeof(UpdInst) * n, cudaMemcpyHostToDevice));
@@ -595,9 +594,18 @@ dlm_status enqueue_iteration(Runner& R) {
   return DLM_OK;
 }
 
-dlm_status enqueue_certificate(Runner& R, const InstDesc* inst_tab, const StatsInst* st_tab) {
-  CK(dispatch_sweep(R, launch_of(R, inst_tab), true, R.bf16));
-  CK(launch_stats(st_tab, static_cast<int>(R.probs.size()), R.stream));
+// A certificate of the runner's instances, or of the one instance described
+// by the host's descriptors.
+dlm_status enqueue_certificate(Runner& R, const InstDesc* one = nullptr, const StatsInst* st_one = nullptr) {
+  const int n = static_cast<int>(R.probs.size());
+  if (n == 1 && !one) {
+    one = &R.h_stats0;
+    st_one = &R.h_st0;
+  }
+  SweepLaunch L = launch_of(R, R.inst_stats);
+  L.inst0 = one;
+  CK(dispatch_sweep(R, L, true, R.bf16));
+  CK(launch_stats(one ? nullptr : R.st_stats, st_one, n, R.smemJ, R.stream));
   return DLM_OK;
 }
 
@@ -700,21 +708,19 @@ dlm_status runner_configure(Runner& R, const dlm_options& o, bool force) {
 }
 
 dlm_status read_stats(dlm_problem* p, dlm_stats* out) {
-  CK(cudaMemcpyAsync(p->h_out, p->stats_out, sizeof(double) * 8, cudaMemcpyDeviceToHost, p->stream));
+  CK(cudaMemcpyAsync(p->h_out, p->stats_out, sizeof(double) * kStatsOut, cudaMemcpyDeviceToHost, p->stream));
   CK(cudaStreamSynchronize(p->stream));
-  DevState hs;
-  CK(cudaMemcpy(&hs, p->state, sizeof(DevState), cudaMemcpyDeviceToHost));
   if (out) {
-    out->iter = hs.iter;
-    out->gamma = hs.gamma;
+    const int32_t status = static_cast<int32_t>(p->h_out[7]);
+    out->iter = static_cast<int64_t>(p->h_out[6]);
+    out->gamma = p->h_out[8];
     out->dual_obj = p->h_out[0];
     out->primal_obj = p->h_out[1];
     out->rel_gap = p->h_out[2];
     out->uncert_gap = p->h_out[3];
     out->max_viol = p->h_out[4];
     out->seconds = p->last_solve_seconds;
-    out->status =
-        (hs.status & kStatNumeric) ? DLM_ERR_NUMERIC : (hs.status & kStatTimeout) ? DLM_ERR_TIMEOUT : DLM_OK;
+    out->status = (status & kStatNumeric) ? DLM_ERR_NUMERIC : (status & kStatTimeout) ? DLM_ERR_TIMEOUT : DLM_OK;
     out->converged = 0;
   }
   return DLM_OK;
@@ -733,13 +739,11 @@ void free_problem(dlm_problem* p) {
     cudaFree(p->xsum);
     cudaFree(p->csum);
   }
-  void* ptrs[] = {p->b,         p->curv,      p->lam,      p->y,      p->gamma_tab, p->calc_gamma, p->stats_out,
-                  p->state,     p->inst_calc, p->st_calc,  p->lam64,  p->y64,       p->traj,       p->upd_part,
+  void* ptrs[] = {p->b,         p->curv,      p->lam,      p->y,      p->gamma_tab, p->stats_out,
+                  p->state,     p->lam64,  p->y64,       p->traj,       p->upd_part,
                   p->upd_ticket};
   for (void* q : ptrs) cudaFree(q);
   cudaFreeHost(p->h_out);
-  cudaFreeHost(p->h_inst);
-  cudaFreeHost(p->h_stinst);
   if (p->ev) cudaEventDestroy(p->ev);
   if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
   delete p;
@@ -994,6 +998,12 @@ dlm_status check_options(const dlm_options* opt) {
       opt->restart > 1 || (opt->topk != 0 && opt->topk != 4 && opt->topk != 8) || opt->short_rows < 0 ||
       opt->short_rows > 1)
     return fail(DLM_ERR_INVALID_ARG, "bad option value");
+  return DLM_OK;
+}
+
+// Certificate sweeps of one family write the edges with x > 0 only.
+dlm_status clear_x(const dlm_problem* p, float* x) {
+  if (x && p->m == 1 && p->kind != DLM_BOX_CUT) CK(cudaMemsetAsync(x, 0, sizeof(float) * p->nnz, p->stream));
   return DLM_OK;
 }
 
@@ -1343,14 +1353,9 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
   p->cnt2 = p->csum + MJ + 2 * J;
   CKC(cudaMemsetAsync(p->lam, 0, sizeof(float) * (MJ + 1), p->stream));
   CKC(cudaMemsetAsync(p->y, 0, sizeof(float) * (MJ + 1), p->stream));
-  CKC(dalloc(&p->calc_gamma, 1));
-  CKC(dalloc(&p->stats_out, 8));
+  CKC(dalloc(&p->stats_out, kStatsOut));
   CKC(dalloc(&p->state, 1));
-  CKC(dalloc(&p->inst_calc, 1));
-  CKC(dalloc(&p->st_calc, 1));
-  CKC(cudaMallocHost(reinterpret_cast<void**>(&p->h_out), sizeof(double) * 8));
-  CKC(cudaMallocHost(reinterpret_cast<void**>(&p->h_inst), sizeof(InstDesc)));
-  CKC(cudaMallocHost(reinterpret_cast<void**>(&p->h_stinst), sizeof(StatsInst)));
+  CKC(cudaMallocHost(reinterpret_cast<void**>(&p->h_out), sizeof(double) * kStatsOut));
   CKC(sweep_prepare(p->bf16));
   if (p->kind == DLM_BOX_CUT) CKC(sweep_boxcut_prepare(p->bf16));
   CKC(cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming));
@@ -1489,7 +1494,7 @@ dlm_status dlm_step_timed(dlm_problem* p, int64_t n_iters, double* sweep_ms, dou
 dlm_status dlm_get_stats(dlm_problem* p, dlm_stats* out) {
   if (!p) return fail(DLM_ERR_INVALID_ARG, "null handle");
   if (p->sharded) return shard_only_error();
-  dlm_status st = enqueue_certificate(p->run, p->run.inst_stats, p->run.st_stats);
+  dlm_status st = enqueue_certificate(p->run);
   if (st != DLM_OK) return st;
   return read_stats(p, out);
 }
@@ -1539,29 +1544,25 @@ dlm_status dlm_calculate(dlm_problem* p, const float* lambda, double gamma, doub
   if (!p || !lambda) return fail(DLM_ERR_INVALID_ARG, "null argument");
   if (p->sharded) return shard_only_error();
   if (!(gamma > 0) || !std::isfinite(gamma)) return fail(DLM_ERR_INVALID_ARG, "gamma must be > 0");
-  CK(cudaStreamSynchronize(p->stream));
-  k_set_double<<<1, 1, 0, p->stream>>>(p->calc_gamma, gamma);
-  CK(cudaGetLastError());
   InstDesc d = base_desc(p);
   d.y = lambda;
-  d.gamma = p->calc_gamma;
+  d.gamma = nullptr;
+  d.gamma_val = gamma;
   d.acc = p->acc2;
   d.accC = p->accC;
   d.accQ = p->accQ;
   d.seg_obj = p->run.seg_obj;
   d.xout = x;
-  *p->h_inst = d;
-  CK(cudaMemcpyAsync(p->inst_calc, p->h_inst, sizeof(InstDesc), cudaMemcpyHostToDevice, p->stream));
   StatsInst s = base_stats(p, p->run, 0);
   s.lam = lambda;
-  s.gamma = p->calc_gamma;
+  s.gamma = nullptr;
+  s.gamma_val = gamma;
   s.grad_out = grad;
   s.state = nullptr;
-  *p->h_stinst = s;
-  CK(cudaMemcpyAsync(p->st_calc, p->h_stinst, sizeof(StatsInst), cudaMemcpyHostToDevice, p->stream));
-  dlm_status st = enqueue_certificate(p->run, p->inst_calc, p->st_calc);
+  dlm_status st = clear_x(p, x);
+  if (st == DLM_OK) st = enqueue_certificate(p->run, &d, &s);
   if (st != DLM_OK) return st;
-  CK(cudaMemcpyAsync(p->h_out, p->stats_out, sizeof(double) * 8, cudaMemcpyDeviceToHost, p->stream));
+  CK(cudaMemcpyAsync(p->h_out, p->stats_out, sizeof(double) * kStatsOut, cudaMemcpyDeviceToHost, p->stream));
   CK(cudaStreamSynchronize(p->stream));
   if (g) *g = p->h_out[0];
   return DLM_OK;
@@ -1583,7 +1584,6 @@ dlm_status dlm_get_x(dlm_problem* p, float* out, int32_t memspace) {
     CK(dalloc(&tmp, p->nnz));
     dst = tmp;
   }
-  CK(cudaStreamSynchronize(p->stream));
   InstDesc d = base_desc(p);
   d.y = p->lam;
   d.gamma = &p->state->gamma;
@@ -1592,15 +1592,12 @@ dlm_status dlm_get_x(dlm_problem* p, float* out, int32_t memspace) {
   d.accQ = p->accQ;
   d.seg_obj = p->run.seg_obj;
   d.xout = dst;
-  *p->h_inst = d;
-  CK(cudaMemcpyAsync(p->inst_calc, p->h_inst, sizeof(InstDesc), cudaMemcpyHostToDevice, p->stream));
   StatsInst s = base_stats(p, p->run, 0);
   s.lam = p->lam;
   s.gamma = &p->state->gamma;
   s.state = p->state;
-  *p->h_stinst = s;
-  CK(cudaMemcpyAsync(p->st_calc, p->h_stinst, sizeof(StatsInst), cudaMemcpyHostToDevice, p->stream));
-  dlm_status st = enqueue_certificate(p->run, p->inst_calc, p->st_calc);
+  dlm_status st = clear_x(p, dst);
+  if (st == DLM_OK) st = enqueue_certificate(p->run, &d, &s);
   if (st == DLM_OK && tmp) {
     CK(cudaMemcpyAsync(out, tmp, sizeof(float) * p->nnz, cudaMemcpyDeviceToHost, p->stream));
     CK(cudaStreamSynchronize(p->stream));
@@ -1746,7 +1743,9 @@ dlm_status dlm_shard_update(dlm_problem* p) {
 dlm_status dlm_shard_cert_sweep(dlm_problem* p) {
   dlm_status st = shard_handle(p);
   if (st != DLM_OK) return st;
-  CK(dispatch_sweep(p->run, launch_of(p->run, p->run.inst_stats), true, p->bf16));
+  SweepLaunch L = launch_of(p->run, p->run.inst_stats);
+  L.inst0 = &p->run.h_stats0;
+  CK(dispatch_sweep(p->run, L, true, p->bf16));
   CK(launch_seg_sum(p->run.st_stats, p->cobj, p->stream));
   return DLM_OK;
 }
@@ -1754,7 +1753,7 @@ dlm_status dlm_shard_cert_sweep(dlm_problem* p) {
 dlm_status dlm_shard_cert_finish(dlm_problem* p, dlm_stats* out) {
   dlm_status st = shard_handle(p);
   if (st != DLM_OK) return st;
-  CK(launch_stats(p->run.st_stats, 1, p->stream));
+  CK(launch_stats(nullptr, &p->run.h_st0, 1, p->run.smemJ, p->stream));
   return read_stats(p, out);
 }
 
@@ -1910,7 +1909,7 @@ dlm_status dlm_batch_get_stats(dlm_batch* bt, dlm_stats* out) {
   if (!bt) return fail(DLM_ERR_INVALID_ARG, "null batch");
   Runner& R = bt->run;
   dlm_status st = batch_enter(R);
-  if (st == DLM_OK) st = enqueue_certificate(R, R.inst_stats, R.st_stats);
+  if (st == DLM_OK) st = enqueue_certificate(R);
   if (st != DLM_OK) return st;
   CK(cudaStreamSynchronize(R.stream));
   for (size_t i = 0; i < R.probs.size(); ++i) {

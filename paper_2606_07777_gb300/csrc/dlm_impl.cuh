@@ -17,6 +17,7 @@ constexpr int kWarp = 32;
 constexpr int kSweepThreads = 1024;  // 32 warps per sweep CTA, one CTA per SM
 constexpr int kUpdThreads = 1024;    // one CTA per instance for the O(J) kernels
 constexpr int64_t kMaxStageTable = int64_t(1) << 20;  // continuation stages a schedule may take to reach gamma_end
+constexpr int kStatsOut = 16;        // doubles of a certificate's result
 constexpr int kTrajCap = 4096;       // dual objective values kept per handle (ring, one per iteration)
 constexpr int kMaxSegTasks = 16;     // tasks of one instance in one CTA
 constexpr int kMaxFamilies = 4;      // capacity families per instance (Def. 1)
@@ -83,7 +84,8 @@ struct InstDesc {
   int64_t nusers;           // users with edges (sorted users 0 .. nusers-1)
   int32_t* status;          // device error word (kStat* bits)
   const float* y;           // sweep point [J]
-  const double* gamma;      // ridge used by this sweep
+  const double* gamma;      // ridge used by this sweep (nullptr: gamma_val)
+  double gamma_val;
   unsigned long long* acc;  // [J] fixed-point sum a x
   unsigned long long* accC; // [J] fixed-point sum c x (stats)
   unsigned long long* accQ; // [J] fixed-point sum x^2 (stats)
@@ -174,7 +176,7 @@ struct SweepLaunch {
   bool count;               // some instance has a global count constraint (its own instantiation)
   int32_t fam;              // capacity families (> 1: the general sweep of sweep_multi.cu)
   int32_t topk = 4;         // one-family sweep: largest values tracked per row in the first pass (4 or 8)
-  // iteration sweeps of one instance: host copy of its descriptor (a kernel parameter)
+  // one instance: host copy of its descriptor (a kernel parameter instead of the table)
   const InstDesc* inst0 = nullptr;
   // Short-row sweep (iteration sweeps of a single one-family handle without a
   // count constraint, sweep_short.cu): slices 0 .. nslices0 - 1 of instance 0.
@@ -186,7 +188,8 @@ constexpr int kDefaultCoopMax = 12;
 struct StatsInst {
   const double* b;
   const float* lam;           // dual point the certificate sweep used
-  const double* gamma;
+  const double* gamma;        // nullptr: gamma_val
+  double gamma_val;
   unsigned long long *acc, *accC, *accQ;
   const double* seg_obj;
   const int32_t* seg_list;    // task indices that start a segment of this instance, ascending
@@ -194,7 +197,9 @@ struct StatsInst {
   int32_t J;
   double inv_sG, inv_sC, inv_sQ;
   float* grad_out;            // optional [J] (+1 with the count constraint)
-  double* out;                // [8]: g, P, rel_gap, uncert_gap, max_viol, obj, iter, status
+  double* out;                // [kStatsOut]: g, P, rel_gap, uncert_gap, max_viol, obj, iter, status, gamma
+  double* part;               // [update_parts(m J + 1)] per-CTA partials (the update's: work on one stream)
+  unsigned* ticket;           // CTAs of the instance done (reset by the last)
   const DevState* state;
   int32_t certified;          // 0: scaled point not certified (EQ simplex or a < 0)
   int32_t count_on;
@@ -232,7 +237,9 @@ cudaError_t launch_sweep_short(const SweepLaunch& L, bool bf16);
 cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, cudaStream_t s);
 int update_ctas(int64_t D);
 int update_parts(int64_t D);  // doubles of UpdInst::part for D coordinates
-cudaError_t launch_stats(const StatsInst* dev_tab, int ninst, cudaStream_t s);
+// The certificate's reductions: of ninst instances of the table, the largest of
+// maxJ items, or (dev_tab null) of the one instance *one.
+cudaError_t launch_stats(const StatsInst* dev_tab, const StatsInst* one, int ninst, int maxJ, cudaStream_t s);
 // The certificate sweep's objective partials of instance 0 summed into *out.
 cudaError_t launch_seg_sum(const StatsInst* dev_tab, double* out, cudaStream_t s);
 // sweep_multi.cu (m > 1 families; static tasks only)

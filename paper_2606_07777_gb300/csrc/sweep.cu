@@ -55,6 +55,21 @@ struct Counted : Base {
   static constexpr bool kCount = true;
 };
 
+// Where a certificate sweep writes a row's x, in the caller's order: the
+// output is cleared before the sweep (by the caller) and only the edges with
+// x > 0 are written, as they are deposited.  (Every edge written by the row's lane, its
+// position decoded from the lead record each time: 315 us for 1M rows, 25M
+// edges FP32; that evaluation went from 378 to 166 us with this and the
+// reductions of stats_kernel spread over CTAs.)
+struct XRow {
+  float* x;  // the row's first edge, or nullptr
+  uint64_t lead;
+  int d;
+  __device__ __forceinline__ void put(int k, float v) const {
+    if (x != nullptr) x[lead_caller_pos(lead, k, d)] = v;
+  }
+};
+
 // Threshold of user t of the slice computed by the whole warp: lane l takes
 // edges l, l + 32, ... of the user (re-read from L1/L2; the warp has just
 // streamed them), the Michelot sums and the pair-arithmetic refinement are
@@ -67,8 +82,8 @@ template <class P, bool STATS>
 __device__ __forceinline__ void coop_user(const Seg& S, const float* __restrict__ ys, unsigned long long* accG,
                                           unsigned long long* accC, unsigned long long* accQ,
                                           const typename P::IX* __restrict__ cp0, const typename P::T* __restrict__ vp0,
-                                          int w, int w4, int t, float tau0, bool exact, float& tau, float& taul,
-                                          bool& zero, float& ob, unsigned long long& cn) {
+                                          int w, int w4, int t, float tau0, bool exact, const XRow& xr, float& tau,
+                                          float& taul, bool& zero, float& ob, unsigned long long& cn) {
   const int lane = threadIdx.x & 31;
   const bool box = S.kind == DLM_BOX;
   const bool eq = S.kind == DLM_SIMPLEX_EQ;
@@ -142,7 +157,10 @@ __device__ __forceinline__ void coop_user(const Seg& S, const float* __restrict_
     float c, a;
     if (uval(k, j, c, a) > tau) {
       const float x = x_general(S, box, tau, taul, c, a, ys[j]);
-      if (x > 0.f) deposit<P, STATS>(S, j, c, a, x, accG, accC, accQ, ob, cn);
+      if (x > 0.f) {
+        deposit<P, STATS>(S, j, c, a, x, accG, accC, accQ, ob, cn);
+        if (STATS) xr.put(k, x);
+      }
     }
   }
 }
@@ -261,6 +279,11 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
   const bool eq = S.kind == DLM_SIMPLEX_EQ;
   const float v0 = tk.v[0];
   const int i0 = tk.id[0];
+  XRow xr{nullptr, 0, 0};
+  if (STATS && D.xout != nullptr) {
+    const int64_t u = 32 * s + lane;
+    if (u < D.nusers) xr = XRow{D.xout + __ldg(D.orig_off + u), __ldg(D.lead + u), __ldg(D.udeg + u)};
+  }
 
   // The equality threshold solves sum_k max(u_k - tau, 0) = gamma z.  With
   // the values sorted, tau_r = (v_0 + ... + v_{r-1} - gamma z) / r and the
@@ -335,7 +358,10 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
       float c, a;
       P::get(__ldg(ca0 + el), c, a);
       const float x = x_general(S, false, tau, taul, c, a, ys[j]);
-      if (x > 0.f) deposit<P, STATS>(S, j, c, a, x, accG, accC, accQ, ob, cn);
+      if (x > 0.f) {
+        deposit<P, STATS>(S, j, c, a, x, accG, accC, accQ, ob, cn);
+        if (STATS) xr.put(tk.id[i], x);
+      }
     }
   } else if (mode == 1) {
     const int el = sell_el(i0, lane, w4);
@@ -343,6 +369,7 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
     float c, a;
     P::get(__ldg(ca0 + el), c, a);
     deposit<P, STATS>(S, j, c, a, S.z, accG, accC, accQ, ob, cn);
+    if (STATS) xr.put(i0, S.z);
   }
 
   // Mode 3 (K or more active edges, or the box): the whole warp per user
@@ -361,7 +388,11 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
       // goes to fixed point on its own, so the total does not depend on
       // which users share the warp
       float obu = 0.f;
-      coop_user<P, STATS>(S, ys, accG, accC, accQ, col0, ca0, w, w4, t, tt, false, ta, tl, zr, obu, cn);
+      XRow xt{nullptr, 0, 0};
+      if (STATS)
+        xt = XRow{reinterpret_cast<float*>(__shfl_sync(kFull, reinterpret_cast<unsigned long long>(xr.x), t)),
+                  __shfl_sync(kFull, xr.lead, t), __shfl_sync(kFull, xr.d, t)};
+      coop_user<P, STATS>(S, ys, accG, accC, accQ, col0, ca0, w, w4, t, tt, false, xt, ta, tl, zr, obu, cn);
       if (STATS)
         ob += obu;
       else
@@ -383,16 +414,14 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
         P::idx4(col0, q, jj);
         float c[4], a[4];
         P::get4(ca0, q, c, a);
-        visit(jj[0], c[0], a[0]);
-        visit(jj[1], c[1], a[1]);
-        visit(jj[2], c[2], a[2]);
-        visit(jj[3], c[3], a[3]);
+#pragma unroll
+        for (int e = 0; e < 4; ++e) visit(4 * g + e, jj[e], c[e], a[e]);
       }
       for (int k = 4 * w4; k < w; ++k) {
         const int el = 128 * w4 + 32 * (k - 4 * w4) + lane;
         float c, a;
         P::get(__ldg(ca0 + el), c, a);
-        visit(static_cast<int>(__ldg(col0 + el)), c, a);
+        visit(k, static_cast<int>(__ldg(col0 + el)), c, a);
       }
     };
     if (!box) {
@@ -408,7 +437,7 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
         float sm = 0.f;
         int cnt = 0;
         F2 ps{0.f, 0.f};
-        row_pass([&](int j, float c, float a) {
+        row_pass([&](int k, int j, float c, float a) {
           const float y = ys[j];
           const float u = -fmaf(a, y, c);
           if (u > tau) {
@@ -436,7 +465,7 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
         if (!settled) {  // iteration cap: the sum over the current set
           psum = F2{0.f, 0.f};
           n = 0;
-          row_pass([&](int j, float c, float a) {
+          row_pass([&](int k, int j, float c, float a) {
             if (-fmaf(a, ys[j], c) > tau) {
               psum = f2_add(psum, u_pair(c, a, ys[j]));
               ++n;
@@ -457,36 +486,19 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
       taul = 0.f;
     }
     // x on the active edges (u > tau; for the box and tau = 0, u > 0)
-    row_pass([&](int j, float c, float a) {
+    row_pass([&](int k, int j, float c, float a) {
       const float y = ys[j];
       if (-fmaf(a, y, c) > tau) {
         const float x = x_general(S, box, tau, taul, c, a, y);
-        if (x > 0.f) deposit<P, STATS>(S, j, c, a, x, accG, accC, accQ, ob, cn);
+        if (x > 0.f) {
+          deposit<P, STATS>(S, j, c, a, x, accG, accC, accQ, ob, cn);
+          if (STATS) xr.put(k, x);
+        }
       }
     });
   }
 
   if (STATS) {
-    const int64_t u = 32 * s + lane;
-    if (D.xout != nullptr && u < D.nusers) {
-      // x in the caller's order, every edge of the user
-      const int64_t o = __ldg(D.orig_off + u);
-      const int d = __ldg(D.udeg + u);
-      const uint64_t ld = __ldg(D.lead + u);  // slice position k is caller edge lead_caller_pos(ld, k, d)
-      for (int k = 0; k < d; ++k) {
-        float x = 0.f;
-        if (mode == 1) {
-          x = (k == i0) ? S.z : 0.f;
-        } else if (mode >= 2) {
-          const int el = sell_el(k, lane, w4);
-          const int j = static_cast<int>(__ldg(col0 + el));
-          float c, a;
-          P::get(__ldg(ca0 + el), c, a);
-          if (-fmaf(a, ys[j], c) > tau) x = x_general(S, box, tau, taul, c, a, ys[j]);
-        }
-        D.xout[o + lead_caller_pos(ld, k, d)] = x;
-      }
-    }
     wobj += static_cast<double>(ob);
   } else {
     // the user's objective part, added exactly (64-bit fixed point)
@@ -617,6 +629,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     if (ONE) {
       S.z = sD.z;
       S.scaleG = sD.scaleG;
+      S.scaleC = sD.scaleC;
+      S.scaleQ = sD.scaleQ;
       S.scaleN = sD.scaleN;
       S.scaleO = sD.scaleO;
       S.kind = sD.kind;
@@ -797,6 +811,8 @@ cudaError_t prepare_width(int lim) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(&sweep_kernel<P, false, K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(&sweep_kernel<P, true, K, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(&sweep_kernel<P, true, K, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
@@ -815,8 +831,12 @@ cudaError_t launch_width(const SweepLaunch& L, bool stats) {
     if (w < 1) return cudaErrorInvalidValue;
     const size_t sm = sweep_stats_smem_bytes(L.smemJ, w);
     for (int jlo = 0; jlo < L.smemJ || jlo == 0; jlo += w) {
-      sweep_kernel<P, true, K, false>
-          <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, cm, jlo, w);
+      if (L.inst0 != nullptr)
+        sweep_kernel<P, true, K, true>
+            <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, cm, jlo, w);
+      else
+        sweep_kernel<P, true, K, false>
+            <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, cm, jlo, w);
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }

@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     }
     if (threadIdx.x == 0) {  // FP64 work once per CTA (as fill_seg)
       BSeg& S = sS;
-      const double g = *sD.gamma;
+      const double g = sD.gamma != nullptr ? *sD.gamma : sD.gamma_val;
       S.gamma = static_cast<float>(g);
       S.invg = static_cast<float>(1.0 / g);
       S.z = sD.z;
@@ -415,6 +415,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     if (ONE) {
       S.z = sD.z;
       S.scaleG = sD.scaleG;
+      S.scaleC = sD.scaleC;
+      S.scaleQ = sD.scaleQ;
       S.scaleO = sD.scaleO;
     }
     double wobj = 0.0;
@@ -480,6 +482,8 @@ cudaError_t prepare_values(int lim) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(&sweep_boxcut_kernel<V, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(&sweep_boxcut_kernel<V, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(&sweep_boxcut_kernel<V, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
 }
 
@@ -491,8 +495,12 @@ cudaError_t launch_values(const SweepLaunch& L, bool stats, const double* cuts) 
     if (w < 1) return cudaErrorInvalidValue;
     const size_t sm = sweep_stats_smem_bytes(L.smemJ, w);
     for (int jlo = 0; jlo < L.smemJ || jlo == 0; jlo += w) {
-      sweep_boxcut_kernel<V, true, false>
-          <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, jlo, w, cuts);
+      if (L.inst0 != nullptr)
+        sweep_boxcut_kernel<V, true, true>
+            <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, jlo, w, cuts);
+      else
+        sweep_boxcut_kernel<V, true, false>
+            <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, jlo, w, cuts);
       const cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }

@@ -116,7 +116,7 @@ struct Seg {
 // (With the update's scalars taken the same way, an iteration of the tiny
 // instance, 10,000 x 100, went from 11.6 to 6.0 us.)
 __device__ __forceinline__ void fill_seg(const InstDesc& D, int jlo, int jw, Seg& S) {
-  const double g = *D.gamma;
+  const double g = D.gamma != nullptr ? *D.gamma : D.gamma_val;
   S.gamma = static_cast<float>(g);
   S.invg = static_cast<float>(1.0 / g);
   const double gz = g * static_cast<double>(D.z);

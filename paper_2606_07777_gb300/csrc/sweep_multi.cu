@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
       for (int j = threadIdx.x; j < J; j += blockDim.x) accC[j] = accQ[j] = 0ull;
     if (threadIdx.x == 0) {  // FP64 work once per CTA (as fill_seg)
       MSeg& S = sS;
-      const double g = *sD.gamma;
+      const double g = sD.gamma != nullptr ? *sD.gamma : sD.gamma_val;
       S.gamma = static_cast<float>(g);
       S.invg = static_cast<float>(1.0 / g);
       const double gz = g * static_cast<double>(sD.z);
@@ -391,6 +391,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     if (ONE) {
       S.z = sD.z;
       S.scaleG = sD.scaleG;
+      S.scaleC = sD.scaleC;
+      S.scaleQ = sD.scaleQ;
       S.scaleO = sD.scaleO;
       S.kind = sD.kind;
       S.m = sD.m;
@@ -465,6 +467,8 @@ cudaError_t prepare_m(int lim) {
   if (e != cudaSuccess) return e;
   e = cudaFuncSetAttribute(&sweep_multi_kernel<P, false, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
   if (e != cudaSuccess) return e;
+  e = cudaFuncSetAttribute(&sweep_multi_kernel<P, true, M, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+  if (e != cudaSuccess) return e;
   return cudaFuncSetAttribute(&sweep_multi_kernel<P, true, M, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               lim);
 }
@@ -473,7 +477,10 @@ template <class P, int M>
 cudaError_t launch_m(const SweepLaunch& L, bool stats, bool bf16) {
   const size_t sm = sweep_multi_smem_bytes(L.smemJ, L.fam, stats);
   const int th = L.threads > 0 ? L.threads : kSweepThreads;
-  if (stats)
+  if (stats && L.inst0 != nullptr)
+    sweep_multi_kernel<P, true, M, true>
+        <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
+  else if (stats)
     sweep_multi_kernel<P, true, M, false>
         <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
   else if (L.inst0 != nullptr)

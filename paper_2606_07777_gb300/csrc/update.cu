@@ -1,8 +1,7 @@
 // update.cu -- the O(J) kernels that follow a sweep: the accelerated
 // projected dual step with gamma continuation, and the dual objective /
-// certified-gap statistics.  One CTA per instance; every reduction runs in a
-// fixed order (thread-strided, then a fixed shuffle tree, then warps in
-// order), so results are bit-identical from run to run.
+// certified-gap statistics.  Every reduction runs in a fixed order, so results
+// are bit-identical from run to run.
 #include <math.h>
 
 #include "dlm_impl.cuh"
@@ -30,20 +29,6 @@ __device__ double block_sum(double v, double* sh) {
   __syncthreads();
   return s;
 }
-__device__ double block_max(double v, double* sh) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_down_sync(kFull, v, o));
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  __syncthreads();
-  if (lane == 0) sh[w] = v;
-  __syncthreads();
-  double s = -INFINITY;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < static_cast<int>(blockDim.x >> 5); ++k) s = fmax(s, sh[k]);
-  __syncthreads();
-  return s;
-}
-
 // Accelerated projected step (Sec. 4.4; App. B.2), for iteration t at y:
 //   G_j    = (A x(y))_j - b_j
 //   lam+_j = max(0, y_j + step_j G_j),  step_j = gamma / max_k h_k  (1/L)
@@ -223,23 +208,30 @@ __global__ void __launch_bounds__(kUpdChunk) fista_update_kernel(const UpdInst* 
 // and every s_j is multiplied by t = min(1, M / sum x), which keeps the scaled
 // point within the count (sum_j s_j (sum_i x_ij) <= sum x).  With m capacity
 // families, s_j = min over the families of min(1, b_kj / (A_k x)_j).
-__global__ void __launch_bounds__(kUpdThreads) stats_kernel(const StatsInst* __restrict__ tab) {
-  __shared__ double sh[32];
-  const StatsInst S = tab[blockIdx.x];
-  const double gamma = *S.gamma;
-  double obj = 0.0;
-  if (S.obj_in) {
-    if (threadIdx.x == 0) obj = *S.obj_in;
-  } else {
-    for (int k = threadIdx.x; k < S.nseg; k += blockDim.x) obj += S.seg_obj[S.seg_list[k]];
-  }
+// Grid as the update's: 64 items per CTA, fixed-order partials, the last CTA
+// of the instance finishes.  (One CTA of 1,024 threads per instance: 28 us at
+// 1,000 items, most of it FP64 issue and serial sums.)
+__global__ void __launch_bounds__(kUpdChunk) stats_kernel(const StatsInst* __restrict__ tab,
+                                                          const __grid_constant__ StatsInst one) {
+  constexpr int kW = kUpdChunk / 32;
+  __shared__ StatsInst S;
+  __shared__ double sh[kUpdParts][kW];
+  __shared__ int s_last;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int k = tid; k < static_cast<int>(sizeof(StatsInst) / 8); k += kUpdChunk)
+    reinterpret_cast<uint64_t*>(&S)[k] =
+        tab ? __ldg(reinterpret_cast<const uint64_t*>(tab + blockIdx.y) + k) : reinterpret_cast<const uint64_t*>(&one)[k];
+  __syncthreads();
+  const int nct = (S.J + kUpdChunk - 1) / kUpdChunk;
+  if (static_cast<int>(blockIdx.x) >= nct) return;
+  const double gamma = S.gamma ? *S.gamma : S.gamma_val;
   // count constraint: sum x and the common scaling t = min(1, M / sum x)
   const double total = S.count_on ? to_real(*S.cnt, S.inv_sN) : 0.0;
   const double t = (S.count_on && total > S.count_M) ? S.count_M / total : 1.0;
-  __syncthreads();  // every thread has read the count sum before it is reset below
   double lg = 0.0, P = 0.0, viol = 0.0;
   const int m = S.m > 0 ? S.m : 1;
-  for (int j = threadIdx.x; j < S.J; j += blockDim.x) {
+  const int j = blockIdx.x * kUpdChunk + tid;
+  if (j < S.J) {
     double s = t;
     for (int f = 0; f < m; ++f) {
       const int q = f * S.J + j;
@@ -253,22 +245,71 @@ __global__ void __launch_bounds__(kUpdThreads) stats_kernel(const StatsInst* __r
     }
     const double Cx = to_real(S.accC[j], S.inv_sC);
     const double Qx = to_real(S.accQ[j], S.inv_sQ);
-    P += s * Cx + 0.5 * gamma * s * s * Qx;
+    P = s * Cx + 0.5 * gamma * s * s * Qx;
     S.accC[j] = 0ull;
     S.accQ[j] = 0ull;
   }
-  if (S.count_on && threadIdx.x == 0) {
-    const double G = total - S.count_M;
-    lg += static_cast<double>(S.lam[m * S.J]) * G;
-    viol = fmax(viol, G);
-    if (S.grad_out) S.grad_out[m * S.J] = static_cast<float>(G);
-    *S.cnt = 0ull;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lg += __shfl_down_sync(kFull, lg, o);
+    P += __shfl_down_sync(kFull, P, o);
+    viol = fmax(viol, __shfl_down_sync(kFull, viol, o));
   }
-  obj = block_sum(obj, sh);
-  lg = block_sum(lg, sh);
-  P = block_sum(P, sh);
-  viol = block_max(viol, sh);
-  if (threadIdx.x == 0) {
+  if (lane == 0) {
+    sh[0][warp] = lg;
+    sh[1][warp] = P;
+    sh[2][warp] = viol;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double p0 = sh[0][0], p1 = sh[1][0], p2 = sh[2][0];
+#pragma unroll
+    for (int w = 1; w < kW; ++w) {
+      p0 += sh[0][w];
+      p1 += sh[1][w];
+      p2 = fmax(p2, sh[2][w]);
+    }
+    S.part[kUpdParts * blockIdx.x] = p0;
+    S.part[kUpdParts * blockIdx.x + 1] = p1;
+    S.part[kUpdParts * blockIdx.x + 2] = p2;
+    __threadfence();
+    s_last = atomicAdd(S.ticket, 1u) == static_cast<unsigned>(nct) - 1u;
+    if (s_last) *S.ticket = 0u;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  // the last CTA: warp 0 adds the partials, warp 1 the objective's
+  double obj = 0.0;
+  lg = P = viol = 0.0;
+  if (warp == 0) {
+    for (int k = lane; k < nct; k += 32) {
+      lg += __ldcg(S.part + kUpdParts * k);
+      P += __ldcg(S.part + kUpdParts * k + 1);
+      viol = fmax(viol, __ldcg(S.part + kUpdParts * k + 2));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      lg += __shfl_down_sync(kFull, lg, o);
+      P += __shfl_down_sync(kFull, P, o);
+      viol = fmax(viol, __shfl_down_sync(kFull, viol, o));
+    }
+  } else if (!S.obj_in) {
+    for (int k = lane; k < S.nseg; k += 32) obj += S.seg_obj[S.seg_list[k]];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) obj += __shfl_down_sync(kFull, obj, o);
+    if (lane == 0) sh[0][0] = obj;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    obj = S.obj_in ? *S.obj_in : sh[0][0];
+    if (S.count_on) {
+      const double G = total - S.count_M;
+      lg += static_cast<double>(S.lam[m * S.J]) * G;
+      viol = fmax(viol, G);
+      if (S.grad_out) S.grad_out[m * S.J] = static_cast<float>(G);
+      *S.cnt = 0ull;
+    }
     const double g = obj + lg;
     const double den = fabs(g) > 1e-30 ? fabs(g) : 1e-30;
     S.out[0] = g;
@@ -279,6 +320,7 @@ __global__ void __launch_bounds__(kUpdThreads) stats_kernel(const StatsInst* __r
     S.out[5] = obj;
     S.out[6] = S.state ? static_cast<double>(S.state->iter) : 0.0;
     S.out[7] = S.state ? static_cast<double>(S.state->status) : 0.0;
+    S.out[8] = S.state ? S.state->gamma : gamma;
   }
 }
 
@@ -305,8 +347,9 @@ int update_parts(int64_t D) { return kUpdParts * update_ctas(D); }
 
 int update_ctas(int64_t D) { return static_cast<int>((D + kUpdChunk - 1) / kUpdChunk); }
 
-cudaError_t launch_stats(const StatsInst* dev_tab, int ninst, cudaStream_t s) {
-  stats_kernel<<<ninst, kUpdThreads, 0, s>>>(dev_tab);
+cudaError_t launch_stats(const StatsInst* dev_tab, const StatsInst* one, int ninst, int maxJ, cudaStream_t s) {
+  const dim3 grid(static_cast<unsigned>((maxJ + kUpdChunk - 1) / kUpdChunk), static_cast<unsigned>(ninst));
+  stats_kernel<<<grid, kUpdChunk, 0, s>>>(dev_tab, one ? *one : StatsInst{});
   return cudaGetLastError();
 }
 
