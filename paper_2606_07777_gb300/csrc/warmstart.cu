@@ -505,8 +505,8 @@ __global__ void k_to_bf16(const float* __restrict__ src, int64_t n, bf16* __rest
 // the chain of a tile -- load, five products, three epilogues -- and not any
 // throughput; the tiles are spread one per SM.  As separate launches (five
 // products through global memory with scalar staging, six elementwise kernels,
-// six reductions) loss and gradient took MLP_BEFORE us at 17,000 x 128; fused
-// MLP_NOW us.
+// six reductions) the loss and gradient of 17,000 rows and a prediction of
+// 1,000 took 525 us at width 128; fused they take 84 us, copies to the host included.
 //
 // Shared-memory operands are unswizzled 8 x 16-byte core matrices in columns
 // of 16-byte pieces: element (r, k) of a row buffer at
