@@ -137,6 +137,32 @@ __device__ __forceinline__ int lead_caller_pos(uint64_t lead, int k, int d) {
   return c;
 }
 
+// Programmatic dependent launch: the kernels of consecutive iterations are
+// launched with the attribute (launch_chained), so that the next kernel's blocks may
+// start, set up what needs no result, and wait in chain_wait() while the last
+// ones of the kernel before it finish.  Every block calls chain_wait() before it
+// reads what earlier kernels write and before it ends (a kernel that has ended
+// then implies that all before it have), and chain_go() after it, which lets the kernel after it start.
+// Without the attribute both do nothing.
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_go() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... KA, class... A>
+cudaError_t launch_chained(bool chain, void (*kernel)(KA...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                           const A&... args) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = chain ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
+}
+
 // f rounded to a 64-bit integer (ties to even), |f| < 2^55: the bits of
 // __float2ll_rn without the FP64 pipe it runs on (two lanes per clock and SM).
 // The part above 2^32 is read off the significand of a sum rounded
@@ -181,6 +207,7 @@ struct SweepLaunch {
   // Short-row sweep (iteration sweeps of a single one-family handle without a
   // count constraint, sweep_short.cu): slices 0 .. nslices0 - 1 of instance 0.
   bool short_rows = false;
+  bool chain = false;       // launched as one of a chain of iterations (launch_chained)
   int64_t nslices0 = 0;
 };
 constexpr int kDefaultCoopMax = 12;
@@ -234,7 +261,7 @@ cudaError_t sweep_short_prepare(bool bf16);
 cudaError_t launch_sweep_short(const SweepLaunch& L, bool bf16);
 // The update of ninst instances: a grid of max_cta x ninst CTAs (instance i
 // uses its first update_ctas(D_i)).
-cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, cudaStream_t s);
+cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, cudaStream_t s, bool chain = false);
 int update_ctas(int64_t D);
 int update_parts(int64_t D);  // doubles of UpdInst::part for D coordinates
 // The certificate's reductions: of ninst instances of the table, the largest of

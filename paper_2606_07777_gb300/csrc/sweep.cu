@@ -600,6 +600,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   const int nw = blockDim.x >> 5;
   const int t_last = cta_task[blockIdx.x + 1];
   int t = cta_task[blockIdx.x];
+  if (ONE)  // one segment: its sums are cleared ahead of the wait
+    for (int j = threadIdx.x; j < (STATS ? 3 : 1) * accN; j += blockDim.x) accG[j] = 0ull;
+  chain_wait();
+  chain_go();
   while (t < t_last) {
     const int inst = tasks[t].inst;
     int te = t + 1;
@@ -612,11 +616,13 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     // items with sums in this launch (STATS: the window, clipped to J)
     const int nacc = STATS ? max(0, min(J - jlo, jw)) : J;
     for (int j = threadIdx.x; j < J; j += blockDim.x) ys[j] = sD.y[j];
-    for (int j = threadIdx.x; j < nacc; j += blockDim.x) {
-      accG[j] = 0ull;
-      if (STATS) {
-        accC[j] = 0ull;
-        accQ[j] = 0ull;
+    if (!ONE) {
+      for (int j = threadIdx.x; j < nacc; j += blockDim.x) {
+        accG[j] = 0ull;
+        if (STATS) {
+          accC[j] = 0ull;
+          accQ[j] = 0ull;
+        }
       }
     }
     unsigned long long cn = 0ull, oq = 0ull;
@@ -720,6 +726,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   Seg S{};
   double wobj = 0.0;
   unsigned long long cn = 0ull, oq = 0ull;
+  chain_wait();
+  chain_go();
   for (;;) {
     if (threadIdx.x == 0) {
       s_unit = atomicAdd(ctr, 1u);
@@ -844,14 +852,13 @@ cudaError_t launch_width(const SweepLaunch& L, bool stats) {
   }
   const size_t sm = sweep_smem_bytes(L.smemJ, false);
   if (L.units != nullptr)
-    sweep_dyn_kernel<P, K><<<L.grid, th, sm, L.stream>>>(L.inst, L.units, L.nunits, L.ctr, L.smemJ, cm);
-  else if (L.inst0 != nullptr)
-    sweep_kernel<P, false, K, true>
-        <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, cm, 0, L.smemJ);
-  else
-    sweep_kernel<P, false, K, false>
-        <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, cm, 0, L.smemJ);
-  return cudaGetLastError();
+    return launch_chained(L.chain, &sweep_dyn_kernel<P, K>, L.grid, th, sm, L.stream, L.inst, L.units, L.nunits, L.ctr,
+                          L.smemJ, cm);
+  if (L.inst0 != nullptr)
+    return launch_chained(L.chain, &sweep_kernel<P, false, K, true>, L.grid, th, sm, L.stream, *L.inst0, L.inst, L.tasks,
+                          L.cta_task, L.smemJ, cm, 0, L.smemJ);
+  return launch_chained(L.chain, &sweep_kernel<P, false, K, false>, L.grid, th, sm, L.stream, InstDesc{}, L.inst, L.tasks,
+                        L.cta_task, L.smemJ, cm, 0, L.smemJ);
 }
 
 template <class P>

@@ -370,6 +370,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   const int nw = blockDim.x >> 5;
   const int t_last = cta_task[blockIdx.x + 1];
   int t = cta_task[blockIdx.x];
+  chain_wait();
+  chain_go();
   while (t < t_last) {
     const int inst = tasks[t].inst;
     int te = t + 1;
@@ -508,12 +510,10 @@ cudaError_t launch_values(const SweepLaunch& L, bool stats, const double* cuts) 
   }
   const size_t sm = sweep_smem_bytes(L.smemJ, false);
   if (L.inst0 != nullptr)
-    sweep_boxcut_kernel<V, false, true>
-        <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
-  else
-    sweep_boxcut_kernel<V, false, false>
-        <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
-  return cudaGetLastError();
+    return launch_chained(L.chain, &sweep_boxcut_kernel<V, false, true>, L.grid, th, sm, L.stream, *L.inst0, L.inst,
+                          L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
+  return launch_chained(L.chain, &sweep_boxcut_kernel<V, false, false>, L.grid, th, sm, L.stream, InstDesc{}, L.inst,
+                        L.tasks, L.cta_task, L.smemJ, 0, L.smemJ, cuts);
 }
 
 }  // namespace

@@ -353,6 +353,8 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   const int nw = blockDim.x >> 5;
   const int t_last = cta_task[blockIdx.x + 1];
   int t = cta_task[blockIdx.x];
+  chain_wait();
+  chain_go();
   while (t < t_last) {
     const int inst = tasks[t].inst;
     int te = t + 1;
@@ -484,11 +486,11 @@ cudaError_t launch_m(const SweepLaunch& L, bool stats, bool bf16) {
     sweep_multi_kernel<P, true, M, false>
         <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
   else if (L.inst0 != nullptr)
-    sweep_multi_kernel<P, false, M, true>
-        <<<L.grid, th, sm, L.stream>>>(*L.inst0, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
+    return launch_chained(L.chain, &sweep_multi_kernel<P, false, M, true>, L.grid, th, sm, L.stream, *L.inst0, L.inst,
+                          L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
   else
-    sweep_multi_kernel<P, false, M, false>
-        <<<L.grid, th, sm, L.stream>>>(InstDesc{}, L.inst, L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
+    return launch_chained(L.chain, &sweep_multi_kernel<P, false, M, false>, L.grid, th, sm, L.stream, InstDesc{}, L.inst,
+                          L.tasks, L.cta_task, L.smemJ, L.fam, bf16);
   return cudaGetLastError();
 }
 

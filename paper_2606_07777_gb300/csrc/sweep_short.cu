@@ -352,10 +352,10 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   const int J = D.J;
   unsigned long long* accG = reinterpret_cast<unsigned long long*>(smem_raw);
   float* ys = reinterpret_cast<float*>(accG + J);
-  for (int j = threadIdx.x; j < J; j += blockDim.x) {
-    ys[j] = D.y[j];
-    accG[j] = 0ull;
-  }
+  for (int j = threadIdx.x; j < J; j += blockDim.x) accG[j] = 0ull;
+  chain_wait();
+  chain_go();
+  for (int j = threadIdx.x; j < J; j += blockDim.x) ys[j] = D.y[j];
   if (threadIdx.x == 0) fill_seg(D, 0, J, sS);
   __syncthreads();
   Seg S = sS;
@@ -401,8 +401,7 @@ template <class V>
 cudaError_t launch_short_values(const SweepLaunch& L) {
   const int th = L.threads > 0 ? L.threads : kSweepThreads;
   const size_t sm = sweep_smem_bytes(L.smemJ, false);
-  sweep_short_kernel<Narrow<V>><<<L.grid, th, sm, L.stream>>>(*L.inst0, L.nslices0);
-  return cudaGetLastError();
+  return launch_chained(L.chain, &sweep_short_kernel<Narrow<V>>, L.grid, th, sm, L.stream, *L.inst0, L.nslices0);
 }
 
 }  // namespace

@@ -94,7 +94,11 @@ __global__ void __launch_bounds__(kUpdChunk) fista_update_kernel(const UpdInst* 
   __shared__ int s_last;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const UpdInst* __restrict__ I = tab + blockIdx.y;
-  if (static_cast<int>(blockIdx.x) >= I->nct) return;
+  if (static_cast<int>(blockIdx.x) >= I->nct) {
+    chain_wait();
+    return;
+  }
+  chain_go();  // (the sweep after it waits for this kernel's end)
   for (int k = tid; k < static_cast<int>(sizeof(UpdInst) / 8); k += kUpdChunk)
     reinterpret_cast<uint64_t*>(&U)[k] = __ldg(reinterpret_cast<const uint64_t*>(I) + k);
   __syncthreads();
@@ -114,6 +118,7 @@ __global__ void __launch_bounds__(kUpdChunk) fista_update_kernel(const UpdInst* 
   double step = c.step0;
   if (U.precondition) step = h > 0.0 ? c.st.gamma / h : 0.0;
   double lg = 0.0, dot = 0.0, bad = 0.0;
+  chain_wait();  // the sweep's sums; all read before it was written before the sweep began
   if (in) {
     const double G =
         j < NC ? to_real(U.acc[j], U.inv_scaleG) - bj : to_real(*U.cnt, U.inv_scaleN) - bj;
@@ -337,10 +342,9 @@ __global__ void __launch_bounds__(kUpdThreads) seg_sum_kernel(const StatsInst* _
 
 }  // namespace
 
-cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, cudaStream_t s) {
+cudaError_t launch_update(const UpdInst* dev_tab, int ninst, int max_cta, cudaStream_t s, bool chain) {
   const dim3 grid(static_cast<unsigned>(max_cta > 0 ? max_cta : 1), static_cast<unsigned>(ninst));
-  fista_update_kernel<<<grid, kUpdChunk, 0, s>>>(dev_tab);
-  return cudaGetLastError();
+  return launch_chained(chain, &fista_update_kernel, grid, kUpdChunk, 0, s, dev_tab);
 }
 
 int update_parts(int64_t D) { return kUpdParts * update_ctas(D); }
