@@ -7,11 +7,12 @@
 // which is continuous, nonincreasing and piecewise linear: on a piece the set
 // F of free edges (0 < u - tau < gamma z) and the set U of capped ones
 // (u - tau >= gamma z) are fixed and phi(tau) = (sum_F u - |F| tau) / gamma
-// + z |U| - cut.  Each lane brackets the root of its own row, tries the root
-// of the piece at the bracket's left end (a Newton step from the left), keeps
+// + z |U| - cut.  Nearly every row's piece is found from its four largest
+// values.  The others' root is bracketed, a row at a time by the whole warp: it
+// tries the root of the piece at the bracket's left end (a Newton step from the left), keeps
 // it when the sets at the trial point are those of the piece (then it is the
 // root), and otherwise narrows the bracket (bisecting when the trial point
-// falls outside).  Every trial is one pass over the row, re-read from L1/L2.
+// falls outside).
 // The final threshold is recomputed over F in float-pair arithmetic, as the
 // simplex sweep does, so x keeps FP32 relative accuracy at small gamma.
 //
@@ -58,6 +59,124 @@ __device__ __forceinline__ F2 budget_pair(const BSeg& S, int n) {
   return {d.h, d.l + (S.gcl - (pe + fn * S.gzl))};
 }
 
+// phi(t) * gamma = sum_F (u - t) + gamma (z |U| - cut)
+__device__ __forceinline__ float phi_g(const BSeg& S, float t, int nf, int nu, float sf) {
+  return (sf - static_cast<float>(nf) * t) + (static_cast<float>(nu) * S.gzh - S.gch);
+}
+
+// The bracketed search of row t of the slice, by the whole warp: lane l takes
+// edges l, l + 32, ..., every trial is a warp sum of the sets' counts and free
+// sum; then the pair-arithmetic refinement and the deposits.  The search
+// starts from the bracket [0, umax] and the sets at 0 (nf, nu, sf).  Few rows
+// need it (one in ten thousand to one in a hundred), and they are the widest:
+// with each lane over its own row, a trial was a chain of w / 4 loads from L2,
+// 40 us for 500 edges, and a dozen trials of one row held the whole sweep
+// (2M x 2,000 BF16: 255 -> 110 us an iteration alone).
+template <class V, bool STATS>
+__device__ __forceinline__ void search_row(const BSeg& S, const float* __restrict__ ys, unsigned long long* accG,
+                                        unsigned long long* accC, unsigned long long* accQ,
+                                        const uint16_t* __restrict__ col0, const typename V::T* __restrict__ ca0, int w,
+                                        int t, float umax, int nfl, int nul, float sfl, float& tau, float& taul,
+                                        float& ob) {
+  constexpr int KU = 4;  // of each lane's values kept in registers (rows of at most 32 KU edges read once)
+  const int lane = threadIdx.x & 31;
+  const int w4 = w >> 2;
+  auto value = [&](int k, int& j, float& c, float& a) {
+    const int el = sell_el(k, t, w4);
+    j = static_cast<int>(__ldg(col0 + el));
+    V::get(__ldg(ca0 + el), c, a);
+    return -fmaf(a, ys[j], c);
+  };
+  float uc[KU];
+#pragma unroll
+  for (int i = 0; i < KU; ++i) {
+    int j;
+    float c, a;
+    const int k = 32 * i + lane;
+    uc[i] = k < w ? value(k, j, c, a) : -INFINITY;
+  }
+  const float gz = S.gzh;
+  float lo = 0.f, hi = umax;
+  for (int it = 0; it < 96; ++it) {
+    bool newton = nfl > 0;
+    float cand = newton ? __fdiv_rn(sfl + (static_cast<float>(nul) * gz - S.gch), static_cast<float>(nfl)) : 0.f;
+    if (!(cand > lo && cand < hi)) {
+      cand = 0.5f * (lo + hi);
+      newton = false;
+    }
+    if (!(cand > lo && cand < hi)) break;  // the bracket is at float resolution
+    int nf = 0, nu = 0;
+    float sf = 0.f;
+    auto count = [&](float u) {
+      const float y = u - cand;
+      if (y >= gz) {
+        ++nu;
+      } else if (y > 0.f) {
+        ++nf;
+        sf += u;
+      }
+    };
+#pragma unroll
+    for (int i = 0; i < KU; ++i) count(uc[i]);
+    for (int k = 32 * KU + lane; k < w; k += 32) {
+      int j;
+      float c, a;
+      count(value(k, j, c, a));
+    }
+    nf = __reduce_add_sync(kFull, nf);
+    nu = __reduce_add_sync(kFull, nu);
+    sf = warp_sum(sf);
+    if (newton && nf == nfl && nu == nul) {  // same piece: cand is its root
+      lo = cand;
+      break;
+    }
+    if (phi_g(S, cand, nf, nu, sf) > 0.f) {
+      lo = cand;
+      nfl = nf;
+      nul = nu;
+      sfl = sf;
+    } else {
+      hi = cand;
+    }
+  }
+  // the threshold over the final free set in pair arithmetic
+  F2 ps{0.f, 0.f};
+  int n_f = 0, n_u = 0;
+  for (int k = lane; k < w; k += 32) {
+    int j;
+    float c, a;
+    const float d = value(k, j, c, a) - lo;
+    if (d >= gz) {
+      ++n_u;
+    } else if (d > 0.f) {
+      ++n_f;
+      ps = f2_add(ps, u_pair(c, a, ys[j]));
+    }
+  }
+  n_f = __reduce_add_sync(kFull, n_f);
+  n_u = __reduce_add_sync(kFull, n_u);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1)
+    ps = f2_add(ps, F2{__shfl_xor_sync(kFull, ps.h, o), __shfl_xor_sync(kFull, ps.l, o)});
+  tau = lo;  // (a flat piece: every x is 0 or z there)
+  taul = 0.f;
+  if (n_f > 0) {
+    const F2 b = budget_pair(S, n_u);
+    const F2 t2 = f2_threshold(ps, b.h, b.l, n_f);
+    tau = t2.h;
+    taul = t2.l;
+  }
+  for (int k = lane; k < w; k += 32) {
+    int j;
+    float c, a;
+    if (value(k, j, c, a) > tau) {
+      const F2 up = u_pair(c, a, ys[j]);
+      const float x = fminf(fmaxf(((up.h - tau) + (up.l - taul)) * S.invg, 0.f), S.z);
+      if (x > 0.f) deposit_b<V, STATS>(S, j, c, a, x, accG, accC, accQ, ob);
+    }
+  }
+}
+
 template <class V, bool STATS>
 __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, const float* __restrict__ ys,
                                              unsigned long long* accG, unsigned long long* accC,
@@ -70,7 +189,7 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
   const uint16_t* __restrict__ col0 = D.col16 + off;
   const typename V::T* __restrict__ ca0 = static_cast<const typename V::T*>(D.ca) + off;
   // the row in groups of four (one 64-bit index load, value loads as in the
-  // simplex sweep), then the tail: edges 0 .. w-1 in order
+  // simplex sweep), then the tail: edges 0 .. w-1 in order (rows that meet the budget)
   auto row_pass = [&](auto&& visit) {
     for (int g = 0; g < w4; ++g) {
       const int q = 32 * g + lane;
@@ -90,27 +209,6 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
     }
   };
   const float gz = S.gzh;
-  // sets at a trial threshold t: free count and sum, capped count
-  auto sets_at = [&](float t, int& nf, int& nu, float& sf) {
-    nf = 0;
-    nu = 0;
-    sf = 0.f;
-    row_pass([&](int j, float c, float a) {
-      const float u = -fmaf(a, ys[j], c);
-      const float y = u - t;
-      if (y >= gz) {
-        ++nu;
-      } else if (y > 0.f) {
-        ++nf;
-        sf += u;
-      }
-    });
-  };
-  // phi(t) * gamma = sum_F (u - t) + gamma (z |U| - cut)
-  auto phi_g = [&](float t, int nf, int nu, float sf) {
-    return (sf - static_cast<float>(nf) * t) + (static_cast<float>(nu) * gz - S.gch);
-  };
-
   // Pass A: the four largest u (v0 >= v1 >= v2 >= v3) and the sets at tau = 0.
   float v[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
   int nf = 0, nu = 0;
@@ -180,16 +278,13 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
   const float umax = v[0];
   float tau = 0.f, taul = 0.f;
   float ob = 0.f;
-  bool deposited = false;
+  bool deposited = false, search = false;
   if (umax > 0.f) {  // padding lanes and rows without a positive u deposit nothing
-    if (phi_g(0.f, nf, nu, sf) > 0.f) {
+    if (phi_g(S, 0.f, nf, nu, sf) > 0.f) {
       // The budget binds.  First try the pieces spanned by the four largest
       // values: a capped, f free (a + f <= 3), the rest at most v[a + f]; the
       // consistent one is the root's piece (phi is monotone).  A flat piece
       // (no free edge, a z = cut) has every point of it as a root.
-      float lo = 0.f, hi = umax;
-      int nfl = nf, nul = nu;
-      float sfl = sf;
       bool found = false;
       const float ka = rintf(S.cut / S.z);
       const bool flat_ok = fabsf(S.cut / S.z - ka) <= 1e-6f * fmaxf(ka, 1.f);
@@ -215,7 +310,7 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
           if (a > 0 && !(v[a - 1] - t >= gz)) continue;
           if (!(next <= t)) continue;
           found = true;
-          lo = t;
+          tau = t;
           if (a + f > 0) {
             // the nonzero edges are the a + f <= 3 largest, at the recorded
             // positions: load them once, refine the threshold over the free
@@ -256,58 +351,10 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
           }
         }
       }
-      for (int it = 0; it < 96 && !found; ++it) {
-        bool newton = nfl > 0;
-        float cand = newton ? __fdiv_rn(sfl + (static_cast<float>(nul) * gz - S.gch), static_cast<float>(nfl))
-                            : 0.f;
-        if (!(cand > lo && cand < hi)) {
-          cand = 0.5f * (lo + hi);
-          newton = false;
-        }
-        if (!(cand > lo && cand < hi)) break;  // the bracket is at float resolution
-        int nf2, nu2;
-        float sf2;
-        sets_at(cand, nf2, nu2, sf2);
-        if (newton && nf2 == nfl && nu2 == nul) {  // same piece: cand is its root
-          lo = cand;
-          break;
-        }
-        if (phi_g(cand, nf2, nu2, sf2) > 0.f) {
-          lo = cand;
-          nfl = nf2;
-          nul = nu2;
-          sfl = sf2;
-        } else {
-          hi = cand;
-        }
-      }
-      // the threshold over the final free set in pair arithmetic
-      F2 ps{0.f, 0.f};
-      int n_f = 0, n_u = 0;
-      if (!deposited) row_pass([&](int j, float c, float a) {
-        const float y = ys[j];
-        const float u = -fmaf(a, y, c);
-        const float d = u - lo;
-        if (d >= gz) {
-          ++n_u;
-        } else if (d > 0.f) {
-          ++n_f;
-          ps = f2_add(ps, u_pair(c, a, y));
-        }
-      });
-      if (deposited) {
-        // tau, taul set on the fast path
-      } else if (n_f > 0) {
-        const F2 b = budget_pair(S, n_u);
-        const F2 t2 = f2_threshold(ps, b.h, b.l, n_f);
-        tau = t2.h;
-        taul = t2.l;
-      } else {
-        tau = lo;  // a flat piece: every x is 0 or z there
-      }
+      search = !found;
     }
     // x = clip((u - tau) / gamma, 0, z) on the edges with u > tau
-    if (!deposited) row_pass([&](int j, float c, float a) {
+    if (!deposited && !search) row_pass([&](int j, float c, float a) {
       const float y = ys[j];
       if (-fmaf(a, y, c) > tau) {
         const F2 up = u_pair(c, a, y);
@@ -317,6 +364,23 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
     });
   } else {
     tau = INFINITY;
+  }
+  unsigned todo = __ballot_sync(kFull, search);
+  while (todo) {
+    const int t = __ffs(todo) - 1;
+    todo &= todo - 1;
+    float tt, tl, obt = 0.f;
+    search_row<V, STATS>(S, ys, accG, accC, accQ, col0, ca0, w, t, __shfl_sync(kFull, umax, t),
+                         __shfl_sync(kFull, nf, t), __shfl_sync(kFull, nu, t), __shfl_sync(kFull, sf, t), tt, tl, obt);
+    // (the lanes' parts of the row's objective go to fixed point each on its own)
+    if (STATS)
+      ob += obt;
+    else
+      oq += fixp(obt, S.scaleO);
+    if (lane == t) {
+      tau = tt;
+      taul = tl;
+    }
   }
   if (STATS) {
     const int64_t u = 32 * s + lane;
