@@ -433,12 +433,6 @@ __global__ void __launch_bounds__(32 * kGatherWarps)
   if (__any_sync(kFullMask, twice) && lane == 0) *dup = 1;
 }
 
-// f rounded to a 64-bit integer: fix64 where it holds, the conversion elsewhere
-// (items of small degree leave terms of up to 2^61).
-__device__ __forceinline__ unsigned long long fix_any(float f) {
-  return fabsf(f) < 36028797018963968.f ? fix64(f) : static_cast<unsigned long long>(__float2ll_rn(f));
-}
-
 // sum_i a_ij^2 (sums[0 .. J)) and sum_i a_ij (sums[J .. 2 J)) per item in
 // 64-bit fixed point (exact, order independent); SQ, S1: which of the two.
 // Blocks add in shared memory where it holds the sums (SMEM) and flush once per
@@ -458,9 +452,15 @@ __global__ void __launch_bounds__(1024) k_item_sums(const int32_t* __restrict__ 
     for (int64_t j = threadIdx.x; j < held; j += blockDim.x) sacc[j] = 0ull;
     __syncthreads();
   }
+  auto add = [](unsigned long long* p, unsigned long long v) {
+    if (SMEM)
+      shared_add64(p, v);
+    else
+      atomicAdd(p, v);
+  };
   auto take = [&](int32_t j, float av) {
-    if (SQ) atomicAdd(&sq[j], fix_any(av * av * scale_sq));
-    if (S1) atomicAdd(&s1[j], fix_any(av * scale_s1));
+    if (SQ) add(&sq[j], static_cast<unsigned long long>(__float2ll_rn(av * av * scale_sq)));
+    if (S1) add(&s1[j], static_cast<unsigned long long>(__float2ll_rn(av * scale_s1)));
   };
   const int64_t t = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
   const int64_t nt = static_cast<int64_t>(gridDim.x) * blockDim.x;

@@ -144,12 +144,12 @@ __device__ __forceinline__ void deposit(const Seg& S, int j, float c, float a, f
   if (STATS) {
     const unsigned jj = static_cast<unsigned>(j - S.jlo);
     if (jj < static_cast<unsigned>(S.jw)) {
-      atomicAdd(&accG[jj], fixp(a * x, S.scaleG));
-      atomicAdd(&accC[jj], fixp(c * x, S.scaleC));
-      atomicAdd(&accQ[jj], fixp(x * x, S.scaleQ));
+      shared_add64(&accG[jj], fixp(a * x, S.scaleG));
+      shared_add64(&accC[jj], fixp(c * x, S.scaleC));
+      shared_add64(&accQ[jj], fixp(x * x, S.scaleQ));
     }
   } else {
-    atomicAdd(&accG[j], fixp(a * x, S.scaleG));
+    shared_add64(&accG[j], fixp(a * x, S.scaleG));
   }
   ob += fmaf(0.5f * S.gamma * x, x, c * x);
 }

@@ -106,10 +106,10 @@ __device__ __forceinline__ void deposit_m(const MSeg& S, int j, float c, const f
                                           unsigned long long* accQ, float& ob) {
 #pragma unroll
   for (int f = 0; f < M; ++f)
-    if (fam_on<M>(S, f)) atomicAdd(&accG[f * S.J + j], fixp(a[f] * x, S.scaleG));
+    if (fam_on<M>(S, f)) shared_add64(&accG[f * S.J + j], fixp(a[f] * x, S.scaleG));
   if (STATS) {
-    atomicAdd(&accC[j], fixp(c * x, S.scaleC));
-    atomicAdd(&accQ[j], fixp(x * x, S.scaleQ));
+    shared_add64(&accC[j], fixp(c * x, S.scaleC));
+    shared_add64(&accQ[j], fixp(x * x, S.scaleQ));
   }
   ob += fmaf(0.5f * S.gamma * x, x, c * x);
 }

@@ -228,7 +228,7 @@ __device__ __forceinline__ void short_slice(const InstDesc& D, const Seg& S, con
         }
         if (x > 0.f) {
           // the item sum a x in 64-bit fixed point; the objective c x + gamma/2 x^2
-          atomicAdd(&accG[rg.j[e]], fixp(rg.a[e] * x, S.scaleG));
+          shared_add64(&accG[rg.j[e]], fixp(rg.a[e] * x, S.scaleG));
           ob = fmaf(fmaf(hg, x, rg.c[e]), x, ob);
         }
       }
