@@ -303,7 +303,7 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
 #pragma unroll
             for (int i = 0; i < 4; ++i)
               if (i >= a && i < a + f) sfree += v[i];
-            t = __fdiv_rn(sfree - (S.gch - static_cast<float>(a) * gz), static_cast<float>(f));
+            t = div_by(sfree - (S.gch - static_cast<float>(a) * gz), static_cast<float>(f), 1.f / static_cast<float>(f));
             if (!(v[a] - t < gz && v[a + f - 1] - t > 0.f)) continue;
           }
           if (!(t > 0.f) && f > 0) continue;
@@ -335,7 +335,7 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
               for (int i = 0; i < 3; ++i)
                 if (i >= a && i < a + f) ps = f2_add(ps, u_pair(cr[i], ar[i], ys[jr[i]]));
               const F2 b = budget_pair(S, a);
-              const F2 t2 = f2_threshold(ps, b.h, b.l, f);
+              const F2 t2 = f2_threshold_small<3>(ps, b.h, b.l, f);
               tau = t2.h;
               taul = t2.l;
             }
@@ -428,7 +428,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   __shared__ InstDesc s_inst;
   const InstDesc& sD = ONE ? one : s_inst;
   __shared__ BSeg sS;
-  __shared__ unsigned long long s_next;
+  __shared__ unsigned s_next;
   __shared__ unsigned long long s_red[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nw = blockDim.x >> 5;
@@ -500,9 +500,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
         // any order
         const int64_t nsl = (T.end - T.first + T.stride - 1) / T.stride;
         for (;;) {
-          int64_t i = 0;
-          if (lane == 0) i = static_cast<int64_t>(atomicAdd(&s_next, 1ull));
-          i = __shfl_sync(kFull, i, 0);
+          const int64_t i = next_ticket(&s_next);
           if (i >= nsl) break;
           boxcut_slice<V, STATS>(sD, S, ys, accG, accC, accQ, T.first + i * T.stride, wobj, oq);
         }

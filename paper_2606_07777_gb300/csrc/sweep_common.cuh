@@ -85,6 +85,32 @@ __device__ __forceinline__ F2 f2_threshold(F2 sum, float gzh, float gzl, int n) 
   return {th, __fdiv_rn(r + num.l, fn)};
 }
 
+// x / n for a small whole n, rounded to nearest, from n's rounded reciprocal
+// and one correction (Markstein 1990; the same bits as the division on every
+// significand for n = 1 .. 8): three instructions instead of the division's ten and its
+// slow-path call.
+__device__ __forceinline__ float div_by(float x, float n, float rcp) {
+  const float q = x * rcp;
+  return fmaf(fmaf(-q, n, x), rcp, q);
+}
+// The rounded reciprocal of n = 1 .. N.
+template <int N>
+__device__ __forceinline__ float small_rcp(int n) {
+  float r = 1.f;
+#pragma unroll
+  for (int q = 2; q <= N; ++q) r = n == q ? 1.f / static_cast<float>(q) : r;
+  return r;
+}
+// f2_threshold for n = 1 .. N.
+template <int N>
+__device__ __forceinline__ F2 f2_threshold_small(F2 sum, float gzh, float gzl, int n) {
+  const F2 num = f2_add(sum, F2{-gzh, -gzl});
+  const float fn = static_cast<float>(n), rcp = small_rcp<N>(n);
+  const float th = div_by(num.h, fn, rcp);
+  const float r = fmaf(-th, fn, num.h);
+  return {th, div_by(r + num.l, fn, rcp)};
+}
+
 // Item indices as uint16: the shared-memory item arrays bound a handle to
 // fewer than 65,536 items, so the layout keeps the index stream in 16 bits
 // (2 bytes per edge less to stream than int32).  A group of four edges of a
@@ -99,6 +125,14 @@ struct Narrow : V {
     j[2] = static_cast<int>(v.y & 0xffffu), j[3] = static_cast<int>(v.y >> 16);
   }
 };
+
+// The CTA's next ticket, the same in every lane of the warp (a 32-bit shared
+// addition; a task has fewer than 2^26 slices).
+__device__ __forceinline__ int next_ticket(unsigned* next) {
+  unsigned i = 0;
+  if ((threadIdx.x & 31) == 0) i = atomicAdd(next, 1u);
+  return static_cast<int>(__shfl_sync(kFull, i, 0));
+}
 
 struct Seg {
   float gamma, invg, gz, gzl, z;

@@ -215,15 +215,15 @@ __device__ __forceinline__ void multi_slice(const InstDesc& D, const MSeg& S, co
     if (v1 > tau) {
       sm += v1;
       r = 2;
-      tau = __fdiv_rn(sm - S.gz, 2.f);
+      tau = div_by(sm - S.gz, 2.f, 0.5f);
       if (v2 > tau) {
         sm += v2;
         r = 3;
-        tau = __fdiv_rn(sm - S.gz, 3.f);
+        tau = div_by(sm - S.gz, 3.f, 1.f / 3.f);
         if (v3 > tau) {
           sm += v3;
           r = 4;
-          tau = __fdiv_rn(sm - S.gz, 4.f);
+          tau = div_by(sm - S.gz, 4.f, 0.25f);
         }
       }
     }
@@ -231,18 +231,24 @@ __device__ __forceinline__ void multi_slice(const InstDesc& D, const MSeg& S, co
   }
   float ob = 0.f;
   bool zero = box;
-  if (mode == 1) {
-    load_edge<P, M>(D, S, off, i0, lane, w4, bf16, j, c, a);
-    deposit_m<STATS, M>(S, j, c, a, S.z, accG, accC, accQ, ob);
-  } else if (mode == 2) {
+  if (mode == 1 || mode == 2) {
+    // the recorded edges, loaded together; the maximum alone takes x = z (one
+    // path for both: nearly every warp has both kinds of row)
+    const bool single = mode == 1;
+    int jr[3];
+    float cr[3], ar[3][M];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      jr[i] = 0;
+      if (i < r) load_edge<P, M>(D, S, off, i == 0 ? i0 : (i == 1 ? i1 : i2), lane, w4, bf16, jr[i], cr[i], ar[i]);
+    }
     zero = !eq && tau <= 0.f;
-    if (!zero) {
+    if (!zero && !single) {
       F2 sum{0.f, 0.f};
-      for (int i = 0; i < r; ++i) {
-        load_edge<P, M>(D, S, off, i == 0 ? i0 : (i == 1 ? i1 : i2), lane, w4, bf16, j, c, a);
-        sum = f2_add(sum, u_pair_m<M>(S, ys, j, c, a));
-      }
-      const F2 t2 = f2_threshold(sum, S.gz, S.gzl, r);
+#pragma unroll
+      for (int i = 0; i < 3; ++i)
+        if (i < r) sum = f2_add(sum, u_pair_m<M>(S, ys, jr[i], cr[i], ar[i]));
+      const F2 t2 = f2_threshold_small<3>(sum, S.gz, S.gzl, r);
       if (!eq && t2.h + t2.l <= 0.f) {
         zero = true;
       } else {
@@ -251,10 +257,12 @@ __device__ __forceinline__ void multi_slice(const InstDesc& D, const MSeg& S, co
       }
     }
     if (zero) tau = taul = 0.f;
-    for (int i = 0; i < r; ++i) {
-      load_edge<P, M>(D, S, off, i == 0 ? i0 : (i == 1 ? i1 : i2), lane, w4, bf16, j, c, a);
-      const float x = x_of(S, false, tau, taul, u_pair_m<M>(S, ys, j, c, a));
-      if (x > 0.f) deposit_m<STATS, M>(S, j, c, a, x, accG, accC, accQ, ob);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      if (i < r) {
+        const float x = single ? S.z : x_of(S, false, tau, taul, u_pair_m<M>(S, ys, jr[i], cr[i], ar[i]));
+        if (x > 0.f) deposit_m<STATS, M>(S, jr[i], cr[i], ar[i], x, accG, accC, accQ, ob);
+      }
     }
   } else if (mode == 3) {
     if (!box) {
@@ -347,7 +355,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   __shared__ InstDesc s_inst;
   const InstDesc& sD = ONE ? one : s_inst;
   __shared__ MSeg sS;
-  __shared__ unsigned long long s_next;
+  __shared__ unsigned s_next;
   __shared__ unsigned long long s_red[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nw = blockDim.x >> 5;
@@ -415,9 +423,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
         __syncthreads();
         const int64_t nsl = (T.end - T.first + T.stride - 1) / T.stride;
         for (;;) {
-          int64_t i = 0;
-          if (lane == 0) i = static_cast<int64_t>(atomicAdd(&s_next, 1ull));
-          i = __shfl_sync(kFull, i, 0);
+          const int64_t i = next_ticket(&s_next);
           if (i >= nsl) break;
           multi_slice<P, STATS, M>(sD, S, ys, accG, accC, accQ, T.first + i * T.stride, bf16, wobj, oq);
         }
