@@ -115,7 +115,7 @@ def load_peaks():
     return 6800.0, "fallback"
 
 
-SWEEP_SOURCES = ("sweep.cu", "sweep_multi.cu", "sweep_common.cuh", "dlm_impl.cuh")
+SWEEP_SOURCES = ("sweep_kernels.cuh", "sweep_multi.cu", "sweep_common.cuh", "dlm_impl.cuh")
 
 
 def sweep_source_hash(files=SWEEP_SOURCES):

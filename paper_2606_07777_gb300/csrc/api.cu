@@ -155,6 +155,7 @@ struct dlm_problem {
   int device = 0;
   LayoutOut lay;
   std::vector<int64_t> h_slice_off;  // host copy of the slice offsets (task balancing)
+  int64_t nwide = 0;                 // slices swept in quarters (wide_slices)
   int sG = 0, sC = 0, sQ = 0;
   bool certified = true;
 
@@ -217,6 +218,31 @@ struct dlm_batch {
 
 namespace {
 
+// Slices (widest first) that the one-family sweep takes in quarters: those
+// whose warp would stream for more than a third of the whole sweep -- about
+// 80 ns an edge of the row's width, against the layout's bytes at 5 TB/s -- and
+// never rows under 64 edges.  FP32 only: a BF16 pass is half as long, and
+// quarters, whose warps finish eight rows at a time, gave 2 us of 22 on small
+// instances alone but took a 16-member batch from 1,405 to 1,560 us.  Not the
+// box, whose rows are summed in an order that depends on how many of the warp's
+// rows there are (it equals the box cut with a slack budget bit for bit).  A
+// rule on the instance alone, so every mapping and batch sweeps it alike.
+int64_t wide_slices(const dlm_problem* p) {
+  if (p->kind == DLM_BOX || p->bf16) return 0;
+  const double sweep_ns = static_cast<double>(p->lay.padded_nnz) * 10 / 5000.0;
+  const double edge_ns = 80.0;
+  const double w0 = std::max(64.0, sweep_ns / 3 / edge_ns);
+  int64_t a = 0, b = p->lay.nslices;  // the first slice narrower than w0
+  while (a < b) {
+    const int64_t m = (a + b) / 2;
+    if (static_cast<double>(p->h_slice_off[m + 1] - p->h_slice_off[m]) / 32 >= w0)
+      a = m + 1;
+    else
+      b = m;
+  }
+  return a;
+}
+
 InstDesc base_desc(const dlm_problem* p) {
   InstDesc d{};
   d.slice_off = p->lay.slice_off;
@@ -227,6 +253,7 @@ InstDesc base_desc(const dlm_problem* p) {
   d.udeg = p->lay.udeg;
   d.lead = p->lay.lead;
   d.nusers = p->lay.num_active_users;
+  d.nwide = p->nwide;
   d.status = &p->state->status;
   d.scaleG = std::ldexp(1.0f, p->sG);
   d.scaleC = std::ldexp(1.0f, p->sC);
@@ -562,6 +589,7 @@ SweepLaunch launch_of(const Runner& R, const InstDesc* tab) {
   for (const dlm_problem* p : R.probs) {
     L.count = L.count || p->count_on;
     L.fam = std::max(L.fam, p->m);
+    L.wide = L.wide || p->nwide > 0;
   }
   L.units = R.h_units.empty() ? nullptr : R.units;
   L.nunits = static_cast<int32_t>(R.h_units.size());
@@ -690,7 +718,7 @@ dlm_status runner_step_timed(Runner& R, int64_t n_iters, double* sweep_ms, doubl
 // launches that small CTAs allow: 302 -> 178 us).
 int default_threads(const Runner& R, int grid) {
   int64_t slices = 0;
-  for (const dlm_problem* p : R.probs) slices += p->lay.nslices;
+  for (const dlm_problem* p : R.probs) slices += p->lay.nslices + 3 * p->nwide;
   const int64_t want = std::max<int64_t>(32 * ((slices + grid - 1) / grid), (R.smemJ + 15) / 16);
   int t = 128;
   while (t < want && t < kSweepThreads) t *= 2;
@@ -1387,6 +1415,7 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
   cleanup_all();
   for (void*& q : tmp) q = nullptr;
 #undef CKC
+  p->nwide = wide_slices(p);
   // The handle's own runner: this one instance.
   Runner& R = p->run;
   R.probs = {p};

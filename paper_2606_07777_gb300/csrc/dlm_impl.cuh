@@ -82,6 +82,7 @@ struct InstDesc {
   const int32_t* udeg;      // [users with edges] degree of each sorted user
   const uint64_t* lead;     // [users with edges] caller positions of the row's lead edges (lead_caller_pos)
   int64_t nusers;           // users with edges (sorted users 0 .. nusers-1)
+  int64_t nwide;            // slices 0 .. nwide - 1 are swept in quarters (wide_slices in api.cu)
   int32_t* status;          // device error word (kStat* bits)
   const float* y;           // sweep point [J]
   const double* gamma;      // ridge used by this sweep (nullptr: gamma_val)
@@ -219,6 +220,7 @@ struct SweepLaunch {
   // Short-row sweep (iteration sweeps of a single one-family handle without a
   // count constraint, sweep_short.cu): slices 0 .. nslices0 - 1 of instance 0.
   bool short_rows = false;
+  bool wide = false;        // some instance has slices swept in quarters
   bool chain = false;       // launched as one of a chain of iterations (launch_chained)
   int64_t nslices0 = 0;
 };
