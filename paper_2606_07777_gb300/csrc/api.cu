@@ -7,6 +7,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -95,6 +96,58 @@ template <typename T>
 cudaError_t dalloc(T** p, size_t n) {
   return cudaMalloc(reinterpret_cast<void**>(p), sizeof(T) * (n > 0 ? n : 1));
 }
+// From the stream-ordered pool (freed with dev_free on the same stream): the
+// arrays of handles and runners, two dozen of them.  cudaMalloc and cudaFree
+// map and unmap memory and wait for the device, some 10 us each.
+template <typename T>
+cudaError_t dalloc(T** p, size_t n, cudaStream_t s) {
+  return dev_alloc(reinterpret_cast<void**>(p), sizeof(T) * (n > 0 ? n : 1), s);
+}
+
+// Pinned host blocks of kStatsOut doubles, kept for later handles (at most
+// kPinnedKept; dlm_release_cached_memory returns them).
+constexpr size_t kPinnedKept = 64;
+std::mutex g_pinned_mu;
+std::vector<double*> g_pinned;
+cudaError_t pinned_get(double** p) {
+  {
+    std::lock_guard<std::mutex> lk(g_pinned_mu);
+    if (!g_pinned.empty()) {
+      *p = g_pinned.back();
+      g_pinned.pop_back();
+      return cudaSuccess;
+    }
+  }
+  return cudaHostAlloc(reinterpret_cast<void**>(p), sizeof(double) * kStatsOut, cudaHostAllocPortable);
+}
+void pinned_put(double* p) {
+  if (!p) return;
+  {
+    std::lock_guard<std::mutex> lk(g_pinned_mu);
+    if (g_pinned.size() < kPinnedKept) {
+      g_pinned.push_back(p);
+      return;
+    }
+  }
+  cudaFreeHost(p);
+}
+void pinned_release() {
+  std::lock_guard<std::mutex> lk(g_pinned_mu);
+  for (double* p : g_pinned) cudaFreeHost(p);
+  g_pinned.clear();
+}
+
+// Pieces of one buffer: arrays placed one after another on 16-byte boundaries,
+// filled on the host and brought over in one copy.
+struct Packed {
+  std::vector<char> host;
+  size_t put(const void* src, size_t bytes) {
+    const size_t at = (host.size() + 15) & ~static_cast<size_t>(15);
+    host.resize(at + bytes);
+    if (src && bytes) std::memcpy(host.data() + at, src, bytes);
+    return at;
+  }
+};
 
 // Slice-to-CTA assignment orders.
 enum : int { kAssignInterleaved = 0, kAssignContiguous = 1, kAssignDynamic = 2 };
@@ -119,6 +172,8 @@ struct Runner {
   int topk = 4;  // one-family sweeps: values tracked per row in the first pass
   bool short_rows = false;   // iteration sweeps take the short-row sweep (sweep_short.cu)
   int upd_ctas = 1;      // update grid width (the largest member's)
+  void* tabs = nullptr;  // the instances' tables (inst_iter, inst_stats, upd, st_stats)
+  void* plan = nullptr;  // the tasks and their lists (tasks .. ctr)
   InstDesc *inst_iter = nullptr, *inst_stats = nullptr;
   InstDesc h_iter0{}, h_stats0{};  // host copies of inst_iter[0], inst_stats[0]
   StatsInst h_st0{};               // and of st_stats[0]
@@ -304,9 +359,10 @@ void invalidate_graph(Runner& R) {
 
 void runner_free(Runner& R) {
   invalidate_graph(R);
-  void* ptrs[] = {R.inst_iter, R.inst_stats, R.upd,   R.st_stats, R.tasks, R.cta_task,
-                  R.seg_lists, R.seg_obj,    R.units, R.ctr,      R.cuts};
-  for (void* q : ptrs) cudaFree(q);
+  dev_free(R.tabs, R.stream);
+  dev_free(R.plan, R.stream);
+  dev_free(R.cuts, R.stream);
+  R.tabs = R.plan = nullptr;
   for (cudaEvent_t e : R.events) cudaEventDestroy(e);
   R.events.clear();
   if (R.done) cudaEventDestroy(R.done);
@@ -501,12 +557,21 @@ dlm_status write_tables(Runner& R) {
   R.h_iter0 = it[0];
   R.h_stats0 = ss[0];
   R.h_st0 = st[0];
-  CK(cudaMemcpy(R.inst_iter, it.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(R.inst_stats, ss.data(), sizeof(InstDesc) * n, cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(R.upd, up.data(), sizeof(UpdInst) * n, cudaMemcpyHostToDevice));
   R.upd_ctas = 1;
   for (const UpdInst& u : up) R.upd_ctas = std::max(R.upd_ctas, u.nct);
-  CK(cudaMemcpy(R.st_stats, st.data(), sizeof(StatsInst) * n, cudaMemcpyHostToDevice));
+  Packed pk;
+  const size_t o_it = pk.put(it.data(), sizeof(InstDesc) * n), o_ss = pk.put(ss.data(), sizeof(InstDesc) * n),
+               o_up = pk.put(up.data(), sizeof(UpdInst) * n), o_st = pk.put(st.data(), sizeof(StatsInst) * n);
+  if (!R.tabs) {  // (n is fixed for a runner, and with it the size)
+    char* t = nullptr;
+    CK(dalloc(&t, pk.host.size(), R.stream));
+    R.tabs = t;
+    R.inst_iter = reinterpret_cast<InstDesc*>(t + o_it);
+    R.inst_stats = reinterpret_cast<InstDesc*>(t + o_ss);
+    R.upd = reinterpret_cast<UpdInst*>(t + o_up);
+    R.st_stats = reinterpret_cast<StatsInst*>(t + o_st);
+  }
+  CK(cudaMemcpyAsync(R.tabs, pk.host.data(), pk.host.size(), cudaMemcpyHostToDevice, R.stream));
   return DLM_OK;
 }
 
@@ -515,44 +580,35 @@ dlm_status runner_build(Runner& R) {
   CK(cudaStreamSynchronize(R.stream));
   invalidate_graph(R);
   const int n = static_cast<int>(R.probs.size());
-  if (!R.inst_iter) {
-    CK(dalloc(&R.inst_iter, n));
-    CK(dalloc(&R.inst_stats, n));
-    CK(dalloc(&R.upd, n));
-    CK(dalloc(&R.st_stats, n));
-  }
   if (R.probs[0]->kind == DLM_BOX_CUT && !R.cuts) {
     std::vector<double> h(n);
     for (int i = 0; i < n; ++i) h[i] = R.probs[i]->cut;
-    CK(dalloc(&R.cuts, n));
-    CK(cudaMemcpy(R.cuts, h.data(), sizeof(double) * n, cudaMemcpyHostToDevice));
+    CK(dalloc(&R.cuts, n, R.stream));
+    CK(cudaMemcpyAsync(R.cuts, h.data(), sizeof(double) * n, cudaMemcpyHostToDevice, R.stream));
   }
   build_task_list(R);
-  cudaFree(R.tasks);
-  cudaFree(R.cta_task);
-  cudaFree(R.seg_lists);
-  cudaFree(R.seg_obj);
-  R.tasks = nullptr;
-  R.cta_task = R.seg_lists = nullptr;
-  R.seg_obj = nullptr;
-  CK(dalloc(&R.tasks, R.h_tasks.size()));
-  CK(dalloc(&R.cta_task, R.h_cta.size()));
-  CK(dalloc(&R.seg_lists, R.h_tasks.size()));
-  CK(dalloc(&R.seg_obj, R.h_tasks.size()));
-  if (!R.h_tasks.empty())
-    CK(cudaMemcpy(R.tasks, R.h_tasks.data(), sizeof(Task) * R.h_tasks.size(), cudaMemcpyHostToDevice));
-  CK(cudaMemcpy(R.cta_task, R.h_cta.data(), sizeof(int32_t) * R.h_cta.size(), cudaMemcpyHostToDevice));
   std::vector<int32_t> flat;
   for (const auto& v : R.h_seg) flat.insert(flat.end(), v.begin(), v.end());
-  if (!flat.empty()) CK(cudaMemcpy(R.seg_lists, flat.data(), sizeof(int32_t) * flat.size(), cudaMemcpyHostToDevice));
-  cudaFree(R.units);
-  R.units = nullptr;
-  if (!R.h_units.empty()) {
-    CK(dalloc(&R.units, R.h_units.size()));
-    CK(cudaMemcpy(R.units, R.h_units.data(), sizeof(Task) * R.h_units.size(), cudaMemcpyHostToDevice));
-  }
-  if (!R.ctr) CK(dalloc(&R.ctr, 2));
-  CK(cudaMemset(R.ctr, 0, 2 * sizeof(unsigned)));
+  const unsigned zero[2] = {0u, 0u};
+  Packed pk;
+  const size_t o_t = pk.put(R.h_tasks.data(), sizeof(Task) * R.h_tasks.size()),
+               o_c = pk.put(R.h_cta.data(), sizeof(int32_t) * R.h_cta.size()),
+               o_l = pk.put(flat.data(), sizeof(int32_t) * flat.size()),
+               o_u = pk.put(R.h_units.data(), sizeof(Task) * R.h_units.size()),
+               o_z = pk.put(zero, sizeof(zero)),
+               o_s = pk.put(nullptr, sizeof(double) * R.h_tasks.size());
+  dev_free(R.plan, R.stream);
+  R.plan = nullptr;
+  char* t = nullptr;
+  CK(dalloc(&t, pk.host.size(), R.stream));
+  R.plan = t;
+  R.tasks = reinterpret_cast<Task*>(t + o_t);
+  R.cta_task = reinterpret_cast<int32_t*>(t + o_c);
+  R.seg_lists = reinterpret_cast<int32_t*>(t + o_l);
+  R.units = reinterpret_cast<Task*>(t + o_u);
+  R.ctr = reinterpret_cast<unsigned*>(t + o_z);
+  R.seg_obj = reinterpret_cast<double*>(t + o_s);
+  CK(cudaMemcpyAsync(t, pk.host.data(), pk.host.size(), cudaMemcpyHostToDevice, R.stream));
   return write_tables(R);
 }
 
@@ -780,19 +836,14 @@ void free_problem(dlm_problem* p) {
   if (p->stream) cudaStreamSynchronize(p->stream);
   runner_free(p->run);
   cudaStream_t s = p->stream;
-  void* pooled[] = {p->lay.slice_off, p->lay.slice_w, p->lay.col16, p->lay.ca, p->lay.orig_off,
-                    p->lay.udeg,      p->lay.lead,    p->a_ext};
+  void* pooled[] = {p->lay.slice_off, p->lay.slice_w, p->lay.col16, p->lay.ca,    p->lay.orig_off, p->lay.udeg,
+                    p->lay.lead,      p->a_ext,       p->b,         p->curv,      p->lam,          p->y,
+                    p->gamma_tab,     p->stats_out,   p->state,     p->lam64,     p->y64,          p->traj,
+                    p->upd_part,      p->upd_ticket,  p->own_sums ? p->xsum : nullptr,
+                    p->own_sums ? p->csum : nullptr};
   for (void* q : pooled) dev_free(q, s);
   if (s) cudaStreamSynchronize(s);
-  if (p->own_sums) {
-    cudaFree(p->xsum);
-    cudaFree(p->csum);
-  }
-  void* ptrs[] = {p->b,         p->curv,      p->lam,      p->y,      p->gamma_tab, p->stats_out,
-                  p->state,     p->lam64,  p->y64,       p->traj,       p->upd_part,
-                  p->upd_ticket};
-  for (void* q : ptrs) cudaFree(q);
-  cudaFreeHost(p->h_out);
+  pinned_put(p->h_out);
   if (p->ev) cudaEventDestroy(p->ev);
   if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
   delete p;
@@ -859,13 +910,15 @@ dlm_status upload_schedule(dlm_problem* p) {
     const double n = tab.back() * p->factor;
     tab.push_back(n > p->gamma_end ? n : p->gamma_end);
   }
-  CK(cudaStreamSynchronize(p->stream));
   if (static_cast<int64_t>(tab.size()) > p->gamma_tab_cap) {
-    cudaFree(p->gamma_tab);
+    // (a batch on another stream may still read the old table)
+    CK(cudaStreamSynchronize(p->stream));
+    dev_free(p->gamma_tab, p->stream);
     p->gamma_tab = nullptr;
     p->gamma_tab_cap = 0;
-    CK(dalloc(&p->gamma_tab, tab.size()));
-    p->gamma_tab_cap = static_cast<int64_t>(tab.size());
+    const size_t cap = std::max<size_t>(tab.size(), 64);
+    CK(dalloc(&p->gamma_tab, cap, p->stream));
+    p->gamma_tab_cap = static_cast<int64_t>(cap);
   }
   p->h_gamma_tab = tab;
   p->nstages = static_cast<int64_t>(tab.size());
@@ -877,7 +930,6 @@ dlm_status upload_schedule(dlm_problem* p) {
   k_momentum_reset<<<blocks_for(p->D()), 256, 0, p->stream>>>(p->lam64, p->y64, p->lam, p->y, p->D(), p->state);
   CK(cudaGetLastError());
   CK(cudaMemsetAsync(p->objq, 0, sizeof(unsigned long long), p->stream));
-  CK(cudaStreamSynchronize(p->stream));
   p->traj_from = 0;
   invalidate_graph(p->run);
   return write_tables(p->run);
@@ -1368,16 +1420,16 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
     cudaFree(gacc);
     CKC(sweep_multi_prepare(p->bf16));
   }
-  CKC(dalloc(&p->b, MJ));
+  CKC(dalloc(&p->b, MJ, p->stream));
   CKC(cudaMemcpyAsync(p->b, b, sizeof(double) * MJ, cudaMemcpyDeviceToDevice, p->stream));
-  CKC(dalloc(&p->curv, MJ + 1));
-  CKC(dalloc(&p->lam, MJ + 1));
-  CKC(dalloc(&p->y, MJ + 1));
-  CKC(dalloc(&p->lam64, MJ + 1));
-  CKC(dalloc(&p->y64, MJ + 1));
-  CKC(dalloc(&p->traj, kTrajCap));
-  CKC(dalloc(&p->upd_part, static_cast<size_t>(update_parts(MJ + 1))));
-  CKC(dalloc(&p->upd_ticket, 1));
+  CKC(dalloc(&p->curv, MJ + 1, p->stream));
+  CKC(dalloc(&p->lam, MJ + 1, p->stream));
+  CKC(dalloc(&p->y, MJ + 1, p->stream));
+  CKC(dalloc(&p->lam64, MJ + 1, p->stream));
+  CKC(dalloc(&p->y64, MJ + 1, p->stream));
+  CKC(dalloc(&p->traj, kTrajCap, p->stream));
+  CKC(dalloc(&p->upd_part, static_cast<size_t>(update_parts(MJ + 1)), p->stream));
+  CKC(dalloc(&p->upd_ticket, 1, p->stream));
   CKC(cudaMemsetAsync(p->upd_ticket, 0, sizeof(unsigned), p->stream));
   CKC(cudaMemsetAsync(p->lam64, 0, sizeof(double) * (MJ + 1), p->stream));
   CKC(cudaMemsetAsync(p->y64, 0, sizeof(double) * (MJ + 1), p->stream));
@@ -1388,8 +1440,8 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
     p->cobj = shard->cert_obj;
     p->own_sums = false;
   } else {
-    CKC(dalloc(&p->xsum, MJ + 2));
-    CKC(dalloc(&p->csum, MJ + 2 * J + 1));
+    CKC(dalloc(&p->xsum, MJ + 2, p->stream));
+    CKC(dalloc(&p->csum, MJ + 2 * J + 1, p->stream));
   }
   CKC(cudaMemsetAsync(p->xsum, 0, sizeof(unsigned long long) * (MJ + 2), p->stream));
   CKC(cudaMemsetAsync(p->csum, 0, sizeof(unsigned long long) * (MJ + 2 * J + 1), p->stream));
@@ -1402,9 +1454,9 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
   p->cnt2 = p->csum + MJ + 2 * J;
   CKC(cudaMemsetAsync(p->lam, 0, sizeof(float) * (MJ + 1), p->stream));
   CKC(cudaMemsetAsync(p->y, 0, sizeof(float) * (MJ + 1), p->stream));
-  CKC(dalloc(&p->stats_out, kStatsOut));
-  CKC(dalloc(&p->state, 1));
-  CKC(cudaMallocHost(reinterpret_cast<void**>(&p->h_out), sizeof(double) * kStatsOut));
+  CKC(dalloc(&p->stats_out, kStatsOut, p->stream));
+  CKC(dalloc(&p->state, 1, p->stream));
+  CKC(pinned_get(&p->h_out));
   CKC(sweep_prepare(p->bf16));
   if (p->kind == DLM_BOX_CUT) CKC(sweep_boxcut_prepare(p->bf16));
   CKC(cudaEventCreateWithFlags(&p->ev, cudaEventDisableTiming));
@@ -1808,6 +1860,7 @@ dlm_status dlm_shard_cert_finish(dlm_problem* p, dlm_stats* out) {
 }
 
 dlm_status dlm_release_cached_memory(void) {
+  pinned_release();
   const cudaError_t e = release_cached_memory();
   if (e != cudaSuccess) return fail(DLM_ERR_CUDA, std::string("memory pool trim: ") + cudaGetErrorString(e));
   return DLM_OK;
