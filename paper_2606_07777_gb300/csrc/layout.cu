@@ -31,6 +31,7 @@
 #include <cstdint>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include "dlm_impl.cuh"
@@ -268,34 +269,313 @@ __device__ __forceinline__ unsigned cost_key(float c) {
   return (u & 0x80000000u) ? ~u : u | 0x80000000u;
 }
 
+// Four edges of a lane written at 16-byte pieces (q: quadruple).
+__device__ __forceinline__ void put4(uint32_t* o, int64_t q, const uint32_t (&v)[4]) {
+  reinterpret_cast<uint4*>(o)[q] = make_uint4(v[0], v[1], v[2], v[3]);
+}
+__device__ __forceinline__ void put4(float2* o, int64_t q, const float2 (&v)[4]) {
+  reinterpret_cast<float4*>(o)[2 * q] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+  reinterpret_cast<float4*>(o)[2 * q + 1] = make_float4(v[2].x, v[2].y, v[3].x, v[3].y);
+}
+
+// A lane's four lowest edges by cost, of equal costs the earlier one: the
+// cost's key above the position, so that an insertion is minima and maxima --
+// 32 bits a key for BF16 costs and positions of up to 16 bits, 64 for FP32.
+template <typename CA>
+using LeadKey = typename std::conditional<sizeof(CA) == 4, unsigned, unsigned long long>::type;
+__device__ __forceinline__ unsigned lead_key(uint32_t v, int k) {
+  return (cost_key(__uint_as_float(v << 16)) & 0xffff0000u) | static_cast<unsigned>(k);
+}
+__device__ __forceinline__ unsigned long long lead_key(float2 v, int k) {
+  return static_cast<unsigned long long>(cost_key(v.x)) << 32 | static_cast<unsigned>(k);
+}
+template <typename K>
+__device__ __forceinline__ void lowest4(K x, K (&lk)[4]) {
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const K lo = min(x, lk[q]);
+    x = max(x, lk[q]);
+    lk[q] = lo;
+  }
+}
+// Adds the record of the lane o away.
+template <typename K>
+__device__ __forceinline__ void lowest4_merge(int o, K (&lk)[4]) {
+  K x[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) x[q] = __shfl_xor_sync(kFullMask, lk[q], o);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) lowest4(x[q], lk);
+}
+// The record as lead edges (0xFFFF past the row's d edges).
+template <typename K>
+__device__ __forceinline__ uint64_t lead_of(const K (&lk)[4], int d) {
+  uint64_t ld = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) ld |= static_cast<uint64_t>(q < d ? static_cast<unsigned>(lk[q]) & 0xFFFFu : 0xFFFFu) << (16 * q);
+  return ld;
+}
+
 // The slices' edge streams, rows in lead order (dlm_impl.cuh: the four
 // lowest-cost edges first, of equal costs the earlier one).
 //
-// A warp takes a slice and reads each of its rows with consecutive lanes (the
-// caller's rows are contiguous), where a lane per row read every sector eight
-// times over: first for the lead edges (warp minima of the costs' keys), then
-// 32 slice positions of every row at a time, put into the slice's order in shared
-// memory -- groups of four edges 4 elements further apart than in the slice,
-// so that a row's groups fall into different banks -- and written out in whole
-// 128-bit pieces.  Slices are dealt by a counter, widest first.  The row's
-// items are at hand, so the check that none repeats is taken here too (rows of
-// at most 32 edges by __match_any_sync, longer ones by marking a bitmap of the
-// items in shared memory).  50M BF16 edges (2M rows): 1,015 us with a lane per
-// row and 480 us for the check in a pass of its own; with the item sums, a new
-// handle of that size and ten iterations went from 4,346 to 3,274 us.
+// A warp takes a slice.  Rows of up to kRawWidth edges (gather_raw) are read
+// once, with consecutive lanes (the caller's rows are contiguous, where a lane per row
+// read every sector eight times over), as many rows at a time as fill 32 reads of
+// the warp, eight of which are in flight together; they stay in shared memory
+// in the caller's order while the lead edges are picked (warp minima of the costs'
+// keys), the items checked (no item twice: a bitmap of the items in shared
+// memory), and the slice's elements written, four positions of a row per
+// lane.  Longer rows (gather_strips) are read for the lead edges, for the check and then
+// once more, 32 slice positions of every row at a time, put into the slice's
+// order in shared memory -- groups of four edges 4 elements further apart than
+// in the slice, so that a row's groups fall into different banks -- and
+// written out in whole 128-bit pieces.  Slices are dealt by a counter, widest first.
+// 50M BF16 edges (2M rows of 25 on average, the longest 500): 939 us with every
+// row read twice and the longest rows' chains of loads at the end, now 439 us.
 // Every item is in [0, J) here (checked before).
 constexpr int kGatherWarps = 8;
-constexpr int kStripGroups = 8;                             // groups of four edges of a strip
-constexpr int kStripElems = kStripGroups * 132 + 3 * 32;    // staged elements: the groups, then the slice's tail
+constexpr int kStripGroups = 8;                           // groups of four edges of a strip
+constexpr int kStripElems = kStripGroups * 132 + 3 * 32;  // staged elements: the groups, then the slice's tail
+constexpr int kRawWidth = 1024;                           // longest rows of gather_raw
+constexpr int kRawElems = 32 * 33;                        // its staged elements, at most: R rows of 32 nc + 1
+static_assert(kRawElems <= kStripElems, "one buffer");
+
+// What a warp works on: its slice, lane t's row of it, its shared memory.
 template <typename CA>
-__global__ void __launch_bounds__(32 * kGatherWarps)
+struct GatherWarp {
+  const int32_t* __restrict__ col;
+  const void* __restrict__ c;
+  const void* __restrict__ a;
+  uint16_t* __restrict__ col_o;  // the slice's elements
+  CA* __restrict__ ca_o;
+  CA* sca;
+  uint16_t* scol;
+  unsigned* seen;
+  int64_t r;  // first edge and degree of the lane's row
+  int d, w, J;
+};
+
+// A row's lead edges in ascending order of position (0x7fff after the last),
+// 16 bits each: with it a slice position past them is found by four comparisons.
+__device__ __forceinline__ uint64_t lead_sorted(uint64_t lead, int d) {
+  unsigned p[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) p[i] = i < d ? static_cast<unsigned>(lead >> (16 * i)) & 0xffffu : 0x7fffu;
+  auto order = [&](int i, int j) {
+    const unsigned lo = min(p[i], p[j]), hi = max(p[i], p[j]);
+    p[i] = lo;
+    p[j] = hi;
+  };
+  order(0, 1), order(2, 3), order(0, 2), order(1, 3), order(1, 2);
+  return p[0] | static_cast<uint64_t>(p[1]) << 16 | static_cast<uint64_t>(p[2]) << 32 | static_cast<uint64_t>(p[3]) << 48;
+}
+
+// Slices of rows of up to kRawWidth edges.  Returns the lane's row's lead edges.
+template <typename CA>
+__device__ __forceinline__ uint64_t gather_raw(const GatherWarp<CA>& W, bool& twice) {
+  const int lane = threadIdx.x & 31;
+  const int w4 = W.w >> 2;
+  const int nc = (W.w + 31) >> 5;  // reads of a row
+  const int lg = nc > 1 ? 32 - __clz(nc - 1) : 0;
+  const int R = 32 >> lg;  // rows at a time: R nc <= 32
+  const int rs = 32 * nc + 1;
+  using K = LeadKey<CA>;
+  uint64_t lead = 0;
+  for (int t0 = 0; t0 < 32; t0 += R) {
+    // the rows as they are
+    int row = 0, ch = 0;
+    for (int x = 0; x < R * nc; x += 8) {
+      int j[8], at[8];
+      CA v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int64_t rt = __shfl_sync(kFullMask, W.r, (t0 + row) & 31);
+        const int dt = __shfl_sync(kFullMask, W.d, (t0 + row) & 31);
+        const int k = 32 * ch + lane;
+        at[i] = -1;
+        if (row < R && k < dt) {
+          at[i] = row * rs + k;
+          j[i] = __ldg(W.col + rt + k);
+          v[i] = pack_ca<CA>(W.c, W.a, rt + k);
+        }
+        if (++ch == nc) ch = 0, ++row;
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (at[i] >= 0) {
+          W.scol[at[i]] = static_cast<uint16_t>(j[i]);
+          W.sca[at[i]] = v[i];
+        }
+    }
+    __syncwarp();
+    // no item repeats: the row's items set their bits, and clear them again
+    if (nc == 1) {
+#pragma unroll 4
+      for (int t = 0; t < 32; ++t) {
+        const bool on = lane < __shfl_sync(kFullMask, W.d, t);
+        const int j = on ? W.scol[t * rs + lane] : 0;
+        const unsigned bit = on ? 1u << (j & 31) : 0u;
+        if (on && (atomicOr(&W.seen[j >> 5], bit) & bit)) twice = true;
+        __syncwarp();
+        if (on) W.seen[j >> 5] = 0u;
+        __syncwarp();
+      }
+    } else {
+      for (int t = 0; t < R; ++t) {
+        const int dt = __shfl_sync(kFullMask, W.d, t0 + t);
+        for (int k = lane; k < dt; k += 32) {
+          const int j = W.scol[t * rs + k];
+          const unsigned bit = 1u << (j & 31);
+          if (atomicOr(&W.seen[j >> 5], bit) & bit) twice = true;
+        }
+        __syncwarp();
+        for (int k = lane; k < dt; k += 32) W.seen[W.scol[t * rs + k] >> 5] = 0u;
+        __syncwarp();
+      }
+    }
+    // 1 << lg lanes a row, R apart: its lead edges (every one of them holds the record at the end)
+    const int t = lane & (R - 1), part = lane >> (5 - lg);
+    const int dt = __shfl_sync(kFullMask, W.d, t0 + t);
+    K lk[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) lk[q] = ~K{0};
+#pragma unroll 2
+    for (int k = part; k < dt; k += 1 << lg) lowest4<K>(lead_key(W.sca[t * rs + k], k), lk);
+    __syncwarp();
+    for (int o = R; o < 32; o <<= 1) lowest4_merge<K>(o, lk);
+    const uint64_t lt = lead_of<K>(lk, dt);
+    {
+      const uint64_t mine = __shfl_sync(kFullMask, lt, lane & (R - 1));
+      if (lane >= t0 && lane < t0 + R) lead = mine;
+    }
+    // the rows' slice elements: a lane writes a group of four positions of a row
+    const uint64_t ls = lead_sorted(lt, dt);
+    const unsigned p0 = ls & 0xffffu, p1 = (ls >> 16) & 0xffffu, p2 = (ls >> 32) & 0xffffu, p3 = ls >> 48;
+    auto edge = [&](int k, CA& v, unsigned& j) {
+      v = pad_ca<CA>();
+      j = 0u;
+      if (k < dt) {
+        unsigned e;
+        if (k < 4) {
+          e = static_cast<unsigned>(lt >> (16 * k)) & 0xffffu;
+        } else {
+          e = static_cast<unsigned>(k - 4);
+          e += e >= p0;
+          e += e >= p1;
+          e += e >= p2;
+          e += e >= p3;
+        }
+        v = W.sca[t * rs + e];
+        j = W.scol[t * rs + e];
+      }
+    };
+    for (int g = part; g < w4; g += 1 << lg) {
+      CA v[4];
+      unsigned j[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) edge(4 * g + e, v[e], j[e]);
+      const int64_t q = 32 * static_cast<int64_t>(g) + t0 + t;
+      reinterpret_cast<uint2*>(W.col_o)[q] = make_uint2(j[0] | j[1] << 16, j[2] | j[3] << 16);
+      put4(W.ca_o, q, v);
+    }
+    for (int k = 4 * w4 + part; k < W.w; k += 1 << lg) {  // the tail
+      CA v;
+      unsigned j;
+      edge(k, v, j);
+      const int64_t q = 128 * static_cast<int64_t>(w4) + 32 * (k - 4 * w4) + t0 + t;
+      W.col_o[q] = static_cast<uint16_t>(j);
+      W.ca_o[q] = v;
+    }
+    __syncwarp();
+  }
+  return lead;
+}
+
+// Slices of longer rows.
+template <typename CA>
+__device__ __noinline__ uint64_t gather_strips(const GatherWarp<CA>& W, bool& twice) {
+  using K = LeadKey<CA>;
+  constexpr bool kBf = sizeof(CA) == 4;
+  const int lane = threadIdx.x & 31;
+  const int w4 = W.w >> 2;
+  uint64_t lead = 0;
+  for (int t = 0; t < 32; ++t) {
+    const int64_t rt = __shfl_sync(kFullMask, W.r, t);
+    const int dt = __shfl_sync(kFullMask, W.d, t);
+    K lk[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) lk[q] = ~K{0};
+    const int de = dt < 0xFFFF ? dt : 0xFFFF;  // (positions fit 16 bits)
+#pragma unroll 4
+    for (int k = lane; k < de; k += 32) lowest4<K>(lead_key(pack_ca<CA>(W.c, W.a, rt + k), k), lk);
+    __syncwarp();
+    for (int o = 1; o < 32; o <<= 1) lowest4_merge<K>(o, lk);
+    const uint64_t ld = lead_of<K>(lk, dt);
+    if (lane == t) lead = ld;
+    twice = twice || dt > W.J;  // more edges than items: some item repeats
+    if (dt > W.J) continue;     // (warp-uniform)
+    for (int k = lane; k < dt; k += 32) {
+      const int j = __ldg(W.col + rt + k);
+      const unsigned bit = 1u << (j & 31);
+      if (atomicOr(&W.seen[j >> 5], bit) & bit) twice = true;
+    }
+    __syncwarp();
+    for (int k = lane; k < dt; k += 32) W.seen[__ldg(W.col + rt + k) >> 5] = 0u;
+    __syncwarp();
+  }
+  // positions 32 st .. of every row, then the strip's elements in order
+  for (int st = 0; 32 * st < W.w; ++st) {
+    const int k = 32 * st + lane;
+    const int at = k < 4 * w4 ? (lane >> 2) * 132 + (lane & 3) : kStripGroups * 132 + 32 * (k - 4 * w4);
+    const int by = k < 4 * w4 ? 4 : 1;
+#pragma unroll 4
+    for (int t = 0; t < 32; ++t) {
+      const int64_t rt = __shfl_sync(kFullMask, W.r, t);
+      const int dt = __shfl_sync(kFullMask, W.d, t);
+      const uint64_t lt = __shfl_sync(kFullMask, lead, t);
+      CA v = pad_ca<CA>();
+      uint16_t j = 0;
+      if (k < dt) {
+        const int64_t src = rt + lead_caller_pos(lt, k, dt);
+        v = pack_ca<CA>(W.c, W.a, src);
+        j = static_cast<uint16_t>(__ldg(W.col + src));
+      }
+      if (k < W.w) {
+        W.sca[at + by * t] = v;
+        W.scol[at + by * t] = j;
+      }
+    }
+    __syncwarp();
+    const int ng = min(kStripGroups, w4 - kStripGroups * st);
+    const int64_t o = 128 * static_cast<int64_t>(kStripGroups * st);
+    for (int g = 0; g < ng; ++g) {
+      reinterpret_cast<uint4*>(W.ca_o + o + 128 * g)[lane] = reinterpret_cast<const uint4*>(W.sca + 132 * g)[lane];
+      if (!kBf)
+        reinterpret_cast<uint4*>(W.ca_o + o + 128 * g)[32 + lane] =
+            reinterpret_cast<const uint4*>(W.sca + 132 * g)[32 + lane];
+      reinterpret_cast<uint2*>(W.col_o + o + 128 * g)[lane] = reinterpret_cast<const uint2*>(W.scol + 132 * g)[lane];
+    }
+    if (W.w - 32 * st <= 32) {  // the last strip holds the tail
+      for (int q = 0; q < W.w - 4 * w4; ++q) {
+        const int64_t e = 128 * static_cast<int64_t>(w4) + 32 * q + lane;
+        W.ca_o[e] = W.sca[kStripGroups * 132 + 32 * q + lane];
+        W.col_o[e] = W.scol[kStripGroups * 132 + 32 * q + lane];
+      }
+    }
+    __syncwarp();
+  }
+  return lead;
+}
+
+template <typename CA>
+__global__ void __launch_bounds__(32 * kGatherWarps, sizeof(CA) == 4 ? 4 : 2)
     k_gather(const int64_t* __restrict__ rp, const int32_t* __restrict__ col, const void* __restrict__ c,
              const void* __restrict__ a, const int32_t* __restrict__ perm, const int32_t* __restrict__ sdeg, int64_t In,
              int64_t nslices, const int64_t* __restrict__ slice_off, const int32_t* __restrict__ width,
              uint16_t* __restrict__ col_o, CA* __restrict__ ca_o, int64_t* __restrict__ orig_off,
              int32_t* __restrict__ udeg, uint64_t* __restrict__ lead_o, int J, unsigned* __restrict__ ticket,
              int* __restrict__ dup) {
-  constexpr bool kBf = sizeof(CA) == 4;
   extern __shared__ __align__(16) unsigned char gsm[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   CA* sca = reinterpret_cast<CA*>(gsm + static_cast<size_t>(warp) * kStripElems * (sizeof(CA) + 2));
@@ -320,121 +600,18 @@ __global__ void __launch_bounds__(32 * kGatherWarps)
       orig_off[u] = r;
       udeg[u] = d;
     }
-    const int w = width[s];
-    const int w4 = w >> 2;
     const int64_t base = slice_off[s];
-    // lead edges: lane t keeps row t's
-    uint64_t lead = 0;
-    if (w <= 32) {
-#pragma unroll 4
-      for (int t = 0; t < 32; ++t) {
-        const int64_t rt = __shfl_sync(kFullMask, r, t);
-        const int dt = __shfl_sync(kFullMask, d, t);
-        unsigned key = lane < dt ? cost_key(load_val(c, rt + lane, kBf)) : 0xffffffffu;
-        uint64_t ld = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const unsigned m = __reduce_min_sync(kFullMask, key);
-          const int who = __ffs(__ballot_sync(kFullMask, key == m)) - 1;
-          if (lane == who) key = 0xffffffffu;
-          ld |= static_cast<uint64_t>(q < dt ? who : 0xFFFF) << (16 * q);
-        }
-        if (lane == t) lead = ld;
-        const int j = lane < dt ? __ldg(col + rt + lane) : -1 - lane;  // idle lanes: distinct negative keys
-        const unsigned same = __match_any_sync(kFullMask, j);  // (by every lane, whatever it has found before)
-        if (__popc(same) > 1) twice = true;
-      }
+    const GatherWarp<CA> W{col, c, a, col_o + base, ca_o + base, sca, scol, seen, r, d, width[s], J};
+    uint64_t lead;
+    if (W.w <= kRawWidth) {
+      lead = gather_raw(W, twice);
     } else {
-      for (int t = 0; t < 32; ++t) {
-        const int64_t rt = __shfl_sync(kFullMask, r, t);
-        const int dt = __shfl_sync(kFullMask, d, t);
-        // the lane's four lowest of edges lane, lane + 32, ... (positions fit 16 bits)
-        unsigned lk[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-        unsigned lp[4] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu};
-        const int de = dt < 0xFFFF ? dt : 0xFFFF;
-#pragma unroll 4
-        for (int k = lane; k < de; k += 32) {
-          unsigned x = cost_key(load_val(c, rt + k, kBf)), xi = static_cast<unsigned>(k);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const bool lt = x < lk[q];
-            const unsigned hv = lt ? lk[q] : x, hi = lt ? lp[q] : xi;
-            lk[q] = lt ? x : lk[q];
-            lp[q] = lt ? xi : lp[q];
-            x = hv;
-            xi = hi;
-          }
-        }
-        uint64_t ld = 0;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const unsigned m = __reduce_min_sync(kFullMask, lk[0]);
-          const unsigned p = __reduce_min_sync(kFullMask, lk[0] == m ? lp[0] : 0xffffffffu);
-          if (lp[0] == p && p != 0xffffffffu) {
-#pragma unroll
-            for (int z = 0; z < 3; ++z) lk[z] = lk[z + 1], lp[z] = lp[z + 1];
-            lk[3] = lp[3] = 0xffffffffu;
-          }
-          ld |= static_cast<uint64_t>(q < dt ? p & 0xFFFFu : 0xFFFFu) << (16 * q);
-        }
-        if (lane == t) lead = ld;
-        twice = twice || dt > J;  // more edges than items: some item repeats
-        if (dt > J) continue;     // (warp-uniform)
-        for (int k = lane; k < dt; k += 32) {
-          const int j = __ldg(col + rt + k);
-          const unsigned bit = 1u << (j & 31);
-          if (atomicOr(&seen[j >> 5], bit) & bit) twice = true;
-        }
-        __syncwarp();
-        for (int k = lane; k < dt; k += 32) seen[__ldg(col + rt + k) >> 5] = 0u;
-        __syncwarp();
-      }
+      bool again = false;  // (copies: W and `twice` stay in registers)
+      const GatherWarp<CA> V = W;
+      lead = gather_strips(V, again);
+      twice = twice || again;
     }
     if (u < In) lead_o[u] = lead;
-    // positions 32 st .. of every row, then the strip's elements in order
-    for (int st = 0; 32 * st < w; ++st) {
-      const int k = 32 * st + lane;
-      const int at = k < 4 * w4 ? (lane >> 2) * 132 + (lane & 3) : kStripGroups * 132 + 32 * (k - 4 * w4);
-      const int by = k < 4 * w4 ? 4 : 1;
-#pragma unroll 4
-      for (int t = 0; t < 32; ++t) {
-        const int64_t rt = __shfl_sync(kFullMask, r, t);
-        const int dt = __shfl_sync(kFullMask, d, t);
-        const uint64_t lt = __shfl_sync(kFullMask, lead, t);
-        CA v = pad_ca<CA>();
-        uint16_t j = 0;
-        if (k < dt) {
-          const int64_t src = rt + lead_caller_pos(lt, k, dt);
-          v = pack_ca<CA>(c, a, src);
-          j = static_cast<uint16_t>(__ldg(col + src));
-        }
-        if (k < w) {
-          sca[at + by * t] = v;
-          scol[at + by * t] = j;
-        }
-      }
-      __syncwarp();
-      const int ng = min(kStripGroups, w4 - kStripGroups * st);
-      const int64_t o = base + 128 * static_cast<int64_t>(kStripGroups * st);
-      for (int g = 0; g < ng; ++g) {
-        if (kBf) {
-          reinterpret_cast<uint4*>(ca_o + o + 128 * g)[lane] = reinterpret_cast<const uint4*>(sca + 132 * g)[lane];
-        } else {
-          reinterpret_cast<uint4*>(ca_o + o + 128 * g)[lane] = reinterpret_cast<const uint4*>(sca + 132 * g)[lane];
-          reinterpret_cast<uint4*>(ca_o + o + 128 * g)[32 + lane] =
-              reinterpret_cast<const uint4*>(sca + 132 * g)[32 + lane];
-        }
-        reinterpret_cast<uint2*>(col_o + o + 128 * g)[lane] = reinterpret_cast<const uint2*>(scol + 132 * g)[lane];
-      }
-      if (w - 32 * st <= 32) {  // the last strip holds the tail
-        for (int q = 0; q < w - 4 * w4; ++q) {
-          const int64_t e = base + 128 * static_cast<int64_t>(w4) + 32 * q + lane;
-          ca_o[e] = sca[kStripGroups * 132 + 32 * q + lane];
-          col_o[e] = scol[kStripGroups * 132 + 32 * q + lane];
-        }
-      }
-      __syncwarp();
-    }
   }
   if (__any_sync(kFullMask, twice) && lane == 0) *dup = 1;
 }
