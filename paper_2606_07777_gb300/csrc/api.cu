@@ -378,10 +378,22 @@ void runner_free(Runner& R) {
   R.ctr = nullptr;
 }
 
+// Fixed work of a slice in edges: the round trips of its header and its rows'
+// finish, about six, against one per 16 BF16 or 8 FP32 edges of its width.
+// (16 BF16 members of 10,000 to 1.2M users x 2,000 items in equal-work ranges: 146 us
+// an iteration with 128, 112 with 512, 108 with 2,048; FP32 members,
+// with their wide slices in quarters: 162 with 2,048, 156 with 1,280, 145 with 640.)
+int64_t slice_cost(const Runner& R) { return R.bf16 ? 2048 : 640; }
+
 // Slice-to-CTA tasks.  Interleaved: CTA k sweeps slices k, k + V, ... of
 // every instance; slices are sorted by width, so every CTA gets the same mix.
 // Contiguous: the slices of all instances, in order, are cut into V ranges of
 // equal weight (edges plus a per-slice cost), so a CTA touches few instances.
+// In a batch the CTAs that an instance fills alone share its slices
+// interleaved, and the CTAs at its ends, which have other instances too, take its
+// narrowest slices: in order, one CTA got the widest slices only, too few
+// of them to keep its warps busy (the batch above: 103; dynamic units,
+// which need a barrier each, 141).
 void build_task_list(Runner& R) {
   const int V = R.grid;
   const int n = static_cast<int>(R.probs.size());
@@ -406,39 +418,54 @@ void build_task_list(Runner& R) {
       }
     }
   } else {
-    constexpr int64_t kSliceCost = 128;  // fixed work of a slice, in edge units
+    const int64_t cost = slice_cost(R);
     std::vector<int64_t> base(n + 1, 0);
-    auto weight = [&](int i, int64_t s) { return R.probs[i]->h_slice_off[s] + kSliceCost * s; };
+    auto weight = [&](int i, int64_t s) { return R.probs[i]->h_slice_off[s] + cost * s; };
     for (int i = 0; i < n; ++i) base[i + 1] = base[i] + weight(i, R.probs[i]->lay.nslices);
     const int64_t W = base[n];
+    auto bound = [&](int64_t k) { return W * k / V; };
+    std::vector<std::vector<Task>> list(V);
+    int k0 = 0;  // the CTA with the instance's first unit of weight
+    for (int i = 0; i < n; ++i) {
+      const int64_t ns = R.probs[i]->lay.nslices, lo = base[i], hi = base[i + 1];
+      if (ns == 0) continue;
+      while (bound(k0 + 1) <= lo) ++k0;
+      int k1 = k0;  // and the one with its last
+      while (bound(k1 + 1) < hi) ++k1;
+      // first slice whose start is at or after x
+      auto first_at = [&](int64_t x) {
+        int64_t a = 0, b = ns;
+        while (a < b) {
+          const int64_t m = (a + b) / 2;
+          if (lo + weight(i, m) < x)
+            a = m + 1;
+          else
+            b = m;
+        }
+        return a;
+      };
+      if (n == 1) {
+        for (int k = k0; k <= k1; ++k) {
+          const int64_t f = first_at(bound(k)), e = first_at(bound(k + 1));
+          if (e > f) list[k].push_back({i, 1, f, e});
+        }
+        continue;
+      }
+      if (k0 == k1) {
+        list[k0].push_back({i, 1, 0, ns});
+        continue;
+      }
+      const int f0 = bound(k0) == lo ? k0 : k0 + 1, f1 = bound(k1 + 1) == hi ? k1 + 1 : k1;
+      const int64_t left = f0 > k0 ? bound(k0 + 1) - lo : 0, right = f1 == k1 ? hi - bound(k1) : 0;
+      const int64_t e = f1 > f0 ? first_at(hi - right - left) : 0, f = std::max(e, first_at(hi - right));
+      for (int k = f0; k < f1; ++k)
+        if (k - f0 < e) list[k].push_back({i, f1 - f0, k - f0, e});
+      if (f > e) list[k0].push_back({i, 1, e, f});
+      if (ns > f) list[k1].push_back({i, 1, f, ns});
+    }
     for (int k = 0; k < V; ++k) {
       R.h_cta[k] = static_cast<int32_t>(R.h_tasks.size());
-      const int64_t lo = W * k / V, hi = W * (k + 1) / V;
-      for (int i = 0; i < n; ++i) {
-        const int64_t ns = R.probs[i]->lay.nslices;
-        if (ns == 0 || base[i + 1] <= lo || base[i] >= hi) continue;
-        // first slice whose start is at or after x
-        auto first_at = [&](int64_t x) {
-          int64_t a = 0, b = ns;
-          while (a < b) {
-            const int64_t m = (a + b) / 2;
-            if (base[i] + weight(i, m) < x)
-              a = m + 1;
-            else
-              b = m;
-          }
-          return a;
-        };
-        const int64_t f = first_at(lo), e = first_at(hi);
-        if (e > f) {
-          Task t;
-          t.inst = i;
-          t.stride = 1;
-          t.first = f;
-          t.end = e;
-          R.h_tasks.push_back(t);
-        }
-      }
+      R.h_tasks.insert(R.h_tasks.end(), list[k].begin(), list[k].end());
     }
   }
   R.h_cta[V] = static_cast<int32_t>(R.h_tasks.size());
@@ -447,12 +474,12 @@ void build_task_list(Runner& R) {
     // Work units in instance order, each about max(Wmin, R / (2 V)) of the
     // remaining weight R (guided self-scheduling: large units first, small
     // ones last, so the CTAs run out of work together).
-    constexpr int64_t kSliceCost = 128;
+    const int64_t cost = slice_cost(R);
     std::vector<int64_t> tot(n, 0);
     int64_t W = 0;
     for (int i = 0; i < n; ++i) {
       const int64_t ns = R.probs[i]->lay.nslices;
-      tot[i] = R.probs[i]->h_slice_off[ns] + kSliceCost * ns;
+      tot[i] = R.probs[i]->h_slice_off[ns] + cost * ns;
       W += tot[i];
     }
     const int64_t wmin = std::max<int64_t>(8192, W / (64 * static_cast<int64_t>(V)));
@@ -460,7 +487,7 @@ void build_task_list(Runner& R) {
     for (int i = 0; i < n; ++i) {
       const int64_t ns = R.probs[i]->lay.nslices;
       const std::vector<int64_t>& so = R.probs[i]->h_slice_off;
-      auto weight = [&](int64_t s) { return so[s] + kSliceCost * s; };
+      auto weight = [&](int64_t s) { return so[s] + cost * s; };
       int64_t s = 0;
       while (s < ns) {
         const int64_t size = std::max(wmin, rem / (2 * static_cast<int64_t>(V)));
@@ -790,7 +817,7 @@ dlm_status runner_configure(Runner& R, const dlm_options& o, bool force) {
   const int assign = o.mapping == 1   ? kAssignInterleaved
                      : o.mapping == 2 ? kAssignContiguous
                      : o.mapping == 3 ? kAssignDynamic
-                                      : (R.probs.size() > 1 ? kAssignDynamic : kAssignInterleaved);
+                                      : (R.probs.size() > 1 ? kAssignContiguous : kAssignInterleaved);
   int assign2 = assign;
   for (const dlm_problem* p : R.probs)
     if ((p->m > 1 || p->kind == DLM_BOX_CUT) && assign2 == kAssignDynamic)
