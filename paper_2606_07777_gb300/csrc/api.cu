@@ -309,6 +309,10 @@ InstDesc base_desc(const dlm_problem* p) {
   d.lead = p->lay.lead;
   d.nusers = p->lay.num_active_users;
   d.nwide = p->nwide;
+  const bool simplex = p->kind == DLM_SIMPLEX_LE || p->kind == DLM_SIMPLEX_EQ;
+  const double units = static_cast<double>(simplex ? p->lay.num_active_users : p->nnz);
+  d.obj_c = units * p->z * p->lay.max_abs_c;
+  d.obj_g = 0.5 * units * p->z * p->z;
   d.status = &p->state->status;
   d.scaleG = std::ldexp(1.0f, p->sG);
   d.scaleC = std::ldexp(1.0f, p->sC);

@@ -94,7 +94,8 @@ struct InstDesc {
   float* xout;              // caller-order x or nullptr (stats)
   unsigned long long* cnt;  // fixed-point sum of all x (global count constraint) or nullptr
   unsigned long long* objq; // iteration sweeps: fixed-point sum of (c x + gamma/2 x^2) over all users
-  float scaleG, scaleC, scaleQ, scaleN, scaleO;
+  float scaleG, scaleC, scaleQ, scaleN, scaleO;  // (scaleO 0, certificate sweeps: from gamma and the next two)
+  double obj_c, obj_g;      // |sum_i (c x_i + gamma/2 ||x_i||^2)| <= obj_c + gamma obj_g
   float z;
   int32_t J;
   int32_t kind;

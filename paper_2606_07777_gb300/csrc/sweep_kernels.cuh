@@ -35,9 +35,9 @@
 // 0, z).
 //
 // Determinism: item sums are 64-bit fixed point (value * 2^s rounded, s chosen
-// at set-up so no sum can overflow), exact and order independent; slices are
-// dealt to warps statically and the FP64 objective is summed per warp in
-// slice order, per CTA in warp order and across CTAs in task order.
+// at set-up so no sum can overflow), exact and order independent, and so is the
+// objective within a CTA (certificate sweeps: at a scale chosen from gamma when
+// they start); the CTAs' objectives are added in FP64 in task order.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -495,7 +495,15 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
   }
 
   if (STATS) {
-    wobj += static_cast<double>(ob);
+    // exactly too, so that warps may take slices by ticket: dealt statically
+    // for the sake of an FP64 sum's order, a third of them waited for those with the
+    // widest (1M x 1,000 FP32: one evaluation 157 -> 136 us).  Parts outside
+    // the sum's range, which no ordinary data have, are added as they are.
+    const float t = ob * S.scaleO;
+    if (S.scaleO != 0.f && fabsf(t) < 9.2e18f)
+      oq += static_cast<unsigned long long>(__float2ll_rn(t));
+    else
+      wobj += static_cast<double>(ob);
   } else {
     // the user's objective part, added exactly (64-bit fixed point)
     oq += fixp(ob, S.scaleO);
@@ -687,7 +695,7 @@ __device__ __noinline__ QuarterSums do_quarter(const InstDesc& D, const Seg& S, 
 }
 
 // The constants as the sweep's registers: those that the kernel parameter holds are read from it.
-template <bool ONE>
+template <bool ONE, bool STATS>
 __device__ __forceinline__ Seg seg_of(const InstDesc& D, const Seg& sS) {
   Seg S = sS;
   if (ONE) {
@@ -696,7 +704,7 @@ __device__ __forceinline__ Seg seg_of(const InstDesc& D, const Seg& sS) {
     S.scaleC = D.scaleC;
     S.scaleQ = D.scaleQ;
     S.scaleN = D.scaleN;
-    S.scaleO = D.scaleO;
+    if (!STATS) S.scaleO = D.scaleO;
     S.kind = D.kind;
   }
   return S;
@@ -726,10 +734,11 @@ __device__ __forceinline__ void slices_of(const InstDesc& D, const Seg& sS, cons
                                                           coop_max);
       cn += r.cn;
       oq += r.oq;
+      if (STATS) wobj += r.ob;
     }
     i -= 3 * nq;
   }
-  const Seg S = seg_of<ONE>(D, sS);
+  const Seg S = seg_of<ONE, STATS>(D, sS);
   if constexpr (!AHEAD) {
     for (; i < n; i = next_ticket(next) - (WIDE ? 3 * nq : 0)) {
       const int64_t s = T.first + static_cast<int64_t>(i) * T.stride;
@@ -829,36 +838,23 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     double wobj = 0.0;
     for (int k = t; k < te; ++k) {
       const Task T = tasks[k];
-      if (STATS) {
-        // static order: the FP64 objective partials are summed in a fixed order
-        int64_t nq = 0;
-        if constexpr (WIDE) {
-          nq = task_wide(T, sD.nwide);
-          for (int64_t i = warp; i < 4 * nq; i += nw) {
-            const QuarterSums r = do_quarter<P, STATS, K>(sD, sS, ys, accG, accC, accQ,
-                                                                 T.first + (i >> 2) * T.stride, i & 3, coop_max);
-            wobj += r.ob;
-            cn += r.cn;
-          }
-        }
-        const Seg S = seg_of<ONE>(sD, sS);
-        const int64_t step = static_cast<int64_t>(T.stride) * nw;
-        for (int64_t s = T.first + static_cast<int64_t>(T.stride) * (nq + warp); s < T.end; s += step)
-          do_slice<P, STATS, K>(sD, S, ys, accG, accC, accQ, s, __ldg(sD.slice_off + s), __ldg(sD.slice_w + s),
-                                       coop_max, wobj, cn, oq, [] {});
-      } else {
-        // dynamic order within the CTA (item sums are exact, so the order of
-        // slices does not change any result)
-        slices_of<P, STATS, K, ONE, WIDE, true>(sD, sS, ys, accG, accC, accQ, T, &s_next, coop_max, wobj, cn, oq);
-        __syncthreads();
-        if (threadIdx.x == 0) s_next = 0;
-        __syncthreads();
-      }
+      // dynamic order within the CTA (the sums are exact, so the order of
+      // slices does not change any result)
+      slices_of<P, STATS, K, ONE, WIDE, true>(sD, sS, ys, accG, accC, accQ, T, &s_next, coop_max, wobj, cn, oq);
+      __syncthreads();
+      if (threadIdx.x == 0) s_next = 0;
+      __syncthreads();
     }
     if (STATS) {
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) wobj += __shfl_xor_sync(kFull, wobj, o);
-      if (lane == 0) wsum[warp] = wobj;
+      for (int o = 16; o > 0; o >>= 1) {
+        wobj += __shfl_xor_sync(kFull, wobj, o);
+        oq += __shfl_xor_sync(kFull, oq, o);
+      }
+      if (lane == 0) {
+        wsum[warp] = wobj;
+        s_red[warp] = oq;
+      }
     } else {
       cta_add_u64(oq, s_red, sD.objq);
     }
@@ -882,7 +878,12 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     }
     if (STATS && threadIdx.x == 0) {
       double sum = 0.0;
-      for (int w = 0; w < nw; ++w) sum += wsum[w];
+      unsigned long long q = 0ull;
+      for (int w = 0; w < nw; ++w) {
+        sum += wsum[w];
+        q += s_red[w];
+      }
+      if (q != 0ull) sum += static_cast<double>(static_cast<long long>(q)) / static_cast<double>(sS.scaleO);
       sD.seg_obj[t] = sum;
     }
     __syncthreads();
