@@ -174,6 +174,10 @@ struct Runner {
   int upd_ctas = 1;      // update grid width (the largest member's)
   void* tabs = nullptr;  // the instances' tables (inst_iter, inst_stats, upd, st_stats)
   void* plan = nullptr;  // the tasks and their lists (tasks .. ctr)
+  // the copies' sources: kept, since a copy from pageable memory may be read
+  // after the call that starts it has returned
+  std::vector<char> h_tabs, h_plan;
+  std::vector<double> h_cuts;
   InstDesc *inst_iter = nullptr, *inst_stats = nullptr;
   InstDesc h_iter0{}, h_stats0{};  // host copies of inst_iter[0], inst_stats[0]
   StatsInst h_st0{};               // and of st_stats[0]
@@ -593,16 +597,18 @@ dlm_status write_tables(Runner& R) {
   Packed pk;
   const size_t o_it = pk.put(it.data(), sizeof(InstDesc) * n), o_ss = pk.put(ss.data(), sizeof(InstDesc) * n),
                o_up = pk.put(up.data(), sizeof(UpdInst) * n), o_st = pk.put(st.data(), sizeof(StatsInst) * n);
+  if (R.tabs) CK(cudaStreamSynchronize(R.stream));  // the copy before this one has been read
+  R.h_tabs.swap(pk.host);
   if (!R.tabs) {  // (n is fixed for a runner, and with it the size)
     char* t = nullptr;
-    CK(dalloc(&t, pk.host.size(), R.stream));
+    CK(dalloc(&t, R.h_tabs.size(), R.stream));
     R.tabs = t;
     R.inst_iter = reinterpret_cast<InstDesc*>(t + o_it);
     R.inst_stats = reinterpret_cast<InstDesc*>(t + o_ss);
     R.upd = reinterpret_cast<UpdInst*>(t + o_up);
     R.st_stats = reinterpret_cast<StatsInst*>(t + o_st);
   }
-  CK(cudaMemcpyAsync(R.tabs, pk.host.data(), pk.host.size(), cudaMemcpyHostToDevice, R.stream));
+  CK(cudaMemcpyAsync(R.tabs, R.h_tabs.data(), R.h_tabs.size(), cudaMemcpyHostToDevice, R.stream));
   return DLM_OK;
 }
 
@@ -612,10 +618,10 @@ dlm_status runner_build(Runner& R) {
   invalidate_graph(R);
   const int n = static_cast<int>(R.probs.size());
   if (R.probs[0]->kind == DLM_BOX_CUT && !R.cuts) {
-    std::vector<double> h(n);
-    for (int i = 0; i < n; ++i) h[i] = R.probs[i]->cut;
+    R.h_cuts.resize(n);
+    for (int i = 0; i < n; ++i) R.h_cuts[i] = R.probs[i]->cut;
     CK(dalloc(&R.cuts, n, R.stream));
-    CK(cudaMemcpyAsync(R.cuts, h.data(), sizeof(double) * n, cudaMemcpyHostToDevice, R.stream));
+    CK(cudaMemcpyAsync(R.cuts, R.h_cuts.data(), sizeof(double) * n, cudaMemcpyHostToDevice, R.stream));
   }
   build_task_list(R);
   std::vector<int32_t> flat;
@@ -639,7 +645,8 @@ dlm_status runner_build(Runner& R) {
   R.units = reinterpret_cast<Task*>(t + o_u);
   R.ctr = reinterpret_cast<unsigned*>(t + o_z);
   R.seg_obj = reinterpret_cast<double*>(t + o_s);
-  CK(cudaMemcpyAsync(t, pk.host.data(), pk.host.size(), cudaMemcpyHostToDevice, R.stream));
+  R.h_plan.swap(pk.host);  // (the stream has been synchronized above)
+  CK(cudaMemcpyAsync(t, R.h_plan.data(), R.h_plan.size(), cudaMemcpyHostToDevice, R.stream));
   return write_tables(R);
 }
 
@@ -690,7 +697,7 @@ SweepLaunch launch_of(const Runner& R, const InstDesc* tab) {
   return L;
 }
 
-// One-family instances take the sweep of sweep.cu, several families the
+// One-family instances take the sweep of sweep_kernels.cuh, several families the
 // general sweep of sweep_multi.cu (static tasks only).
 cudaError_t dispatch_sweep(const SweepLaunch& L, bool stats, bool bf16) {
   return L.fam > 1 ? launch_sweep_multi(L, stats, bf16) : launch_sweep(L, stats, bf16);
@@ -941,9 +948,9 @@ dlm_status upload_schedule(dlm_problem* p) {
     const double n = tab.back() * p->factor;
     tab.push_back(n > p->gamma_end ? n : p->gamma_end);
   }
+  // (the host copy of the old table may still be read, and a batch on another stream the device's)
+  if (p->gamma_tab) CK(cudaStreamSynchronize(p->stream));
   if (static_cast<int64_t>(tab.size()) > p->gamma_tab_cap) {
-    // (a batch on another stream may still read the old table)
-    CK(cudaStreamSynchronize(p->stream));
     dev_free(p->gamma_tab, p->stream);
     p->gamma_tab = nullptr;
     p->gamma_tab_cap = 0;

@@ -89,7 +89,8 @@ __device__ __forceinline__ void load_val4(const void* p, int64_t q, bool bf16, f
 // edges need (any array of its own does; a view into one may not).
 inline bool aligned4(const int32_t* col, const void* c, const void* a, bool bf16) {
   const uintptr_t m = bf16 ? 7 : 15;
-  return (reinterpret_cast<uintptr_t>(col) & 15) == 0 && ((reinterpret_cast<uintptr_t>(c) | reinterpret_cast<uintptr_t>(a)) & m) == 0;
+  return (reinterpret_cast<uintptr_t>(col) & 15) == 0 &&
+         ((reinterpret_cast<uintptr_t>(c) | reinterpret_cast<uintptr_t>(a)) & m) == 0;
 }
 
 // Edge checks, item degrees, max |a|, max |c|.  With J <= 16384 each block
@@ -312,7 +313,8 @@ template <typename K>
 __device__ __forceinline__ uint64_t lead_of(const K (&lk)[4], int d) {
   uint64_t ld = 0;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) ld |= static_cast<uint64_t>(q < d ? static_cast<unsigned>(lk[q]) & 0xFFFFu : 0xFFFFu) << (16 * q);
+  for (int q = 0; q < 4; ++q)
+    ld |= static_cast<uint64_t>(q < d ? static_cast<unsigned>(lk[q]) & 0xFFFFu : 0xFFFFu) << (16 * q);
   return ld;
 }
 
@@ -624,9 +626,9 @@ __global__ void __launch_bounds__(32 * kGatherWarps, sizeof(CA) == 4 ? 4 : 2)
 // (`quad`: aligned arrays), conversions off the FP64 pipe.  50M BF16 edges, 1,000 items:
 // 2 x 338 us in two passes.
 template <bool SQ, bool S1, bool SMEM>
-__global__ void __launch_bounds__(1024) k_item_sums(const int32_t* __restrict__ col, const void* __restrict__ a, bool bf16,
-                                                    int64_t nnz, int64_t J, float scale_sq, float scale_s1, bool quad,
-                                                    unsigned long long* __restrict__ sums) {
+__global__ void __launch_bounds__(1024)
+    k_item_sums(const int32_t* __restrict__ col, const void* __restrict__ a, bool bf16, int64_t nnz, int64_t J,
+                float scale_sq, float scale_s1, bool quad, unsigned long long* __restrict__ sums) {
   extern __shared__ unsigned long long sacc[];
   unsigned long long* sq = SMEM ? sacc : sums;
   unsigned long long* s1 = (SMEM && !SQ) ? sacc : sq + J;

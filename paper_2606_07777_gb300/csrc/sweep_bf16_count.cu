@@ -5,6 +5,8 @@
 namespace dlm {
 
 cudaError_t sweep_prepare_bf16_count(int smem_limit) { return prepare_policy<Counted<Narrow<BF16Pair>>>(smem_limit); }
-cudaError_t launch_sweep_bf16_count(const SweepLaunch& L, bool stats) { return launch_policy<Counted<Narrow<BF16Pair>>>(L, stats); }
+cudaError_t launch_sweep_bf16_count(const SweepLaunch& L, bool stats) {
+  return launch_policy<Counted<Narrow<BF16Pair>>>(L, stats);
+}
 
 }  // namespace dlm

@@ -18,7 +18,7 @@
 //
 // Layout, item sums (64-bit fixed point in shared memory, flushed once per
 // CTA), static slice order and the FP64 objective partials are those of the
-// one-family sweep (sweep.cu).
+// one-family sweep (sweep_kernels.cuh).
 #include <algorithm>
 
 #include "boxcut.cuh"
@@ -411,12 +411,12 @@ __device__ __forceinline__ void boxcut_slice(const InstDesc& D, const BSeg& S, c
 // Per CTA its tasks; certificate sweeps deal a task's slices to warps in a
 // static order (first + stride (warp + k nw)), iteration sweeps from a
 // per-CTA ticket counter.
-// ONE: one instance, its descriptor a kernel parameter (as in sweep.cu).
+// ONE: one instance, its descriptor a kernel parameter (as in sweep_kernels.cuh).
 template <class V, bool STATS, bool ONE>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-    sweep_boxcut_kernel(const __grid_constant__ InstDesc one, const InstDesc* __restrict__ insts, const Task* __restrict__ tasks,
-                        const int32_t* __restrict__ cta_task, int smemJ, int jlo, int jw,
-                        const double* __restrict__ cuts) {
+    sweep_boxcut_kernel(const __grid_constant__ InstDesc one, const InstDesc* __restrict__ insts,
+                        const Task* __restrict__ tasks, const int32_t* __restrict__ cta_task, int smemJ, int jlo,
+                        int jw, const double* __restrict__ cuts) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int accN = STATS ? jw : smemJ;
   unsigned long long* accG = reinterpret_cast<unsigned long long*>(smem_raw);

@@ -1,4 +1,4 @@
-// sweep_common.cuh -- device helpers shared by the sweep kernels (sweep.cu,
+// sweep_common.cuh -- device helpers shared by the sweep kernels (sweep_kernels.cuh,
 // sweep_short.cu, sweep_multi.cu, sweep_boxcut.cu): the value layouts of the
 // interleaved (c, a) stream, the slice element order, 64-bit fixed point,
 // float-pair arithmetic, and the per-edge deposit of the one-family sweeps.

@@ -5,6 +5,8 @@
 namespace dlm {
 
 cudaError_t sweep_prepare_f32_count(int smem_limit) { return prepare_policy<Counted<Narrow<F32Pair>>>(smem_limit); }
-cudaError_t launch_sweep_f32_count(const SweepLaunch& L, bool stats) { return launch_policy<Counted<Narrow<F32Pair>>>(L, stats); }
+cudaError_t launch_sweep_f32_count(const SweepLaunch& L, bool stats) {
+  return launch_policy<Counted<Narrow<F32Pair>>>(L, stats);
+}
 
 }  // namespace dlm

@@ -173,9 +173,9 @@ __device__ __forceinline__ void coop_user(const Seg& S, const float* __restrict_
 // A row whose simplex active set is the r <= 3 recorded edges (on the
 // inequality simplex with tau <= 0: those of them with u > 0): load them once,
 // compute the threshold over them in pair arithmetic, deposit x on each.
-// Returns the objective part.  (Iteration sweeps.)  Loading them once saves a re-read (4 % on the 64-instance batch, 6 % on the
-// appendix instance once its rows have several active edges; no change on
-// the precision sweep).
+// Returns the objective part.  (Iteration sweeps.)  Loading them once saves a
+// re-read (4 % on the 64-instance batch, 6 % on the appendix instance once its
+// rows have several active edges; no change on the precision sweep).
 template <class P, int K>
 __device__ __forceinline__ float rows_upto(const Seg& S, const float* __restrict__ ys, unsigned long long* accG,
                                          const typename P::IX* __restrict__ col0, const typename P::T* __restrict__ ca0,

@@ -5,10 +5,10 @@
 //     u_ij = -(c_ij + sum_k a_kij y_kj),   x_i = Proj_C_i(u_i / gamma),
 // and per family and item (A_k x)_j = sum_i a_kij x_ij.
 //
-// Layout: the slices of sweep.cu (users sorted by degree, 32 per slice) with
+// Layout: the slices of sweep_kernels.cuh (users sorted by degree, 32 per slice) with
 // the (c, a_0) stream and, for k >= 1, one more stream of a_k in the same
 // element order (a_ext + (k - 1) * ext_stride).  One lane per user, slices
-// dealt to warps in a static order.  The projection follows sweep.cu: a
+// taken by the CTA's warps by ticket (in a fixed order by certificate sweeps).  The projection follows sweep_kernels.cuh: a
 // streaming pass keeps the four largest u with the positions of the first
 // three, rows with at most three active edges are finished from those
 // positions, larger active sets take the Michelot iteration from tau_4; the
@@ -121,7 +121,7 @@ __device__ __forceinline__ float x_of(const MSeg& S, bool box, float tau, float 
 
 // One slice.  The first pass streams the row in groups of four edges (128-
 // and 64-bit loads) and keeps its four largest u with the positions of the
-// first three, as in sweep.cu: at most three active edges (mode 1, 2) are
+// first three, as in sweep_kernels.cuh: at most three active edges (mode 1, 2) are
 // then handled from those positions; four or more (mode 3), and the box, take
 // the Michelot iteration and full passes.
 template <class P, bool STATS, int M>
@@ -340,11 +340,12 @@ __device__ __forceinline__ void multi_slice(const InstDesc& D, const MSeg& S, co
 
 // Shared memory: accG [m smemJ], then (STATS) accC, accQ [smemJ each], then
 // ys [m smemJ] floats, then 32 doubles of warp partials.
-// ONE: one instance, its descriptor a kernel parameter (as in sweep.cu).
+// ONE: one instance, its descriptor a kernel parameter (as in sweep_kernels.cuh).
 template <class P, bool STATS, int M, bool ONE>
 __global__ void __launch_bounds__(kSweepThreads, 1)
-    sweep_multi_kernel(const __grid_constant__ InstDesc one, const InstDesc* __restrict__ insts, const Task* __restrict__ tasks,
-                       const int32_t* __restrict__ cta_task, int smemJ, int m, bool bf16) {
+    sweep_multi_kernel(const __grid_constant__ InstDesc one, const InstDesc* __restrict__ insts,
+                       const Task* __restrict__ tasks, const int32_t* __restrict__ cta_task, int smemJ, int m,
+                       bool bf16) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned long long* accG = reinterpret_cast<unsigned long long*>(smem_raw);
   unsigned long long* accC = accG + static_cast<size_t>(m) * smemJ;

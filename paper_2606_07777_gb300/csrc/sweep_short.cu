@@ -5,7 +5,7 @@
 // enough rows, each edge's value as a float pair or its dual); a sorting
 // network orders the values and the sort-based threshold rule finds the
 // active set in one scan; the threshold's refinement and the deposits read
-// the row's c, a and items again (from L1).  The general sweep (sweep.cu)
+// the row's c, a and items again (from L1).  The general sweep (sweep_kernels.cuh)
 // tracks the four (or eight) largest values and, for rows with more active
 // edges, iterates over the row, streaming it again for every pass -- the
 // usual case near the optimum on instances whose rows are short and mostly
