@@ -105,7 +105,7 @@ typedef struct {
 typedef struct {
   int32_t gap_every;     /* iterations between certified-gap checks in dlm_solve (default 50) */
   int32_t precondition;  /* 1: row normalization (App. B.2) as the per-item step gamma/sum_i a_ij^2 */
-  int32_t mapping;       /* slice-to-CTA assignment: 0 default (1 for a handle, 2 for a batch),
+  int32_t mapping;       /* slice-to-CTA assignment: 0 default (1 for a handle; for a batch 2, or 3 if it is large),
                             1 interleaved (CTA k sweeps slices k, k + grid, ... of every instance),
                             2 contiguous (equal-work ranges of the instances' slices in order; in a
                               batch, CTAs with one member only share its slices interleaved),
@@ -333,7 +333,7 @@ dlm_status dlm_release_cached_memory(void);
  * member's own handle and on the batch act on the same state, so the caller
  * must not let them overlap.  Destroy the batch before its members. */
 dlm_status dlm_batch_create(dlm_problem* const* probs, int32_t n, void* stream, dlm_batch** out);
-/* Mapping fields of `opt` for the batch (mapping 0 means contiguous here);
+/* Mapping fields of `opt` for the batch (mapping 0 means contiguous here, dynamic for large batches);
  * gap_every and graph_iters apply to dlm_batch_solve and dlm_batch_step. */
 dlm_status dlm_batch_set_options(dlm_batch* bt, const dlm_options* opt);
 /* dlm_autotune over the whole batch (interleaved candidates only up to 8 members). */

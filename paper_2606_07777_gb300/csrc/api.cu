@@ -819,6 +819,20 @@ int default_threads(const Runner& R, int grid) {
   return t;
 }
 
+// A batch's default order: equal-work ranges up to kRangeBytes of the layout a
+// CTA, dynamic units above.  Units cost barriers and changes of instance, some 30 us
+// whatever the size; ranges cost what the weights miss, a share of the sweep
+// (members differ in gamma, and their rows in active edges).  Ranges against
+// units, us an iteration: BF16 102 / 134 at 2.2 MB a CTA, 162 / 174 at 3.5, 245 / 229
+// at 5.8, 518 / 435 at 13.3; FP32 214 / 197 at 5.2, 362 / 286 at 9.3.
+constexpr int64_t kRangeBytes = 5'000'000;
+int default_order(const Runner& R, int grid) {
+  if (R.probs.size() == 1) return kAssignInterleaved;
+  int64_t bytes = 0;
+  for (const dlm_problem* p : R.probs) bytes += p->lay.padded_nnz * (R.bf16 ? 6 : 10);
+  return bytes <= kRangeBytes * grid ? kAssignContiguous : kAssignDynamic;
+}
+
 // Applies mapping options to a runner: grid, threads, cooperative threshold,
 // assignment.  Rebuilds the tasks when the launch shape changes.
 dlm_status runner_configure(Runner& R, const dlm_options& o, bool force) {
@@ -828,7 +842,7 @@ dlm_status runner_configure(Runner& R, const dlm_options& o, bool force) {
   const int assign = o.mapping == 1   ? kAssignInterleaved
                      : o.mapping == 2 ? kAssignContiguous
                      : o.mapping == 3 ? kAssignDynamic
-                                      : (R.probs.size() > 1 ? kAssignContiguous : kAssignInterleaved);
+                                      : default_order(R, grid);
   int assign2 = assign;
   for (const dlm_problem* p : R.probs)
     if ((p->m > 1 || p->kind == DLM_BOX_CUT) && assign2 == kAssignDynamic)
