@@ -250,6 +250,7 @@ struct dlm_problem {
   double* traj = nullptr;                   // [kTrajCap] g(y_t) per iteration (ring)
   double* upd_part = nullptr;               // update partials [update_parts(m J + 1)]
   unsigned* upd_ticket = nullptr;
+  double* slice_obj = nullptr;              // certificate sweeps' objective by slice (one family, not the box cut)
   int64_t traj_from = 0;                    // first iteration whose trajectory entry is valid
   double *gamma_tab = nullptr, *stats_out = nullptr;
   int64_t nstages = 1, gamma_tab_cap = 0;
@@ -313,10 +314,7 @@ InstDesc base_desc(const dlm_problem* p) {
   d.lead = p->lay.lead;
   d.nusers = p->lay.num_active_users;
   d.nwide = p->nwide;
-  const bool simplex = p->kind == DLM_SIMPLEX_LE || p->kind == DLM_SIMPLEX_EQ;
-  const double units = static_cast<double>(simplex ? p->lay.num_active_users : p->nnz);
-  d.obj_c = units * p->z * p->lay.max_abs_c;
-  d.obj_g = 0.5 * units * p->z * p->z;
+  d.slice_obj = p->slice_obj;
   d.status = &p->state->status;
   d.scaleG = std::ldexp(1.0f, p->sG);
   d.scaleC = std::ldexp(1.0f, p->sC);
@@ -891,7 +889,7 @@ void free_problem(dlm_problem* p) {
   void* pooled[] = {p->lay.slice_off, p->lay.slice_w, p->lay.col16, p->lay.ca,    p->lay.orig_off, p->lay.udeg,
                     p->lay.lead,      p->a_ext,       p->b,         p->curv,      p->lam,          p->y,
                     p->gamma_tab,     p->stats_out,   p->state,     p->lam64,     p->y64,          p->traj,
-                    p->upd_part,      p->upd_ticket,  p->own_sums ? p->xsum : nullptr,
+                    p->upd_part,      p->upd_ticket,  p->slice_obj, p->own_sums ? p->xsum : nullptr,
                     p->own_sums ? p->csum : nullptr};
   for (void* q : pooled) dev_free(q, s);
   if (s) cudaStreamSynchronize(s);
@@ -1520,6 +1518,13 @@ dlm_status dlm_create(const dlm_problem_desc* desc, void* stream, dlm_problem** 
   for (void*& q : tmp) q = nullptr;
 #undef CKC
   p->nwide = wide_slices(p);
+  if (m == 1 && p->kind != DLM_BOX_CUT) {
+    const cudaError_t e = dalloc(&p->slice_obj, static_cast<size_t>(p->lay.nslices + 3 * p->nwide), p->stream);
+    if (e != cudaSuccess) {
+      free_problem(p);
+      return fail(DLM_ERR_CUDA, std::string("slice objective parts: ") + cudaGetErrorString(e));
+    }
+  }
   // The handle's own runner: this one instance.
   Runner& R = p->run;
   R.probs = {p};

@@ -91,11 +91,11 @@ struct InstDesc {
   unsigned long long* accC; // [J] fixed-point sum c x (stats)
   unsigned long long* accQ; // [J] fixed-point sum x^2 (stats)
   double* seg_obj;          // [tasks] FP64 objective partial per (CTA, instance) segment (stats)
+  double* slice_obj;        // [nslices + 3 nwide] FP64 objective part per slice or quarter (stats, one-family sweep)
   float* xout;              // caller-order x or nullptr (stats)
   unsigned long long* cnt;  // fixed-point sum of all x (global count constraint) or nullptr
   unsigned long long* objq; // iteration sweeps: fixed-point sum of (c x + gamma/2 x^2) over all users
-  float scaleG, scaleC, scaleQ, scaleN, scaleO;  // (scaleO 0, certificate sweeps: from gamma and the next two)
-  double obj_c, obj_g;      // |sum_i (c x_i + gamma/2 ||x_i||^2)| <= obj_c + gamma obj_g
+  float scaleG, scaleC, scaleQ, scaleN, scaleO;
   float z;
   int32_t J;
   int32_t kind;

@@ -149,12 +149,6 @@ struct Seg {
 // the 32 warps of a CTA computing them each, well under 1 us for one warp.
 // (With the update's scalars taken the same way, an iteration of the tiny
 // instance, 10,000 x 100, went from 11.6 to 6.0 us.)
-// Power of two that takes sums of magnitude up to `bound` to 2^60 at most; 0 if no normal float does.
-__device__ __forceinline__ float objective_scale(double bound) {
-  if (!(bound > 0.0) || !isfinite(bound)) return 0.f;
-  const int e = 59 - ilogb(bound);
-  return e >= -126 && e <= 127 ? __int_as_float((e + 127) << 23) : 0.f;
-}
 __device__ __forceinline__ void fill_seg(const InstDesc& D, int jlo, int jw, Seg& S) {
   const double g = D.gamma != nullptr ? *D.gamma : D.gamma_val;
   S.gamma = static_cast<float>(g);
@@ -167,7 +161,7 @@ __device__ __forceinline__ void fill_seg(const InstDesc& D, int jlo, int jw, Seg
   S.scaleC = D.scaleC;
   S.scaleQ = D.scaleQ;
   S.scaleN = D.scaleN;
-  S.scaleO = D.scaleO != 0.f ? D.scaleO : objective_scale(D.obj_c + g * D.obj_g);
+  S.scaleO = D.scaleO;
   S.kind = D.kind;
   S.count = D.count_on;
   S.mu = D.count_on ? D.y[D.J] : 0.f;

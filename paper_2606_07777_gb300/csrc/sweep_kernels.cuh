@@ -36,8 +36,9 @@
 //
 // Determinism: item sums are 64-bit fixed point (value * 2^s rounded, s chosen
 // at set-up so no sum can overflow), exact and order independent, and so is the
-// objective within a CTA (certificate sweeps: at a scale chosen from gamma when
-// they start); the CTAs' objectives are added in FP64 in task order.
+// iteration's objective.  A certificate's objective is FP64: one part per slice,
+// summed over its rows in lane order, the parts of a CTA's slices in slice order, the
+// CTAs' in task order.
 #pragma once
 
 #include <cuda_bf16.h>
@@ -269,13 +270,14 @@ __device__ __forceinline__ void topk_insert(float u, int k, TopK<K>& t) {
 // col0/ca0 are the slice's element streams.  The lane finishes row ut of the
 // slice when act is set: its own (ut = lane), or with Q (a quarter slice, rows
 // 8 quarter .. 8 quarter + 7) row 8 quarter + lane / 4 in the first lane of each four.
+// part: where a certificate sweep puts the objective of these rows (slice_part).
 template <class P, bool STATS, int K, bool Q = false>
 __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, const float* __restrict__ ys,
                                              unsigned long long* accG, unsigned long long* accC,
                                              unsigned long long* accQ, int64_t s, int w,
                                              const typename P::IX* __restrict__ col0,
                                              const typename P::T* __restrict__ ca0, const TopK<K>& tk, int coop_max,
-                                             double& wobj, unsigned long long& cn, unsigned long long& oq,
+                                             int64_t part, unsigned long long& cn, unsigned long long& oq,
                                              int quarter = 0) {
   const int lane = Q ? 8 * quarter + static_cast<int>((threadIdx.x & 31) >> 2) : static_cast<int>(threadIdx.x & 31);
   const bool act = !Q || (threadIdx.x & 3) == 0;
@@ -496,15 +498,13 @@ __device__ __forceinline__ void finish_slice(const InstDesc& D, const Seg& S, co
   }
 
   if (STATS) {
-    // exactly too, so that warps may take slices by ticket: dealt statically
-    // for the sake of an FP64 sum's order, a third of them waited for those with the
-    // widest (1M x 1,000 FP32: one evaluation 157 -> 136 us).  Parts outside
-    // the sum's range, which no ordinary data have, are added as they are.
-    const float t = ob * S.scaleO;
-    if (S.scaleO != 0.f && fabsf(t) < 9.2e18f)
-      oq += static_cast<unsigned long long>(__float2ll_rn(t));
-    else
-      wobj += static_cast<double>(ob);
+    // FP64, to a place of its own: the warps may then take slices by ticket (dealt
+    // statically for the sake of one running sum's order, a third of them waited for those
+    // with the widest: 1M x 1,000 FP32, one evaluation 157 us, now 136).
+    double o = static_cast<double>(ob);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) o += __shfl_xor_sync(kFull, o, d);
+    if ((threadIdx.x & 31) == 0) D.slice_obj[part] = o;
   } else {
     // the user's objective part, added exactly (64-bit fixed point)
     oq += fixp(ob, S.scaleO);
@@ -588,12 +588,12 @@ template <class P, bool STATS, int K, class Ahead>
 __device__ __forceinline__ void do_slice(const InstDesc& D, const Seg& S, const float* __restrict__ ys,
                                          unsigned long long* accG, unsigned long long* accC,
                                          unsigned long long* accQ, int64_t s, int64_t off, int w, int coop_max,
-                                         double& wobj, unsigned long long& cn, unsigned long long& oq, Ahead&& ahead) {
+                                         int64_t part, unsigned long long& cn, unsigned long long& oq, Ahead&& ahead) {
   const typename P::IX* __restrict__ col0 = P::idx(D) + off;
   const typename P::T* __restrict__ ca0 = static_cast<const typename P::T*>(D.ca) + off;
   const TopK<K> tk = scan_slice<P, K>(ys, w, col0, ca0);
   ahead();
-  finish_slice<P, STATS, K>(D, S, ys, accG, accC, accQ, s, w, col0, ca0, tk, coop_max, wobj, cn, oq);
+  finish_slice<P, STATS, K>(D, S, ys, accG, accC, accQ, s, w, col0, ca0, tk, coop_max, part, cn, oq);
 }
 
 // A quarter of a wide slice: rows 8 quarter .. 8 quarter + 7, four lanes a
@@ -678,7 +678,6 @@ __device__ __forceinline__ TopK<K> scan_quarter(const float* __restrict__ ys, in
 }
 struct QuarterSums {
   unsigned long long cn, oq;
-  double ob;
 };
 template <class P, bool STATS, int K>
 __device__ __noinline__ QuarterSums do_quarter(const InstDesc& D, const Seg& S, const float* __restrict__ ys,
@@ -688,9 +687,10 @@ __device__ __noinline__ QuarterSums do_quarter(const InstDesc& D, const Seg& S, 
   const int w = __ldg(D.slice_w + s);
   const typename P::IX* __restrict__ col0 = P::idx(D) + off;
   const typename P::T* __restrict__ ca0 = static_cast<const typename P::T*>(D.ca) + off;
-  QuarterSums r{0ull, 0ull, 0.0};
+  QuarterSums r{0ull, 0ull};
   const TopK<K> tk = scan_quarter<P, K>(ys, w, col0, ca0, quarter);
-  finish_slice<P, STATS, K, true>(D, S, ys, accG, accC, accQ, s, w, col0, ca0, tk, coop_max, r.ob, r.cn, r.oq, quarter);
+  finish_slice<P, STATS, K, true>(D, S, ys, accG, accC, accQ, s, w, col0, ca0, tk, coop_max, 4 * s + quarter, r.cn, r.oq,
+                                  quarter);
   return r;
 }
 
@@ -704,7 +704,7 @@ __device__ __forceinline__ Seg seg_of(const InstDesc& D, const Seg& sS) {
     S.scaleC = D.scaleC;
     S.scaleQ = D.scaleQ;
     S.scaleN = D.scaleN;
-    if (!STATS) S.scaleO = D.scaleO;
+    S.scaleO = D.scaleO;
     S.kind = D.kind;
   }
   return S;
@@ -715,6 +715,13 @@ __device__ __forceinline__ int64_t task_wide(const Task& T, int64_t nwide) {
   return T.first < end ? (end - T.first + T.stride - 1) / T.stride : 0;
 }
 
+// Where slice s leaves its part of a certificate's objective: after the four parts
+// of each slice taken in quarters (4 s + quarter).
+template <bool WIDE>
+__device__ __forceinline__ int64_t slice_part(const InstDesc& D, int64_t s) {
+  return WIDE ? s + 3 * D.nwide : s;
+}
+
 // The warp's share of a task's slices, by tickets.  AHEAD: the ticket and the
 // header (offset, width) of the next slice are fetched before the finish of
 // the one in hand (16M x 5,000 BF16: 492 -> 470 us an iteration); not where the CTA meets a barrier at the
@@ -723,7 +730,7 @@ template <class P, bool STATS, int K, bool ONE, bool WIDE, bool AHEAD>
 __device__ __forceinline__ void slices_of(const InstDesc& D, const Seg& sS, const float* __restrict__ ys,
                                           unsigned long long* accG, unsigned long long* accC,
                                           unsigned long long* accQ, const Task& T, unsigned* next, int coop_max,
-                                          double& wobj, unsigned long long& cn, unsigned long long& oq) {
+                                          unsigned long long& cn, unsigned long long& oq) {
   const int n = static_cast<int>((T.end - T.first + T.stride - 1) / T.stride);
   const int nq = WIDE ? static_cast<int>(task_wide(T, D.nwide)) : 0;  // its first slices, taken in quarters
   int i = next_ticket(next);
@@ -734,7 +741,6 @@ __device__ __forceinline__ void slices_of(const InstDesc& D, const Seg& sS, cons
                                                           coop_max);
       cn += r.cn;
       oq += r.oq;
-      if (STATS) wobj += r.ob;
     }
     i -= 3 * nq;
   }
@@ -742,8 +748,8 @@ __device__ __forceinline__ void slices_of(const InstDesc& D, const Seg& sS, cons
   if constexpr (!AHEAD) {
     for (; i < n; i = next_ticket(next) - (WIDE ? 3 * nq : 0)) {
       const int64_t s = T.first + static_cast<int64_t>(i) * T.stride;
-      do_slice<P, STATS, K>(D, S, ys, accG, accC, accQ, s, __ldg(D.slice_off + s), __ldg(D.slice_w + s), coop_max, wobj,
-                            cn, oq, [] {});
+      do_slice<P, STATS, K>(D, S, ys, accG, accC, accQ, s, __ldg(D.slice_off + s), __ldg(D.slice_w + s), coop_max,
+                            slice_part<WIDE>(D, s), cn, oq, [] {});
     }
     return;
   }
@@ -760,8 +766,8 @@ __device__ __forceinline__ void slices_of(const InstDesc& D, const Seg& sS, cons
   while (i < n) {
     int ni = 0, nw = 0;
     int64_t noff = 0;
-    do_slice<P, STATS, K>(D, S, ys, accG, accC, accQ, T.first + static_cast<int64_t>(i) * T.stride, off, w,
-                                coop_max, wobj, cn, oq, [&] {
+    const int64_t s = T.first + static_cast<int64_t>(i) * T.stride;
+    do_slice<P, STATS, K>(D, S, ys, accG, accC, accQ, s, off, w, coop_max, slice_part<WIDE>(D, s), cn, oq, [&] {
                                   ni = next_ticket(next) - (WIDE ? 3 * nq : 0);
                                   header(ni, noff, nw);
                                 });
@@ -835,26 +841,31 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
       s_next = 0;
     }
     __syncthreads();
-    double wobj = 0.0;
     for (int k = t; k < te; ++k) {
       const Task T = tasks[k];
       // dynamic order within the CTA (the sums are exact, so the order of
       // slices does not change any result)
-      slices_of<P, STATS, K, ONE, WIDE, true>(sD, sS, ys, accG, accC, accQ, T, &s_next, coop_max, wobj, cn, oq);
+      slices_of<P, STATS, K, ONE, WIDE, true>(sD, sS, ys, accG, accC, accQ, T, &s_next, coop_max, cn, oq);
       __syncthreads();
       if (threadIdx.x == 0) s_next = 0;
       __syncthreads();
     }
     if (STATS) {
+      // the slices' parts (written before the barrier above), in a fixed order
+      double o = 0.0;
+      for (int k = t; k < te; ++k) {
+        const Task T = tasks[k];
+        const int n = static_cast<int>((T.end - T.first + T.stride - 1) / T.stride);
+        const int nq = WIDE ? static_cast<int>(task_wide(T, sD.nwide)) : 0;
+        for (int i = threadIdx.x; i < n + 3 * nq; i += blockDim.x) {
+          const bool q = i < 4 * nq;
+          const int64_t s = T.first + static_cast<int64_t>(q ? i >> 2 : i - 3 * nq) * T.stride;
+          o += sD.slice_obj[q ? 4 * s + (i & 3) : slice_part<WIDE>(sD, s)];
+        }
+      }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        wobj += __shfl_xor_sync(kFull, wobj, o);
-        oq += __shfl_xor_sync(kFull, oq, o);
-      }
-      if (lane == 0) {
-        wsum[warp] = wobj;
-        s_red[warp] = oq;
-      }
+      for (int d = 16; d > 0; d >>= 1) o += __shfl_xor_sync(kFull, o, d);
+      if (lane == 0) wsum[warp] = o;
     } else {
       cta_add_u64(oq, s_red, sD.objq);
     }
@@ -878,12 +889,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
     }
     if (STATS && threadIdx.x == 0) {
       double sum = 0.0;
-      unsigned long long q = 0ull;
-      for (int w = 0; w < nw; ++w) {
-        sum += wsum[w];
-        q += s_red[w];
-      }
-      if (q != 0ull) sum += static_cast<double>(static_cast<long long>(q)) / static_cast<double>(sS.scaleO);
+      for (int w = 0; w < nw; ++w) sum += wsum[w];
       sD.seg_obj[t] = sum;
     }
     __syncthreads();
@@ -913,7 +919,6 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
   __shared__ unsigned long long s_red[32];
   const int lane = threadIdx.x & 31;
   int cur = -1;
-  double wobj = 0.0;
   unsigned long long cn = 0ull, oq = 0ull;
   chain_wait();
   chain_go();
@@ -954,7 +959,7 @@ __global__ void __launch_bounds__(kSweepThreads, 1)
       __syncthreads();
     }
     const Task T = units[u];
-    slices_of<P, false, K, false, WIDE, false>(sD, sS, ys, accG, nullptr, nullptr, T, &s_next, coop_max, wobj, cn, oq);
+    slices_of<P, false, K, false, WIDE, false>(sD, sS, ys, accG, nullptr, nullptr, T, &s_next, coop_max, cn, oq);
     __syncthreads();
   }
   if (threadIdx.x == 0) {
