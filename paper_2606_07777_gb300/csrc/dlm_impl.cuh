@@ -165,19 +165,6 @@ cudaError_t launch_chained(bool chain, void (*kernel)(KA...), dim3 grid, dim3 bl
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<KA>(args)...);
 }
 
-// f rounded to a 64-bit integer (ties to even), |f| < 2^55: the bits of
-// __float2ll_rn without the FP64 pipe it runs on (two lanes per clock and SM).
-// The part above 2^32 is read off the significand of a sum rounded
-// down at 2^23; what is left is exact and converts to 32 bits.
-__device__ __forceinline__ unsigned long long fix64(float f) {
-  const float af = fabsf(f);
-  const float m = __fadd_rd(af * 2.3283064365386963e-10f, 8388608.f);  // 2^23 + floor(|f| / 2^32)
-  const uint32_t lo = __float2uint_rn(fmaf(8388608.f - m, 4294967296.f, af));
-  const uint32_t hi = __float_as_uint(m) - 0x4B000000u;
-  const unsigned long long v = (static_cast<unsigned long long>(hi) << 32) | lo;
-  return f < 0.f ? 0ull - v : v;
-}
-
 // *p += v in shared memory.  The hardware adds 32-bit words in place, but a
 // 64-bit shared addition is a compare-and-swap loop, taken again for every other
 // lane on the same item: here the low word's old value gives the carry, and the
