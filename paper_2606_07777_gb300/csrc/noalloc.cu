@@ -211,11 +211,12 @@ __global__ void __launch_bounds__(kStaticThreads, 2)
   const RowConst C = sC;
   const float* __restrict__ ys = SMEM ? sl : lam;
   unsigned bad = 0;
-  F2 ob{0.f, 0.f};  // objective of the lane's edges
+  double wobj = 0.0;
+  float ob = 0.f;  // objective of the lane's edges of the rows in hand
   auto put = [&](int j, float cv, float av, float x) {
     // one conversion, exact up to 2^63: with max |a| z above 2^55 the exponent is 0 and terms are as large
     atomicAdd(&acc[j], static_cast<unsigned long long>(__float2ll_rn(av * x * C.scG)));
-    ob = f2_add(ob, F2{fmaf(0.5f * C.gamma * x, x, cv * x), 0.f});
+    ob += fmaf(0.5f * C.gamma * x, x, cv * x);
   };
   // edge e of the caller's arrays: its item (-1: out of range, flagged), values, u
   auto edge = [&](int64_t e, int& j, float& cv, float& av) {
@@ -351,6 +352,8 @@ __global__ void __launch_bounds__(kStaticThreads, 2)
         if (xout && i < n) xout[s + i] = x;
       }
     }
+    wobj += static_cast<double>(ob);
+    ob = 0.f;
     // rows of more than kLanes * kSlots edges: the whole warp, re-reading
     unsigned todo = __ballot_sync(kFull, wide && sub == 0);
     while (todo) {
@@ -426,10 +429,11 @@ __global__ void __launch_bounds__(kStaticThreads, 2)
         }
         if (xout) xout[ws + i] = x;
       }
+      wobj += static_cast<double>(ob);
+      ob = 0.f;
     }
   }
   if (__any_sync(kFull, bad) && lane == 0) atomicOr(&S->bad, 1u);
-  double wobj = static_cast<double>(ob.h) + ob.l;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) wobj += __shfl_xor_sync(kFull, wobj, o);
   if (lane == 0) s_obj[warp] = wobj;

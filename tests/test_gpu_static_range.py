@@ -1,6 +1,7 @@
 """The allocation-free evaluation at large magnitudes: item terms |a| x on both
 sides of 2^55, where the exponent of the fixed-point item sums reaches its lower
-end (the sums themselves stay below 2^63).  Against the oracle's FP64 sweep with the bounds of test_gpu_static_rows.py."""
+end (the sums themselves stay below 2^63), and an objective whose sum is past the
+largest float.  Against the oracle's FP64 sweep with the bounds of test_gpu_static_rows.py."""
 import numpy as np
 import pytest
 
@@ -50,4 +51,21 @@ def test_terms_around_2_to_55(dlm_lib, exp, I, degrees, kind):
     allow = np.bincount(p.col, weights=p.a * np.maximum(tol - 2e-6, 0), minlength=J)
     dg = np.abs(grad.astype(np.float64) - ref["grad"])
     assert (dg <= 2e-6 * scale + allow + 1e-6).all(), (dg / scale).max()
+    assert abs(g - ref["g"]) <= 2e-6 * (abs(ref["g"]) + abs(ref["obj"])), (g, ref["g"])
+
+
+def test_objective_past_the_largest_float(dlm_lib):
+    I, J = 200_000, 50  # ten rows a lane, some 5e37 each
+    rng = np.random.default_rng(9)
+    rp = 2 * np.arange(I + 1, dtype=np.int64)
+    first = rng.integers(0, J, size=I)
+    col = np.stack([first, (first + rng.integers(1, J, size=I)) % J], 1).reshape(-1).astype(np.int32)
+    c = (-1e37 * rng.uniform(4, 8, 2 * I)).astype(np.float32)
+    a = rng.uniform(0.5, 1.5, 2 * I).astype(np.float32)
+    inst = synth.Instance(rp, col, c, a, np.ones(J), J)
+    p = oracle_problem(inst, oracle.SIMPLEX_LE, 1.0)
+    lam32 = (1e36 * rng.uniform(0, 1, J)).astype(np.float32)
+    gamma = 1e36
+    ref = oracle.sweep(p, lam32.astype(np.float64), gamma)
+    g, _, _ = evaluate(dlm_lib, inst, oracle.SIMPLEX_LE, lam32, gamma)
     assert abs(g - ref["g"]) <= 2e-6 * (abs(ref["g"]) + abs(ref["obj"])), (g, ref["g"])
