@@ -1006,21 +1006,21 @@ dlm_status save_state(Runner& R, Saved* S) {
   }
   return DLM_OK;
 }
+// (All on the runner's stream, which the default stream may not be ordered with.)
 dlm_status restore_state(Runner& R, const Saved& S) {
-  CK(cudaStreamSynchronize(R.stream));
   for (size_t i = 0; i < R.probs.size(); ++i) {
     dlm_problem* p = R.probs[i];
-    CK(cudaMemcpy(p->lam64, S.lam[i], sizeof(double) * p->D(), cudaMemcpyDeviceToDevice));
-    CK(cudaMemcpy(p->y64, S.y[i], sizeof(double) * p->D(), cudaMemcpyDeviceToDevice));
+    CK(cudaMemcpyAsync(p->lam64, S.lam[i], sizeof(double) * p->D(), cudaMemcpyDeviceToDevice, R.stream));
+    CK(cudaMemcpyAsync(p->y64, S.y[i], sizeof(double) * p->D(), cudaMemcpyDeviceToDevice, R.stream));
     k_shadow<<<blocks_for(p->D()), 256, 0, R.stream>>>(p->lam64, p->y64, p->lam, p->y, p->D());
     CK(cudaGetLastError());
-    CK(cudaStreamSynchronize(R.stream));
-    CK(cudaMemset(p->cnt, 0, sizeof(unsigned long long)));
-    CK(cudaMemset(p->objq, 0, sizeof(unsigned long long)));
-    CK(cudaMemcpy(p->state, &S.st[i], sizeof(DevState), cudaMemcpyHostToDevice));
-    CK(cudaMemset(p->acc, 0, sizeof(unsigned long long) * p->MJ()));
+    CK(cudaMemsetAsync(p->cnt, 0, sizeof(unsigned long long), R.stream));
+    CK(cudaMemsetAsync(p->objq, 0, sizeof(unsigned long long), R.stream));
+    CK(cudaMemcpyAsync(p->state, &S.st[i], sizeof(DevState), cudaMemcpyHostToDevice, R.stream));
+    CK(cudaMemsetAsync(p->acc, 0, sizeof(unsigned long long) * p->MJ(), R.stream));
     p->traj_from = S.st[i].iter;
   }
+  CK(cudaStreamSynchronize(R.stream));  // (S has been read)
   return DLM_OK;
 }
 void free_saved(Saved& S) {
@@ -1579,13 +1579,14 @@ dlm_status dlm_set_count_limit(dlm_problem* p, double M) {
   CK(cudaStreamSynchronize(p->stream));
   p->count_on = std::isfinite(M);
   p->count_M = M;
-  // the count dual starts at 0; its accumulators are clear
-  CK(cudaMemset(p->lam + p->J, 0, sizeof(float)));
-  CK(cudaMemset(p->y + p->J, 0, sizeof(float)));
-  CK(cudaMemset(p->lam64 + p->J, 0, sizeof(double)));
-  CK(cudaMemset(p->y64 + p->J, 0, sizeof(double)));
-  CK(cudaMemset(p->cnt, 0, sizeof(unsigned long long)));
-  CK(cudaMemset(p->cnt2, 0, sizeof(unsigned long long)));
+  // the count dual starts at 0; its accumulators are clear (on the handle's stream, which the default
+  // stream may not be ordered with)
+  CK(cudaMemsetAsync(p->lam + p->J, 0, sizeof(float), p->stream));
+  CK(cudaMemsetAsync(p->y + p->J, 0, sizeof(float), p->stream));
+  CK(cudaMemsetAsync(p->lam64 + p->J, 0, sizeof(double), p->stream));
+  CK(cudaMemsetAsync(p->y64 + p->J, 0, sizeof(double), p->stream));
+  CK(cudaMemsetAsync(p->cnt, 0, sizeof(unsigned long long), p->stream));
+  CK(cudaMemsetAsync(p->cnt2, 0, sizeof(unsigned long long), p->stream));
   dlm_status st = upload_steps(p);
   if (st != DLM_OK) return st;
   invalidate_graph(p->run);
