@@ -685,7 +685,8 @@ cudaError_t launch_item_sums(const int32_t* col, const void* a, bool bf16, int64
   if (e != cudaSuccess) return e;
   const int g = static_cast<int>(std::min<int64_t>(sms, nnz / 8192 + 1));  // one block of 1,024 threads per SM
   auto go = [&](auto kernel, size_t smem) {
-    cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    // (the limit is the process's: the same for every instance, or another thread's launch might find it lowered)
+    cudaError_t f = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(lim));
     if (f != cudaSuccess) return f;
     kernel<<<g, 1024, smem, s>>>(col, a, bf16, nnz, J, fq, f1, quad, sums);
     return cudaGetLastError();
@@ -804,6 +805,9 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
                       (k > 0 ? out->phase_s[0] : 0.0) - (k > 1 ? out->phase_s[1] : 0.0);
   };
   const size_t vs = bf16 ? 2 : 4;
+  // the kernels' limits are the process's: the same for every instance, or another thread's launch might find
+  // one lowered
+  const int smem_limit = static_cast<int>(sweep_smem_limit());
   cudaFuncSetAttribute(k_edges, cudaFuncAttributeMaxDynamicSharedMemorySize, 4 * 16384);
   dlm_status st = DLM_OK;
   int32_t *deg = nullptr, *sdeg = nullptr, *idx = nullptr, *perm = nullptr;
@@ -856,8 +860,7 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
     DLM_CK(cudaGetLastError());
     if (measure) {  // no layout is built: the items' repeats are checked apart
       const size_t dsm = sizeof(unsigned) * static_cast<size_t>((J + 31) / 32) * (kDupThreads / 32);
-      if (dsm > 48 * 1024) DLM_CK(cudaFuncSetAttribute(k_dups, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                      static_cast<int>(dsm)));
+      DLM_CK(cudaFuncSetAttribute(k_dups, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit));
       const int64_t want = (I + kDupThreads - 1) / kDupThreads;
       const int gd = static_cast<int>(want < 8LL * sms ? (want > 0 ? want : 1) : 8LL * sms);
       k_dups<<<gd, kDupThreads, dsm, s>>>(rp, col, I, J, bad);
@@ -977,13 +980,13 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
     const int64_t most = static_cast<int64_t>(sms) * (bf16 ? 4 : 2);  // blocks that fit at once
     const int g = static_cast<int>(want < most ? want : most);
     if (bf16) {
-      DLM_CK(cudaFuncSetAttribute(&k_gather<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, gsm));
+      DLM_CK(cudaFuncSetAttribute(&k_gather<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit));
       k_gather<uint32_t><<<g, 32 * kGatherWarps, gsm, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off,
                                                            out->slice_w, out->col16, static_cast<uint32_t*>(out->ca),
                                                            out->orig_off, out->udeg, out->lead, static_cast<int>(J),
                                                            ticket, bad + 1);
     } else {
-      DLM_CK(cudaFuncSetAttribute(&k_gather<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, gsm));
+      DLM_CK(cudaFuncSetAttribute(&k_gather<float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit));
       k_gather<float2><<<g, 32 * kGatherWarps, gsm, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off,
                                                          out->slice_w, out->col16, static_cast<float2*>(out->ca),
                                                          out->orig_off, out->udeg, out->lead, static_cast<int>(J),
