@@ -54,9 +54,10 @@ __device__ __forceinline__ float load_val(const void* p, int64_t e, bool bf16) {
   return reinterpret_cast<const float*>(p)[e];
 }
 
-// Row pointer checks; degree of every user; users with no edges.
-__global__ void k_rows(const int64_t* rp, int64_t I, int64_t nnz, int32_t* deg, unsigned long long* zero_cnt,
-                       int* bad) {
+// Row pointer checks; degree of every user; users with no edges.  A row of more
+// edges than items repeats one: found here, before a slice is laid out at its length.
+__global__ void k_rows(const int64_t* rp, int64_t I, int64_t nnz, int64_t J, int32_t* deg,
+                       unsigned long long* zero_cnt, int* bad) {
   int flag = 0;
   unsigned long long z = 0;
   for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < I;
@@ -64,6 +65,7 @@ __global__ void k_rows(const int64_t* rp, int64_t I, int64_t nnz, int32_t* deg, 
     const int64_t r0 = rp[i], r1 = rp[i + 1];
     const int64_t d = r1 - r0;
     if (d < 0 || r0 < 0 || r1 > nnz || d > 0x7fffffff) flag |= kBadRowPtr;
+    if (d > J) flag |= kDupItem;
     deg[i] = d < 0 ? 0 : static_cast<int32_t>(d);
     z += (d == 0);
   }
@@ -515,8 +517,6 @@ __device__ __noinline__ uint64_t gather_strips(const GatherWarp<CA>& W, bool& tw
     for (int o = 1; o < 32; o <<= 1) lowest4_merge<K>(o, lk);
     const uint64_t ld = lead_of<K>(lk, dt);
     if (lane == t) lead = ld;
-    twice = twice || dt > W.J;  // more edges than items: some item repeats
-    if (dt > W.J) continue;     // (warp-uniform)
     for (int k = lane; k < dt; k += 32) {
       const int j = __ldg(W.col + rt + k);
       const unsigned bit = 1u << (j & 31);
@@ -833,7 +833,7 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
   DLM_CK(cudaMemsetAsync(item_deg, 0, sizeof(unsigned long long) * (J > 0 ? J : 1), s));
   DLM_CK(cudaMemsetAsync(mx, 0, sizeof(unsigned) * 2, s));
   DLM_CK(cudaMemsetAsync(bad, 0, sizeof(int), s));
-  if (I > 0) k_rows<<<grid_for(I), kT, 0, s>>>(rp, I, nnz, deg, zero_cnt, bad);
+  if (I > 0) k_rows<<<grid_for(I), kT, 0, s>>>(rp, I, nnz, J, deg, zero_cnt, bad);
   DLM_CK(cudaGetLastError());
   if (J > 0) k_b<<<grid_for(J), kT, 0, s>>>(b, J, bad);
   DLM_CK(cudaGetLastError());
