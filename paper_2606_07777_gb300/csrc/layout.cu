@@ -334,7 +334,10 @@ __device__ __forceinline__ uint64_t lead_of(const K (&lk)[4], int d) {
 // once more, 32 slice positions of every row at a time, put into the slice's
 // order in shared memory -- groups of four edges 4 elements further apart than
 // in the slice, so that a row's groups fall into different banks -- and
-// written out in whole 128-bit pieces.  Slices are dealt by a counter, widest first.
+// written out in whole 128-bit pieces.  There are few such slices and each is long, so
+// the whole block takes one: its warps share the rows, then the strips (a new handle of
+// 3,000 rows of 2,000 FP32 edges: 3,844 us with a warp a slice, 889 with a block; 30,000 rows: 5,322, 3,000).
+// Slices are dealt by a counter, widest first.
 // 50M BF16 edges (2M rows of 25 on average, the longest 500): 939 us with every
 // row read twice and the longest rows' chains of loads at the end, now 439 us.
 // Every item is in [0, J) here (checked before).
@@ -496,15 +499,14 @@ __device__ __forceinline__ uint64_t gather_raw(const GatherWarp<CA>& W, bool& tw
   return lead;
 }
 
-// Slices of longer rows.
+// A slice of longer rows, by the whole block (every warp has the same slice in W).
 template <typename CA>
-__device__ __noinline__ uint64_t gather_strips(const GatherWarp<CA>& W, bool& twice) {
+__device__ __noinline__ uint64_t gather_strips(const GatherWarp<CA>& W, uint64_t* s_lead, bool& twice) {
   using K = LeadKey<CA>;
   constexpr bool kBf = sizeof(CA) == 4;
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int w4 = W.w >> 2;
-  uint64_t lead = 0;
-  for (int t = 0; t < 32; ++t) {
+  for (int t = warp; t < 32; t += kGatherWarps) {
     const int64_t rt = __shfl_sync(kFullMask, W.r, t);
     const int dt = __shfl_sync(kFullMask, W.d, t);
     K lk[4];
@@ -516,18 +518,22 @@ __device__ __noinline__ uint64_t gather_strips(const GatherWarp<CA>& W, bool& tw
     __syncwarp();
     for (int o = 1; o < 32; o <<= 1) lowest4_merge<K>(o, lk);
     const uint64_t ld = lead_of<K>(lk, dt);
-    if (lane == t) lead = ld;
+    if (lane == 0) s_lead[t] = ld;
+#pragma unroll 4
     for (int k = lane; k < dt; k += 32) {
       const int j = __ldg(W.col + rt + k);
       const unsigned bit = 1u << (j & 31);
       if (atomicOr(&W.seen[j >> 5], bit) & bit) twice = true;
     }
     __syncwarp();
+#pragma unroll 4
     for (int k = lane; k < dt; k += 32) W.seen[__ldg(W.col + rt + k) >> 5] = 0u;
     __syncwarp();
   }
+  __syncthreads();
+  const uint64_t lead = s_lead[lane];
   // positions 32 st .. of every row, then the strip's elements in order
-  for (int st = 0; 32 * st < W.w; ++st) {
+  for (int st = warp; 32 * st < W.w; st += kGatherWarps) {
     const int k = 32 * st + lane;
     const int at = k < 4 * w4 ? (lane >> 2) * 132 + (lane & 3) : kStripGroups * 132 + 32 * (k - 4 * w4);
     const int by = k < 4 * w4 ? 4 : 1;
@@ -587,33 +593,54 @@ __global__ void __launch_bounds__(32 * kGatherWarps, sizeof(CA) == 4 ? 4 : 2)
                    warp * words;
   for (int k = lane; k < words; k += 32) seen[k] = 0u;
   __syncwarp();
+  __shared__ uint64_t s_lead[32];
+  __shared__ unsigned s_ticket;
   bool twice = false;
-  for (;;) {
-    unsigned tk = 0;
-    if (lane == 0) tk = atomicAdd(ticket, 1u);
-    const int64_t s = __shfl_sync(kFullMask, tk, 0);
-    if (s >= nslices) break;
+  // slice s of every warp of the caller: its rows, and where its elements go
+  auto slice = [&](int64_t s, bool write) {
     const int64_t u = 32 * s + lane;
     int64_t r = 0;
     int d = 0;
     if (u < In) {
       r = rp[perm[u]];
       d = sdeg[u];
-      orig_off[u] = r;
-      udeg[u] = d;
+      if (write) {
+        orig_off[u] = r;
+        udeg[u] = d;
+      }
     }
     const int64_t base = slice_off[s];
-    const GatherWarp<CA> W{col, c, a, col_o + base, ca_o + base, sca, scol, seen, r, d, width[s], J};
-    uint64_t lead;
-    if (W.w <= kRawWidth) {
-      lead = gather_raw(W, twice);
-    } else {
-      bool again = false;  // (copies: W and `twice` stay in registers)
-      const GatherWarp<CA> V = W;
-      lead = gather_strips(V, again);
-      twice = twice || again;
+    return GatherWarp<CA>{col, c, a, col_o + base, ca_o + base, sca, scol, seen, r, d, width[s], J};
+  };
+  // slices of long rows first, a block each; the first ticket that has none is warp 0's
+  int64_t mine = -1;
+  for (;;) {
+    if (threadIdx.x == 0) s_ticket = atomicAdd(ticket, 1u);
+    __syncthreads();
+    const int64_t s = s_ticket;
+    if (s >= nslices || width[s] <= kRawWidth) {
+      if (warp == 0) mine = s;
+      break;
     }
-    if (u < In) lead_o[u] = lead;
+    bool again = false;  // (copies: W and `twice` stay in registers)
+    const GatherWarp<CA> V = slice(s, warp == 0);
+    const uint64_t lead = gather_strips(V, s_lead, again);
+    twice = twice || again;
+    if (warp == 0 && 32 * s + lane < In) lead_o[32 * s + lane] = lead;
+    __syncthreads();  // s_lead and s_ticket have been read
+  }
+  for (;;) {
+    int64_t s = mine;
+    if (s < 0) {
+      unsigned tk = 0;
+      if (lane == 0) tk = atomicAdd(ticket, 1u);
+      s = __shfl_sync(kFullMask, tk, 0);
+    }
+    mine = -1;
+    if (s >= nslices) break;
+    const GatherWarp<CA> W = slice(s, true);
+    const uint64_t lead = gather_raw(W, twice);
+    if (32 * s + lane < In) lead_o[32 * s + lane] = lead;
   }
   if (__any_sync(kFullMask, twice) && lane == 0) *dup = 1;
 }
@@ -976,9 +1003,8 @@ dlm_status build_layout(int64_t I, int64_t J, int64_t nnz, const int64_t* rp, co
     DLM_CK(cudaGetDevice(&dev));
     DLM_CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const int gsm = kGatherWarps * (kStripElems * static_cast<int>(2 + 2 * vs) + 4 * static_cast<int>((J + 31) / 32));
-    const int64_t want = (ns + kGatherWarps - 1) / kGatherWarps;
-    const int64_t most = static_cast<int64_t>(sms) * (bf16 ? 4 : 2);  // blocks that fit at once
-    const int g = static_cast<int>(want < most ? want : most);
+    // blocks that fit at once, or one a slice (a block takes a slice of long rows, a warp another)
+    const int g = static_cast<int>(std::min<int64_t>(ns, static_cast<int64_t>(sms) * (bf16 ? 4 : 2)));
     if (bf16) {
       DLM_CK(cudaFuncSetAttribute(&k_gather<uint32_t>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_limit));
       k_gather<uint32_t><<<g, 32 * kGatherWarps, gsm, s>>>(rp, col, c, a, perm, sdeg, In, ns, out->slice_off,
