@@ -118,8 +118,8 @@ typedef struct {
                             threshold iteration) are handled one after another by all 32 lanes
                             of the warp while fewer than coop_max of its 32 rows need it
                             (default 12; 1 never, 33 always) */
-  int32_t block_threads; /* threads per sweep CTA: 0 or 1024 (default: 1024, fewer for an instance whose
-                            slices of 32 users leave a CTA less than 32), or 512 */
+  int32_t block_threads; /* threads per sweep CTA: 512, 1024, or 0 (default: 1024, fewer for an instance whose
+                            slices of 32 users leave a CTA less than 32) */
   int32_t restart;       /* 1: adaptive momentum restart besides the stage restarts -- theta = 1
                             after a step whose direction opposes the momentum in the step metric,
                             sum_j (lam+_j - y_j)(lam+_j - lam_j) / step_j < 0 (O'Donoghue &

@@ -170,6 +170,7 @@ struct Runner {
   int win = 0;  // item window of certificate sweeps (smemJ when their arrays fit at once)
   int graph_iters = 10;
   int topk = 4;  // one-family sweeps: values tracked per row in the first pass
+  bool small = false;        // fewer slices a CTA than a CTA of 1,024 threads has warps
   bool short_rows = false;   // iteration sweeps take the short-row sweep (sweep_short.cu)
   int upd_ctas = 1;      // update grid width (the largest member's)
   void* tabs = nullptr;  // the instances' tables (inst_iter, inst_stats, upd, st_stats)
@@ -710,11 +711,11 @@ cudaError_t dispatch_sweep(const Runner& R, const SweepLaunch& L, bool stats, bo
 
 dlm_status enqueue_iteration(Runner& R) {
   SweepLaunch L = launch_of(R, R.inst_iter);
-  // Chained launches for sweeps of small CTAs only: a full one would hold its SM
-  // while it waits for the update, and other streams' sweeps with it (three
-  // handles in turn, chained against not: two families 1,035 against 967 us,
-  // appendix 818 against 741 us; 10,000 x 100: 181 against 302 us).
-  L.chain = R.threads < kSweepThreads;
+  // Chained launches for sweeps of small CTAs or of few slices (R.small) only: a
+  // full one would hold its SM while it waits for the update, and other streams'
+  // sweeps with it (three handles in turn, chained against not: two families 1,035
+  // against 967 us, appendix 818 against 741 us; 10,000 x 100: 181 against 302 us).
+  L.chain = R.threads < kSweepThreads || R.small;
   CK(dispatch_sweep(R, L, false, R.bf16));
   CK(launch_update(R.upd, static_cast<int>(R.probs.size()), R.upd_ctas, R.stream, L.chain));
   return DLM_OK;
@@ -802,7 +803,7 @@ dlm_status runner_step_timed(Runner& R, int64_t n_iters, double* sweep_ms, doubl
   return DLM_OK;
 }
 
-// Threads per sweep CTA unless the options ask for 512: a warp per slice of
+// Threads per sweep CTA unless the options name them: a warp per slice of
 // a CTA's share, at least a thread per sixteen items (the dual is loaded and the
 // sums are flushed by the CTA), a power of two from 128 to 1,024.  A small instance has
 // few slices per SM: starting and synchronizing 32 warps for two slices was much
@@ -835,8 +836,10 @@ int default_order(const Runner& R, int grid) {
 // assignment.  Rebuilds the tasks when the launch shape changes.
 dlm_status runner_configure(Runner& R, const dlm_options& o, bool force) {
   const int per_sm = o.ctas_per_sm > 0 ? o.ctas_per_sm : (o.block_threads == 512 ? 2 : 1);
-  const int threads = o.block_threads == 512 ? 512 : default_threads(R, R.sms * per_sm);
   const int grid = R.sms * per_sm;
+  const int fit = default_threads(R, grid);
+  const int threads = o.block_threads > 0 ? o.block_threads : fit;
+  R.small = fit < kSweepThreads;  // (graphs that hold the launches are invalidated below)
   const int assign = o.mapping == 1   ? kAssignInterleaved
                      : o.mapping == 2 ? kAssignContiguous
                      : o.mapping == 3 ? kAssignDynamic
