@@ -75,7 +75,10 @@ struct StepScalars {
   bool stage_restart, test;
 };
 __device__ __forceinline__ void step_scalars(const UpdInst& U, StepScalars& c) {
-  c.st = *U.state;
+  static_assert(sizeof(DevState) % 8 == 0, "read in 64-bit words");
+#pragma unroll
+  for (int k = 0; k < static_cast<int>(sizeof(DevState) / 8); ++k)
+    reinterpret_cast<uint64_t*>(&c.st)[k] = __ldcg(reinterpret_cast<const unsigned long long*>(U.state) + k);
   const int64_t t1 = c.st.iter + 1;
   c.s1 = t1 / U.iters_per_stage;
   c.gamma1 = U.gamma_tab[c.s1 < U.nstages ? c.s1 : U.nstages - 1];
@@ -102,6 +105,11 @@ __global__ void __launch_bounds__(kUpdChunk) fista_update_kernel(const UpdInst* 
   for (int k = tid; k < static_cast<int>(sizeof(UpdInst) / 8); k += kUpdChunk)
     reinterpret_cast<uint64_t*>(&U)[k] = __ldg(reinterpret_cast<const uint64_t*>(I) + k);
   __syncthreads();
+  // Read ahead of chain_wait(): what the sweep between does not write.  The last
+  // update wrote the state, y and lam; it had ended, its writes with it, when this
+  // sweep's blocks passed their own chain_wait(), and they let this kernel start only after that
+  // (chain_go()).  A wait's promise covers reads after one's own, so these go past L1, which may
+  // hold a line of an earlier iteration.
   if (tid == 0) step_scalars(U, c);
   // everything that does not depend on the sweep or on the scalars
   const int NC = U.ncap, D = NC + (U.count_on ? 1 : 0);
@@ -109,8 +117,8 @@ __global__ void __launch_bounds__(kUpdChunk) fista_update_kernel(const UpdInst* 
   const bool in = j < D;
   double yj = 0.0, lam0 = 0.0, h = 0.0, bj = 0.0;
   if (in) {
-    yj = U.y64[j];
-    lam0 = U.lam64[j];
+    yj = __ldcg(U.y64 + j);
+    lam0 = __ldcg(U.lam64 + j);
     if (U.precondition) h = __ldg(U.curv + j);
     bj = j < NC ? __ldg(U.b + j) : U.count_M;
   }
@@ -118,7 +126,7 @@ __global__ void __launch_bounds__(kUpdChunk) fista_update_kernel(const UpdInst* 
   double step = c.step0;
   if (U.precondition) step = h > 0.0 ? c.st.gamma / h : 0.0;
   double lg = 0.0, dot = 0.0, bad = 0.0;
-  chain_wait();  // the sweep's sums; all read before it was written before the sweep began
+  chain_wait();  // the sweep's sums
   if (in) {
     const double G =
         j < NC ? to_real(U.acc[j], U.inv_scaleG) - bj : to_real(*U.cnt, U.inv_scaleN) - bj;
