@@ -506,7 +506,7 @@ __global__ void k_to_bf16(const float* __restrict__ src, int64_t n, bf16* __rest
 // throughput; the tiles are spread one per SM.  As separate launches (five
 // products through global memory with scalar staging, six elementwise kernels,
 // six reductions) the loss and gradient of 17,000 rows and a prediction of
-// 1,000 took 525 us at width 128; fused they take 84 us, copies to the host included.
+// 1,000 took 525 us at width 128; fused they take 87 us, copies to the host included.
 //
 // Shared-memory operands are unswizzled 8 x 16-byte core matrices in columns
 // of 16-byte pieces: element (r, k) of a row buffer at
@@ -519,7 +519,7 @@ __global__ void k_to_bf16(const float* __restrict__ src, int64_t n, bf16* __rest
 //
 // The products' K order, the layer-3 sum's order and every rounding to BF16
 // are those of the separate kernels, so the forward pass gives the same bits.  The
-// column sums (biases, w3) add FP32 terms as float pairs (TwoSum), the tiles'
+// column sums (biases, w3) add FP32 terms in three words (Sum3), the CTAs'
 // results in FP64.  Partial gradients go to one slot per CTA and are added in
 // slot order by k_mlp_reduce: results do not depend on timing.
 // ---------------------------------------------------------------------------
@@ -550,12 +550,27 @@ struct MlpArgs {
   int* err;
 };
 
-__device__ __forceinline__ void pair_add(float& h, float& l, float v) {
-  const float s = h + v;
-  const float b = s - h;
-  l += (h - (s - b)) + (v - b);
-  h = s;
-}
+// A sum of FP32 terms in three words: each TwoSum's error goes to the next word
+// exactly, so at least 53 bits are kept (FP64 additions, at two lanes per clock and SM, would
+// take a tile 26 us; in two words, 48 bits).
+struct Sum3 {
+  float h = 0.f, l = 0.f, e = 0.f;
+  __device__ __forceinline__ void low(float v) {
+    const float s = l + v;
+    const float b = s - l;
+    e += (l - (s - b)) + (v - b);
+    l = s;
+  }
+  __device__ __forceinline__ void add(float v) {
+    const float s = h + v;
+    const float b = s - h;
+    low((h - (s - b)) + (v - b));
+    h = s;
+  }
+  __device__ __forceinline__ double total() const {
+    return static_cast<double>(h) + (static_cast<double>(l) + static_cast<double>(e));
+  }
+};
 
 // Sixteen accumulator columns of the thread's TMEM lane.
 __device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&v)[16]) {
@@ -677,10 +692,10 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
   const uint32_t aX = smem_addr(sX), aW1 = smem_addr(sW1), aH = smem_addr(sH), aD = smem_addr(sD), aW = smem_addr(sW);
   float* part = BWD ? g.part + static_cast<int64_t>(blockIdx.x) * (static_cast<int64_t>(kF) * H + static_cast<int64_t>(H) * H)
                     : nullptr;
-  // column sums of this thread's column (two threads per column at HB = 128, 64 rows each), as float pairs
+  // column sums of this thread's column (two threads per column at HB = 128, 64 rows each), in three words
   const int col = tid & (HB - 1);
   const int rlo = HB == 128 ? 64 * (tid >> 7) : 0, rn = HB == 128 ? 64 : 128;
-  float w3h = 0.f, w3l = 0.f, b2h = 0.f, b2l = 0.f, b1h = 0.f, b1l = 0.f, b3h = 0.f, b3l = 0.f;
+  Sum3 sw, s2, s1, s0;  // dw3, db2, db1 of the column, db3 of the row
   double loss = 0.0;
   const float two_n = BWD ? static_cast<float>(2.0 / static_cast<double>(g.n)) : 0.f;
   const float bias3 = g.b3[0];
@@ -779,7 +794,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
           const float e = o - __ldg(g.y + r);
           dz = two_n * e * sigmoid_f(s);
           loss += static_cast<double>(e) * e;
-          pair_add(b3h, b3l, dz);
+          s0.add(dz);
         }
       }
       if (BWD) sdz[row] = dz;
@@ -799,9 +814,9 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
         const bf16 q = __float2bfloat16_rn(h > 0.f ? d * w : 0.f);
         *e = q;
         const float t = h * d;
-        pair_add(w3h, w3l, t);
-        w3l += fmaf(h, d, -t);
-        pair_add(b2h, b2l, __bfloat162float(q));
+        sw.add(t);
+        sw.low(fmaf(h, d, -t));
+        s2.add(__bfloat162float(q));
       }
     }
     hand_over();
@@ -871,7 +886,7 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
     {  // column sums of dz1
       const unsigned char* p = sW + (col >> 3) * kCS + (col & 7) * 2 + rlo * 16;
 #pragma unroll 8
-      for (int r = 0; r < rn; ++r) pair_add(b1h, b1l, __bfloat162float(*reinterpret_cast<const bf16*>(p + r * 16)));
+      for (int r = 0; r < rn; ++r) s1.add(__bfloat162float(*reinterpret_cast<const bf16*>(p + r * 16)));
     }
     if (NB > 1 && !finished()) break;
     if (NB > 1) store_dw2(0, 128 + row);
@@ -908,15 +923,14 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
     // this CTA's column sums, db3 and loss in FP64 (slots of CTAs without a tile hold zeros)
     double* dp = g.dpart + static_cast<int64_t>(blockIdx.x) * (3 * H + 2);
     double* sc = reinterpret_cast<double*>(sxc);  // [HB = 128: 3][128]
-    const double s1 = static_cast<double>(b1h) + b1l, s2 = static_cast<double>(b2h) + b2l,
-                 s3 = static_cast<double>(w3h) + w3l;
+    const double d1 = s1.total(), d2 = s2.total(), d3 = sw.total();
     __syncthreads();
     if (HB == 128 && tid >= 128) {
-      sc[col] = s1;
-      sc[128 + col] = s2;
-      sc[256 + col] = s3;
+      sc[col] = d1;
+      sc[128 + col] = d2;
+      sc[256 + col] = d3;
     }
-    double t3 = static_cast<double>(b3h) + b3l;
+    double t3 = s0.total();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       t3 += __shfl_down_sync(0xffffffffu, t3, o);
@@ -928,9 +942,9 @@ __global__ void __launch_bounds__(kMlpThreads, 1) k_mlp(const MlpArgs g) {
     }
     __syncthreads();
     if (tid < HB && col < H) {
-      dp[col] = s1 + (HB == 128 ? sc[col] : 0.0);
-      dp[H + col] = s2 + (HB == 128 ? sc[128 + col] : 0.0);
-      dp[2 * H + col] = s3 + (HB == 128 ? sc[256 + col] : 0.0);
+      dp[col] = d1 + (HB == 128 ? sc[col] : 0.0);
+      dp[H + col] = d2 + (HB == 128 ? sc[128 + col] : 0.0);
+      dp[2 * H + col] = d3 + (HB == 128 ? sc[256 + col] : 0.0);
     }
     if (tid == 0) {
       double a = 0.0, b = 0.0;
