@@ -365,6 +365,7 @@ void invalidate_graph(Runner& R) {
 }
 
 void runner_free(Runner& R) {
+  if (R.stream) cudaStreamSynchronize(R.stream);  // the tables' copies read host buffers that end with R
   invalidate_graph(R);
   dev_free(R.tabs, R.stream);
   dev_free(R.plan, R.stream);
