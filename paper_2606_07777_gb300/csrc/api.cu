@@ -284,7 +284,8 @@ namespace {
 // 80 ns an edge of the row's width, against the layout's bytes at 5 TB/s -- and
 // never rows under 64 edges.  FP32 only: a BF16 pass is half as long, and
 // quarters, whose warps finish eight rows at a time, gave 2 us of 22 on small
-// instances alone but took a 16-member batch from 1,405 to 1,560 us.  Not the
+// instances alone but took a 16-member batch from 1,405 to 1,560 us (in dynamic
+// units; in equal-work ranges, its default since, not measured).  Not the
 // box, whose rows are summed in an order that depends on how many of the warp's
 // rows there are (it equals the box cut with a slack budget bit for bit).  A
 // rule on the instance alone, so every mapping and batch sweeps it alike.
@@ -390,7 +391,7 @@ void runner_free(Runner& R) {
 // finish, about six, against one per 16 BF16 or 8 FP32 edges of its width.
 // (16 BF16 members of 10,000 to 1.2M users x 2,000 items in equal-work ranges: 146 us
 // an iteration with 128, 112 with 512, 108 with 2,048; FP32 members,
-// with their wide slices in quarters: 162 with 2,048, 156 with 1,280, 145 with 640.)
+// with their wide slices in quarters: 162 with 2,048, 156 with 1,280, 145 with 640.  No other batch was fitted.)
 int64_t slice_cost(const Runner& R) { return R.bf16 ? 2048 : 640; }
 
 // Slice-to-CTA tasks.  Interleaved: CTA k sweeps slices k, k + V, ... of
@@ -1156,7 +1157,8 @@ dlm_status check_options(const dlm_options* opt) {
   return DLM_OK;
 }
 
-// Certificate sweeps of one family write the edges with x > 0 only.
+// Certificate sweeps of one family write the edges with x > 0 only.  (Those of several
+// families and of the box cut write every edge of a row, scattered.)
 dlm_status clear_x(const dlm_problem* p, float* x) {
   if (x && p->m == 1 && p->kind != DLM_BOX_CUT) CK(cudaMemsetAsync(x, 0, sizeof(float) * p->nnz, p->stream));
   return DLM_OK;

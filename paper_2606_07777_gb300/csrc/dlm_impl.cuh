@@ -15,7 +15,7 @@ namespace dlm {
 
 constexpr int kWarp = 32;
 constexpr int kSweepThreads = 1024;  // 32 warps per sweep CTA, one CTA per SM
-constexpr int kUpdThreads = 1024;    // one CTA per instance for the O(J) kernels
+constexpr int kUpdThreads = 1024;    // the one CTA that adds a shard's certificate objective
 constexpr int64_t kMaxStageTable = int64_t(1) << 20;  // continuation stages a schedule may take to reach gamma_end
 constexpr int kStatsOut = 16;        // doubles of a certificate's result
 constexpr int kTrajCap = 4096;       // dual objective values kept per handle (ring, one per iteration)

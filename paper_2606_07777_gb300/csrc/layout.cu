@@ -235,7 +235,9 @@ __global__ void k_slices(const int32_t* sdeg, int64_t nslices, bool bf16, int32_
     // groups of four -- in BF16, whose edges are smaller, two -- are made a
     // group with padding: the sweeps read the tail an edge at a time, a round trip
     // each (16M x 5,000 BF16: 470 -> 454 us an iteration with three, 451 with two; 8M x 2,000 FP32: 308
-    // -> 305 us with three, 306 with two)
+    // -> 305 us with three, 306 with two).  Rows of a few edges gain and lose by it: with widths under 12
+    // left as they are, ten iterations of 4M x 1,000 at mean 10 take 823 -> 868 us in BF16, 891 -> 917 in
+    // FP32; at mean 4 615 -> 564, 612 -> 638; at mean 2 468 -> 458, 445 -> 442; the short-row sweep 1 % less to 5 % more.
     const int32_t d = sdeg[32 * s];
     const int32_t w = (d & 3) >= (bf16 ? 2 : 3) ? (d | 3) + 1 : d;
     width[s] = w;
@@ -650,8 +652,7 @@ __global__ void __launch_bounds__(32 * kGatherWarps, sizeof(CA) == 4 ? 4 : 2)
 // Blocks add in shared memory where it holds the sums (SMEM) and flush once per
 // item.  Bound by the shared-memory atomics of the popular items: one pass
 // over the edges for both sums instead of two, four edges a step
-// (`quad`: aligned arrays), conversions off the FP64 pipe.  50M BF16 edges, 1,000 items:
-// 2 x 338 us in two passes.
+// (`quad`: aligned arrays).  50M BF16 edges, 1,000 items: 168 us (2 x 338 in two passes).
 template <bool SQ, bool S1, bool SMEM>
 __global__ void __launch_bounds__(1024)
     k_item_sums(const int32_t* __restrict__ col, const void* __restrict__ a, bool bf16, int64_t nnz, int64_t J,

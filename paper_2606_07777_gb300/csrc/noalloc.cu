@@ -451,8 +451,8 @@ __global__ void __launch_bounds__(kStaticThreads, 2)
   }
 }
 
-// g = sum_i (c x + gamma/2 x^2) + lam^T (A x - b), grad = A x - b; then the
-// scratch is cleared for the next call.  A flagged invalid item gives NaN.
+// g = sum_i (c x + gamma/2 x^2) + lam^T (A x - b), grad = A x - b.  A flagged
+// invalid item gives NaN.  (k_static_begin clears the scratch for each call.)
 __global__ void __launch_bounds__(1024) k_static_finish(const double* __restrict__ b, int64_t J, int64_t nnz, double z,
                                                         int blocks, const float* __restrict__ lam, double* g_out,
                                                         float* __restrict__ grad_out, StaticScratch* S) {
@@ -468,7 +468,6 @@ __global__ void __launch_bounds__(1024) k_static_finish(const double* __restrict
   for (int k = threadIdx.x; k < blocks; k += blockDim.x) obj += S->obj[k];
   for (int64_t j = threadIdx.x; j < J; j += blockDim.x) {
     const double G = static_cast<double>(static_cast<long long>(S->acc[j])) * invG - b[j];
-    S->acc[j] = 0ull;
     lg += static_cast<double>(lam[j]) * G;
     if (grad_out) grad_out[j] = bad ? NAN : static_cast<float>(G);
   }
@@ -491,10 +490,7 @@ __global__ void __launch_bounds__(1024) k_static_finish(const double* __restrict
       lg += __shfl_down_sync(kFull, lg, o);
       obj += __shfl_down_sync(kFull, obj, o);
     }
-    if (lane == 0) {
-      *g_out = bad ? NAN : obj + lg;
-      S->bad = 0u;
-    }
+    if (lane == 0) *g_out = bad ? NAN : obj + lg;
   }
 }
 
